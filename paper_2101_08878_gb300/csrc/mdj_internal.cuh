@@ -21,7 +21,10 @@ namespace mdj {
 // ------------------------------------------------------------------ limits
 
 constexpr uint32_t kMaxFanout = 1024;     // buckets of one stable scatter pass
-constexpr uint32_t kMergeFanout = 256;    // pass-1 buckets of a two-pass join plan
+// Pass-1 buckets of a two-pass join plan.  Both passes of a 1e8-row side in
+// 28.7K sub-buckets: 1.39 ms with 128, 1.41 with 160, 1.40 with 192; with
+// 14.4K sub-buckets (250M rows): 3.28 ms with 128, 3.42 with 192.
+constexpr uint32_t kMergeFanout = 128;
 constexpr uint32_t kMaxSubBuckets = 49152;  // final buckets of a two-pass plan
 constexpr uint32_t kPass2SpanMax = 1024;  // local buckets of one pass-2 tile
 

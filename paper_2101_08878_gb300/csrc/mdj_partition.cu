@@ -16,7 +16,10 @@
 //                one atomicAdd per (tile, bucket) - not stable, coalesced
 //
 // Every kernel is bandwidth-bound: no tensor cores, integer hashing only.
+#include <stdlib.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "mdj_internal.cuh"
 #include "mdj_shuffle_dev.cuh"
@@ -265,14 +268,11 @@ __global__ void __launch_bounds__(kNW * 32, 2)
 //   k_tot      rows per final sub-bucket (shared counters, flushed with one
 //              global add per counter); the next chunk's keys load while the
 //              current chunk is counted
-//   k_shuffle  persistent blocks over tiles of 4096 rows: every column of a
-//              row is loaded before the tile is processed (the next tile's
-//              while the current one is written out), a row's rank in its
-//              bucket is a shared-memory atomic, each (tile, bucket) run is
-//              reserved with one global atomicAdd on the bucket's cursor, and
-//              the columns are staged in bucket order and leave as runs;
-//              three block barriers per tile.
-//              PASS2: rows already grouped by pass-1 bucket (sub-bucket / F2)
+//   k_shuffle  persistent blocks: a row's rank in its bucket is a
+//              shared-memory atomic, each (tile, bucket) run is reserved with
+//              one global atomicAdd on the bucket's cursor, and the columns
+//              leave in bucket order as runs.
+//              Pass 2: rows already grouped by pass-1 bucket (sub-bucket / F2)
 //              are split into their sub-buckets, as in k_scatter's RESERVE.
 // A pass-1 bucket holds the rows of sub-buckets [b * F2, (b + 1) * F2)
 // (pass-1 bucket = sub-bucket / F2, see BucketSpec), so the scanned counts
@@ -324,56 +324,173 @@ __global__ void k_pass1_cursors(const uint32_t *__restrict__ off, uint32_t F1, u
   if (cur2 && b < nsub) cur2[b] = off[b];
 }
 
-// Persistent: block b takes tiles b, b + gridDim.x, ...  Once a tile is
-// staged its registers are free, so the next tile's columns are loaded into
-// them before the staged tile is written out; the DRAM latency of the load
-// overlaps the write-out.  `reg_col` is the non-key column carried in
-// registers (-1: none); with EXTRA, the other non-key columns are loaded and
-// staged one at a time after the first write-out (and the next tile's load
-// waits until they are done).  Run destinations are reserved on `cursors`.
-template <typename KeyT, bool PASS2, bool EXTRA>
-__global__ void __launch_bounds__(kShNT, 1)
-    k_shuffle(const KeyT *__restrict__ keys, uint32_t n, uint32_t ntiles, BucketSpec bs, uint32_t F, uint32_t F2,
-              uint32_t *__restrict__ cursors, ColMove cm, int reg_col,
-              const uint32_t *__restrict__ rid_in, uint32_t *__restrict__ rid_out) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5;
-  const int pw = reg_col >= 0 ? cm.width[reg_col] : 0;
-  KeyT kv[kRPL];
-  uint64_t pv[kRPL];
-  uint32_t rv[kRPL];
-  KeyT kfirst = KeyT(0), klast = KeyT(0);
-  uint32_t t = blockIdx.x;
-  const uint32_t tend = ntiles, tstep = gridDim.x;
-  if (t >= tend) return;
-  shuffle_load<KeyT, PASS2>(keys, t * kShTile, min(t * kShTile + kShTile, n), cm, reg_col, pw, rid_in, kv, pv, rv,
-                            kfirst, klast);
-  shuffle_clear_counters(smem);
-  __syncthreads();
-  int parity = 0;  // counter buffer of the next staged tile
+// A batch's segments: their tiles and bucket layouts (see k_scatter).
+struct SegArgs {
+  const SegTile *tiles;
+  const uint32_t *base, *nb, *P, *S;
+};
 
-  while (t < tend) {
-    const uint32_t tn = t + tstep;
-    const uint32_t row0 = t * kShTile, rend = min(row0 + kShTile, n);
-    const uint32_t nrow0 = tn < tend ? tn * kShTile : 0u, nrend = tn < tend ? min(nrow0 + kShTile, n) : 0u;
+// Persistent: block b takes tiles b, b + gridDim.x, ...  Per tile:
+//   1. load: keys, then payload and row ids, by asynchronous copies;
+//   2. rank: a row's rank in its bucket is a shared-memory atomicAdd;
+//   3. counts: local starts by a block scan; each (tile, bucket) run's
+//      destination from one atomicAdd on the bucket's cursor, whose result is
+//      needed only at write-out;
+//   4. perm: each row's number goes to its bucket-ordered position;
+//   5. write-out: the columns are gathered through perm and leave as runs.
+// `reg_col`: the first non-key column (-1: none).  EXTRA: further columns,
+// one at a time through the payload's place.
+template <typename KeyT, int MODE, bool EXTRA>
+__global__ void __launch_bounds__(kShNT, kShBlocks)
+    k_shuffle(const KeyT *__restrict__ keys, uint32_t n, uint32_t tile, uint32_t ntiles, const __grid_constant__ BucketSpec bs,
+              uint32_t F, uint32_t F2, uint32_t span, uint32_t *__restrict__ cursors,
+              const __grid_constant__ ColMove cm, int reg_col, const uint32_t *__restrict__ rid_in,
+              uint32_t *__restrict__ rid_out, const SegArgs sg) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int pw = reg_col >= 0 ? cm.width[reg_col] : 0;
+  const ShLayout lay(tile, sizeof(KeyT), EXTRA ? 8 : pw, MODE == SH_PASS2, span);
+  KeyT *skey = (KeyT *)smem;
+  unsigned char *spay = smem + lay.pay;
+  uint32_t *srid = (uint32_t *)(smem + lay.rid);
+  uint32_t *perm = (uint32_t *)(smem + lay.perm);
+  uint32_t *cnt = (uint32_t *)(smem + lay.cnt);
+  uint32_t *lst = cnt + span;
+  uint32_t *gdelta = lst + span;
+  uint32_t *wsum = gdelta + span;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  KeyT *kdst = (KeyT *)cm.dst[cm.key_index];
+  for (uint32_t i = threadIdx.x; i < span; i += kShNT) cnt[i] = 0;
+  __syncthreads();
+
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    SegTile td = {0, 0, 0};
+    if (MODE == SH_SEG) td = sg.tiles[t];
+    const uint32_t row0 = MODE == SH_SEG ? td.row0 : t * tile;
+    const uint32_t rows = MODE == SH_SEG ? td.rows : min(tile, n - row0);
+    // 1. load
+    load_key_pairs<KeyT>(skey, keys + row0, rows);
+    cp_async_commit();
+    if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
+    if (MODE == SH_PASS2) load_column<4>((unsigned char *)srid, (const unsigned char *)(rid_in + row0), rows);
+    cp_async_commit();
     uint32_t lb0 = 0, Floc = F;
-    if (PASS2) {
-      const uint32_t b1f = sub_bucket_of(fmix64(key_bits(kfirst)), bs) / F2;
-      const uint32_t b1l = sub_bucket_of(fmix64(key_bits(klast)), bs) / F2;
+    BucketSpec sp;
+    if (MODE == SH_SEG) {
+      lb0 = sg.base[td.seg];
+      Floc = sg.nb[td.seg];
+      sp = make_spec_dev(sg.P[td.seg]);
+      sp.S = sg.S[td.seg];
+    }
+    if (MODE == SH_PASS2) {
+      const uint32_t b1f = sub_bucket_of(fmix64(key_bits(keys[row0])), bs) / F2;
+      const uint32_t b1l = sub_bucket_of(fmix64(key_bits(keys[row0 + rows - 1])), bs) / F2;
       lb0 = b1f * F2;
       Floc = (b1l - b1f + 1) * F2;
-      if (Floc > kShSpan) {  // uniform over the block: no barrier inside
-        shuffle_direct<KeyT>(keys, row0 + warp * 32 * kRPL, rend, bs, cursors, cm, rid_in, rid_out);
-        if (nrow0 < nrend)
-          shuffle_load<KeyT, PASS2>(keys, nrow0, nrend, cm, reg_col, pw, rid_in, kv, pv, rv, kfirst, klast);
-        t = tn;
+      if (Floc > span) {  // uniform over the block
+        cp_async_wait<0>();
+        __syncthreads();
+        shuffle_direct<KeyT>(skey, srid, row0, rows, bs, cursors, cm, rid_out);
+        __syncthreads();
         continue;
       }
     }
-    shuffle_tile<KeyT, PASS2, EXTRA>(smem, keys, row0, rend, lb0, Floc, bs, cursors, cm, reg_col, pw, rid_in,
-                                     rid_out, kv, pv, rv, nrow0, nrend, kfirst, klast, parity);
-    parity ^= 1;
-    t = tn;
+    // 2. rank
+    cp_async_wait<1>();
+    uint32_t pk[2 * kShPairs];
+#pragma unroll
+    for (int k = 0; k < kShPairs; k++) {
+      const uint32_t r = 2 * (threadIdx.x + k * kShNT);
+      KeyT kv[2];
+      if (sizeof(KeyT) == 8) {
+        const longlong2 v = *(const longlong2 *)(skey + r);
+        kv[0] = (KeyT)v.x, kv[1] = (KeyT)v.y;
+      } else {
+        const int2 v = *(const int2 *)(skey + r);
+        kv[0] = (KeyT)v.x, kv[1] = (KeyT)v.y;
+      }
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        pk[2 * k + e] = 0xFFFFFFFFu;
+        if (r + e < rows) {
+          const uint64_t h = fmix64(key_bits(kv[e]));
+          const uint32_t lb = MODE == SH_PASS1   ? bucket_of(h, bs)
+                              : MODE == SH_PASS2 ? sub_bucket_of(h, bs) - lb0
+                                                 : sub_bucket_of(h, sp);
+          pk[2 * k + e] = (lb << 16) | atomicAdd(&cnt[lb], 1u);
+        }
+      }
+    }
+    __syncthreads();
+    // 3. counts: this thread's buckets [s0, s1); its counters are cleared for the next tile
+    const uint32_t per = (Floc + kShNT - 1) / kShNT;
+    const uint32_t s0 = min(Floc, threadIdx.x * per), s1 = min(Floc, s0 + per);
+    uint32_t cb[kShScan], gb[kShScan], own = 0;
+#pragma unroll
+    for (int i = 0; i < kShScan; i++) {
+      cb[i] = gb[i] = 0;
+      if (s0 + i < s1) {
+        cb[i] = cnt[s0 + i];
+        cnt[s0 + i] = 0;
+        if (cb[i]) gb[i] = atomicAdd(&cursors[lb0 + s0 + i], cb[i]);
+        own += cb[i];
+      }
+    }
+    const uint32_t inc = warp_inclusive_scan(own);
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    uint32_t ex = inc - own;
+#pragma unroll
+    for (int w = 0; w < kShNT / 32; w++)
+      if (w < warp) ex += wsum[w];
+#pragma unroll
+    for (int i = 0; i < kShScan; i++)
+      if (s0 + i < s1) {
+        lst[s0 + i] = ex;
+        gb[i] -= ex;
+        ex += cb[i];
+      }
+    __syncthreads();
+    // 4. perm
+#pragma unroll
+    for (int k = 0; k < kShPairs; k++) {
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        const uint32_t q = pk[2 * k + e];
+        if (q != 0xFFFFFFFFu)
+          perm[lst[q >> 16] + (q & 0xFFFFu)] = (q & 0xFFFF0000u) | (2 * (threadIdx.x + k * kShNT) + e);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kShScan; i++)
+      if (s0 + i < s1) gdelta[s0 + i] = gb[i];
+    cp_async_wait<0>();
+    __syncthreads();
+    // 5. write-out
+#pragma unroll 4
+    for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
+      const uint32_t m = perm[p], i = m & 0xFFFFu;
+      const uint32_t d = p + gdelta[m >> 16];
+      kdst[d] = skey[i];
+      if (pw == 8) ((uint64_t *)cm.dst[reg_col])[d] = ((const uint64_t *)spay)[i];
+      if (pw == 4) ((uint32_t *)cm.dst[reg_col])[d] = ((const uint32_t *)spay)[i];
+      rid_out[d] = MODE == SH_PASS2 ? srid[i] : row0 + i;
+    }
+    __syncthreads();
+    if (EXTRA) {
+#pragma unroll 1
+      for (int j = 0; j < cm.n; j++) {
+        if (j == cm.key_index || j == reg_col) continue;
+        load_payload(spay, cm.src[j], cm.width[j], row0, rows);
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+        if (cm.width[j] == 8)
+          write_column<uint64_t>((uint64_t *)cm.dst[j], (const uint64_t *)spay, perm, gdelta, rows);
+        else
+          write_column<uint32_t>((uint32_t *)cm.dst[j], (const uint32_t *)spay, perm, gdelta, rows);
+        __syncthreads();
+      }
+    }
   }
 }
 
@@ -545,44 +662,56 @@ bool fast_shuffle_enabled() {
 }
 
 template <typename KeyT>
+auto shuffle_kernel(int mode, bool extra) {
+  if (mode == SH_PASS2) return extra ? k_shuffle<KeyT, SH_PASS2, true> : k_shuffle<KeyT, SH_PASS2, false>;
+  if (mode == SH_SEG) return extra ? k_shuffle<KeyT, SH_SEG, true> : k_shuffle<KeyT, SH_SEG, false>;
+  return extra ? k_shuffle<KeyT, SH_PASS1, true> : k_shuffle<KeyT, SH_PASS1, false>;
+}
+
+template <typename KeyT>
 int set_shuffle_attrs() {
   static PerDeviceOnce once;
   return once_per_device(once, [] {
-    const int sm = (int)ShLayout::total;
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_shuffle<KeyT, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_shuffle<KeyT, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_shuffle<KeyT, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_shuffle<KeyT, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    const int sm = (int)kShSmem;
+    for (int extra = 0; extra < 2; extra++)
+      for (int mode = 0; mode < 3; mode++)
+        MDJ_CUDA_TRY(cudaFuncSetAttribute(shuffle_kernel<KeyT>(mode, extra != 0),
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_tot<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kMaxSubBuckets * 4)));
     return (int)MDJ_OK;
   });
 }
 
-template <typename KeyT>
-auto shuffle_kernel(bool pass2, bool extra) {
-  if (pass2) return extra ? k_shuffle<KeyT, true, true> : k_shuffle<KeyT, true, false>;
-  return extra ? k_shuffle<KeyT, false, true> : k_shuffle<KeyT, false, false>;
+// Payload bytes a row takes in a shuffle tile.
+uint32_t shuffle_pay_width(const mdj_table *t, int32_t key_col) {
+  if (t->ncols > 2) return 8;  // any column may pass through
+  return t->ncols < 2 ? 0u : (uint32_t)dtype_width(t->cols[1 - key_col].dtype);
 }
 
-// One unstable shuffle pass (see k_shuffle) of n rows, one block per SM, with
-// run cursors `cur` (pass 1: one per pass-1 bucket; pass 2: one per sub-bucket).
-template <typename KeyT, bool PASS2>
-int shuffle_pass(Workspace &ws, const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32_t F, uint32_t F2,
-                 uint32_t *cur, const ColMove &cm, const uint32_t *rid_in, uint32_t *rid_out) {
-  const uint32_t ntiles = (n + kShTile - 1) / kShTile;
+// One unstable shuffle pass (see k_shuffle) of n rows in tiles of `tile`
+// rows, with run cursors `cur` (pass 1: one per pass-1 bucket; pass 2 and
+// segments: one per sub-bucket).
+template <typename KeyT>
+int shuffle_pass(Workspace &ws, int mode, const KeyT *keys, uint32_t n, uint32_t tile, uint32_t ntiles,
+                 const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, uint32_t *cur, const ColMove &cm,
+                 const uint32_t *rid_in, uint32_t *rid_out, const SegArgs &sg) {
   if (ntiles == 0) return MDJ_OK;
   int reg_col = -1;
   for (int j = 0; j < cm.n && reg_col < 0; j++)
     if (j != cm.key_index) reg_col = j;
-  const uint32_t sms = (uint32_t)num_sms();
-  const uint32_t grid = ntiles < sms ? ntiles : sms;
-  TraceScope tr(PASS2 ? "shuffle_pass2" : "shuffle_pass1", ws.stream());
-  shuffle_kernel<KeyT>(PASS2, cm.n > 2)<<<grid, kShNT, ShLayout::total, ws.stream()>>>(keys, n, ntiles, bs, F, F2, cur,
-                                                                                       cm, reg_col, rid_in, rid_out);
+  const bool extra = cm.n > 2;
+  const uint32_t pw = extra ? 8u : (reg_col >= 0 ? (uint32_t)cm.width[reg_col] : 0u);
+  const uint32_t sm = ShLayout(tile, sizeof(KeyT), pw, mode == SH_PASS2, span).total;
+  const uint32_t most = (uint32_t)num_sms() * kShBlocks;
+  TraceScope tr(mode == SH_SEG ? "seg_scatter" : (mode == SH_PASS2 ? "shuffle_pass2" : "shuffle_pass1"), ws.stream());
+  shuffle_kernel<KeyT>(mode, extra)<<<std::min(ntiles, most), kShNT, sm, ws.stream()>>>(
+      keys, n, tile, ntiles, bs, F, F2, span, cur, cm, reg_col, rid_in, rid_out, sg);
   MDJ_LAUNCH_CHECK();
   return MDJ_OK;
 }
+
+uint32_t tiles_of(uint32_t n, uint32_t tile) { return (uint32_t)(((uint64_t)n + tile - 1) / tile); }
 
 // The merge's partition of one side with the unstable passes, first half:
 // count the final sub-buckets, scan them into `off`, then the only pass
@@ -630,7 +759,9 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   MDJ_LAUNCH_CHECK();
   ColMove cm = make_move(t, key_col, src, out->cols);
   const BucketSpec spec1 = plan.F2 == 1 ? sub : make_spec(plan.P, plan.S, plan.F2);
-  MDJ_TRY((shuffle_pass<KeyT, false>(ws, keys, n, spec1, F1, plan.F2, cur, cm, nullptr, out->rid)));
+  const uint32_t tile = shuffle_tile_rows(sizeof(KeyT), shuffle_pay_width(t, key_col), false, F1);
+  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS1, keys, n, tile, tiles_of(n, tile), spec1, F1, plan.F2, F1, cur, cm, nullptr,
+                             out->rid, SegArgs{}));
   ws.give_back(cur);
   return MDJ_OK;
 }
@@ -644,8 +775,13 @@ int shuffle_pass2_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Pl
   MDJ_TRY(alloc_table_bufs(ws, t, fin, true));
   if (n == 0) return MDJ_OK;
   ColMove cm2 = make_move(t, key_col, p1.cols, fin->cols);
-  MDJ_TRY((shuffle_pass<KeyT, true>(ws, (const KeyT *)p1.cols[key_col], n, make_spec(plan.P, plan.S, 1), 0, plan.F2,
-                                    cur, cm2, p1.rid, fin->rid)));
+  // local buckets of a tile: the pass-1 buckets it is expected to touch (two
+  // at least); a tile that touches more (a run of small ones) goes direct
+  const uint64_t touched = 2 + (uint64_t)kShMaxTile * plan.F1 / n;
+  const uint32_t span = (uint32_t)std::min<uint64_t>(touched * plan.F2, kPass2SpanMax);
+  const uint32_t tile = shuffle_tile_rows(sizeof(KeyT), shuffle_pay_width(t, key_col), true, span);
+  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS2, (const KeyT *)p1.cols[key_col], n, tile, tiles_of(n, tile),
+                             make_spec(plan.P, plan.S, 1), 0, plan.F2, span, cur, cm2, p1.rid, fin->rid, SegArgs{}));
   ws.give_back(cur);
   return MDJ_OK;
 }

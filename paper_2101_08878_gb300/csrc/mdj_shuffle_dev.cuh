@@ -57,209 +57,154 @@ __device__ void scatter_direct(const KeyT (&kv)[kRPL], uint32_t wrow0, uint32_t 
 
 // ---------------------------------------------------------------- k_shuffle
 //
-// One block of kShNT threads per SM, tiles of kShTile rows (kRPL per thread),
-// at most kShSpan local buckets per tile.  Shared memory per block:
-//   rec    [kShTile]  16 bytes: key bits, first non-key column (bucket order)
-//   meta   [kShTile]   4 bytes: pass 1: (row in tile << 10) | local bucket;
-//                               pass 2: the row id (the local bucket is
-//                               recomputed from the key at write-out: cheaper
-//                               than staging it, measured)
-//   cnt    [2][kShSpan] rank counters (two buffers, alternating tiles)
-//   lst    [kShSpan]   local start of each bucket in the staged tile
-//   gdelta [kShSpan]   destination - staged position, per bucket
-//   wsum   [32]        warp sums of the count scan
-constexpr int kShNT = 1024;
-constexpr uint32_t kShTile = (uint32_t)kShNT * kRPL;  // 8192 rows
-constexpr uint32_t kShSpan = kShNT;                   // one local bucket per thread
-static_assert(kShSpan <= 1024, "pass-1 metadata keeps the local bucket in 10 bits");
-static_assert(kShTile <= (1u << 22), "pass-1 metadata keeps the row in tile in 22 bits");
+// Two blocks of kShNT threads per SM, each with a tile of as many rows as its
+// half of the shared memory holds (5,700 rows of an 8-byte key and payload):
+//   key  [tile]   the key column
+//   pay  [tile]   the first non-key column (every further one in turn)
+//   rid  [tile]   pass 2: row ids
+//   perm [tile]   bucket-ordered position -> local bucket << 16 | row in tile
+//   cnt, lst, gdelta [span]  per local bucket: rank counter, local start,
+//                 destination - position (modulo 2^32)
+//   wsum [32]     warp sums of the count scan
+// Row data stays in input order, brought in by 16-byte asynchronous copies,
+// so no tile data waits in registers, and only the 4-byte perm entry is
+// scattered in shared memory.
+//
+// What bounds it: DRAM, while the runs a tile writes are long (a run is about
+// tile / buckets rows; its two ends are partial 32-byte sectors).  Measured
+// per 1e8 rows of 8 + 8 + 4 bytes: runs of 44 rows 0.62 ms (5.8 TB/s), of 36
+// 0.65, of 28 0.71, of 19 0.80.  So the tile is as large as two blocks per SM
+// allow, and the blocks' load, rank and write-out phases overlap each other.
+// Before (one 1024-thread block per SM, rows held in registers and staged as
+// 16-byte records): 0.83 ms in pass 1 and 0.95 ms in pass 2, now 0.62 and
+// 0.77 (1e8 rows, 28.7K sub-buckets).  Three blocks of 448 threads with
+// smaller tiles: 0.71 and 0.84; 640 or 768 threads: 0.62 and 0.82.
+constexpr int kShNT = 512;
+constexpr int kShPairs = 6;                               // row pairs per thread per tile at most
+constexpr int kShBlocks = 2;                              // blocks per SM
+constexpr uint32_t kShMaxTile = (uint32_t)kShNT * kShPairs * 2;
+constexpr uint32_t kShSmem = 228u * 1024 / kShBlocks - 1024;  // shared memory of a block
+constexpr int kShScan = (1024 + kShNT - 1) / kShNT;       // local buckets a thread scans at most
+static_assert(kShMaxTile <= 65536, "perm keeps the row in tile in 16 bits");
 
+enum { SH_PASS1 = 0, SH_PASS2 = 1, SH_SEG = 2 };
+
+// Shared memory of a block for tiles of `tile` rows (a multiple of 16) and
+// `span` local buckets.
 struct ShLayout {
-  static constexpr size_t rec = 0;
-  static constexpr size_t meta = rec + (size_t)kShTile * 16;
-  static constexpr size_t cnt = meta + (size_t)kShTile * 4;
-  static constexpr size_t lst = cnt + (size_t)2 * kShSpan * 4;
-  static constexpr size_t gdelta = lst + (size_t)kShSpan * 4;
-  static constexpr size_t wsum = gdelta + (size_t)kShSpan * 4;
-  static constexpr size_t total = wsum + 32 * 4;
+  uint32_t pay, rid, perm, cnt, total;
+  __host__ __device__ ShLayout(uint32_t tile, uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t span) {
+    pay = tile * key_width;
+    rid = pay + tile * pay_width;
+    perm = rid + (with_rid ? tile * 4 : 0u);
+    cnt = perm + tile * 4;
+    total = cnt + (3 * span + 32) * 4;
+  }
 };
 
-// scatter_direct for k_shuffle, reading the keys again from memory so that
-// the caller's key registers need no addressable copy.
+// Rows of the largest tile that fits a block's shared memory.
+inline uint32_t shuffle_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t span) {
+  const uint32_t row = key_width + pay_width + (with_rid ? 4u : 0u) + 4u;
+  const uint32_t rows = (kShSmem - (3 * span + 32) * 4) / row / 16 * 16;
+  return rows < kShMaxTile ? rows : kShMaxTile;
+}
+
+template <int W>
+__device__ __forceinline__ void cp_async(void *dst, const void *src) {
+  if (W == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)),
+                 "l"(__cvta_generic_to_global(src))
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)),
+                 "l"(__cvta_generic_to_global(src)), "n"(W)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// `rows` elements of W bytes from src to the 16-byte-aligned dst: 16-byte
+// copies where src is 16-byte aligned, else one copy per element.
+template <int W>
+__device__ __forceinline__ void load_column(unsigned char *dst, const unsigned char *src, uint32_t rows) {
+  uint32_t done = 0;
+  if (((uintptr_t)src & 15) == 0) {
+    const uint32_t n16 = rows * W / 16;
+    for (uint32_t c = threadIdx.x; c < n16; c += kShNT) cp_async<16>(dst + c * 16, src + (size_t)c * 16);
+    done = n16 * (16 / W);
+  }
+  for (uint32_t i = done + threadIdx.x; i < rows; i += kShNT) cp_async<W>(dst + i * W, src + (size_t)i * W);
+}
+
+__device__ __forceinline__ void load_payload(unsigned char *dst, const void *col, int width, uint32_t row0,
+                                             uint32_t rows) {
+  if (width == 8) load_column<8>(dst, (const unsigned char *)col + (size_t)row0 * 8, rows);
+  if (width == 4) load_column<4>(dst, (const unsigned char *)col + (size_t)row0 * 4, rows);
+}
+
+// Keys of the row pairs this thread ranks: rows 2q, 2q + 1 of the tile, q =
+// threadIdx.x + k * kShNT, so that a thread reads only keys it copied itself
+// (visible after its own wait, no barrier).
 template <typename KeyT>
-__device__ __noinline__ void shuffle_direct(const KeyT *__restrict__ keys, uint32_t wrow0, uint32_t rend,
+__device__ __forceinline__ void load_key_pairs(KeyT *skey, const KeyT *keys, uint32_t rows) {
+  constexpr int W2 = 2 * (int)sizeof(KeyT);
+  const bool al = ((uintptr_t)keys & (W2 - 1)) == 0;
+#pragma unroll
+  for (int k = 0; k < kShPairs; k++) {
+    const uint32_t r = 2 * (threadIdx.x + k * kShNT);
+    if (al && r + 1 < rows) {
+      cp_async<W2>(skey + r, keys + r);
+    } else {
+      if (r < rows) cp_async<(int)sizeof(KeyT)>(skey + r, keys + r);
+      if (r + 1 < rows) cp_async<(int)sizeof(KeyT)>(skey + r + 1, keys + r + 1);
+    }
+  }
+}
+
+// A pass-2 tile whose rows span too many buckets for shared memory (tiny or
+// very skewed pass-1 buckets): warp-aggregated reservation, each row written
+// straight to its slot.  key/rid come from the staged tile.
+template <typename KeyT>
+__device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *srid, uint32_t row0, uint32_t rows,
                                             const BucketSpec &bs, uint32_t *__restrict__ cursors, const ColMove &cm,
-                                            const uint32_t *__restrict__ rid_in, uint32_t *__restrict__ rid_out) {
-  KeyT kv[kRPL];
-#pragma unroll
-  for (int c = 0; c < kRPL; c++) {
-    const uint32_t r = wrow0 + c * 32 + (threadIdx.x & 31);
-    kv[c] = r < rend ? keys[r] : KeyT(0);
-  }
-  scatter_direct<KeyT>(kv, wrow0, rend, bs, cursors, cm, rid_in, rid_out);
-}
-
-// Loads the carried columns of the tile of rows [row0, rend) into registers:
-// warp w holds rows row0 + w*256 + c*32 + lane (c < kRPL), the layout
-// scatter_direct uses.  PASS2 also loads the row ids and the tile's first
-// and last key (its pass-1 bucket span).
-template <typename KeyT, bool PASS2>
-__device__ __forceinline__ void shuffle_load(const KeyT *__restrict__ keys, uint32_t row0, uint32_t rend,
-                                             const ColMove &cm, int reg_col, int pw,
-                                             const uint32_t *__restrict__ rid_in, KeyT (&kv)[kRPL],
-                                             uint64_t (&pv)[kRPL], uint32_t (&rv)[kRPL], KeyT &kfirst,
-                                             KeyT &klast) {
-  const uint32_t wrow0 = row0 + (threadIdx.x >> 5) * 32 * kRPL;
+                                            uint32_t *__restrict__ rid_out) {
   const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int c = 0; c < kRPL; c++) {
-    const uint32_t r = wrow0 + c * 32 + lane;
-    const bool ok = r < rend;
-    kv[c] = ok ? keys[r] : KeyT(0);
-    pv[c] = 0;
-    if (ok && pw == 8) pv[c] = ((const uint64_t *)cm.src[reg_col])[r];
-    if (ok && pw == 4) pv[c] = ((const uint32_t *)cm.src[reg_col])[r];
-    if (PASS2) rv[c] = ok ? rid_in[r] : 0u;
-  }
-  if (PASS2) {
-    kfirst = keys[row0];
-    klast = keys[rend - 1];
-  }
-}
-
-// One staged tile: rows [row0, rend) (at most kShTile) whose columns are in
-// registers, local buckets [lb0, lb0 + Floc) (Floc <= kShSpan).
-//   1. rank: a row's rank in its bucket is a shared-memory atomicAdd;
-//   2. counts: thread b scans bucket b's count into its local start and
-//      reserves the run's destination with one atomicAdd on
-//      cursors[lb0 + b], whose result is needed only at write-out (its
-//      latency overlaps the scan and the staging);
-//   3. stage: each row goes to its bucket-ordered slot (16-byte record and
-//      4-byte meta); the other counter buffer is cleared for the next tile;
-//   4. the next tile's columns load into the freed registers (unless EXTRA);
-//   5. write-out: consecutive threads store consecutive rows of one run;
-//   6. EXTRA: every further column, one at a time through the record's
-//      payload half.
-// Four block barriers per tile.
-template <typename KeyT, bool PASS2, bool EXTRA>
-__device__ __forceinline__ void shuffle_tile(unsigned char *smem, const KeyT *__restrict__ keys, uint32_t row0,
-                                             uint32_t rend, uint32_t lb0, uint32_t Floc, const BucketSpec &bs,
-                                             uint32_t *__restrict__ cursors, const ColMove &cm, int reg_col, int pw,
-                                             const uint32_t *__restrict__ rid_in, uint32_t *__restrict__ rid_out,
-                                             KeyT (&kv)[kRPL], uint64_t (&pv)[kRPL], uint32_t (&rv)[kRPL],
-                                             uint32_t next_row0, uint32_t next_rend, KeyT &kfirst, KeyT &klast,
-                                             int parity) {
-  ulonglong2 *rec = (ulonglong2 *)(smem + ShLayout::rec);
-  uint32_t *meta = (uint32_t *)(smem + ShLayout::meta);
-  uint32_t *cnt = (uint32_t *)(smem + ShLayout::cnt) + (size_t)parity * kShSpan;
-  uint32_t *cnt_next = (uint32_t *)(smem + ShLayout::cnt) + (size_t)(1 - parity) * kShSpan;
-  uint32_t *lst = (uint32_t *)(smem + ShLayout::lst);
-  uint32_t *gdelta = (uint32_t *)(smem + ShLayout::gdelta);  // modulo 2^32
-  uint32_t *wsum = (uint32_t *)(smem + ShLayout::wsum);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rows = rend - row0;
-  const uint32_t wl0 = (uint32_t)warp * 32 * kRPL;  // this warp's first row in the tile
-  const uint32_t b = threadIdx.x;                    // the local bucket this thread scans
-
-
-  // 1. rank
-  uint32_t pk[kRPL];
-#pragma unroll
-  for (int c = 0; c < kRPL; c++) {
-    pk[c] = 0xFFFFFFFFu;
-    if (row0 + wl0 + c * 32 + lane < rend) {
-      const uint64_t h = fmix64(key_bits(kv[c]));
-      const uint32_t lb = (PASS2 ? sub_bucket_of(h, bs) : bucket_of(h, bs)) - lb0;
-      pk[c] = (lb << 16) | atomicAdd(&cnt[lb], 1u);
-    }
-  }
-  __syncthreads();
-
-  // 2. counts: local starts by a block scan; the run's destination
-  const uint32_t cb = b < Floc ? cnt[b] : 0u;
-  const uint32_t gb = cb ? atomicAdd(&cursors[lb0 + b], cb) : 0u;
-  const uint32_t inc = warp_inclusive_scan(cb);
-  if (lane == 31) wsum[warp] = inc;
-  __syncthreads();
-  uint32_t before = 0;
-#pragma unroll
-  for (int w = 0; w < kShNT / 32; w++)
-    if (w < warp) before += wsum[w];
-  const uint32_t ex = before + inc - cb;
-  if (b < Floc) lst[b] = ex;
-  __syncthreads();
-
-  // 3. stage
-  cnt_next[threadIdx.x] = 0;
-#pragma unroll
-  for (int c = 0; c < kRPL; c++) {
-    if (pk[c] != 0xFFFFFFFFu) {
-      const uint32_t lb = pk[c] >> 16, rank = pk[c] & 0xFFFFu;
-      const uint32_t lp = lst[lb] + rank;
-      uint64_t kb = 0;
-      memcpy(&kb, &kv[c], sizeof(KeyT));
-      rec[lp] = make_ulonglong2(kb, pv[c]);
-      meta[lp] = PASS2 ? rv[c] : (((wl0 + c * 32 + lane) << 10) | lb);
-    }
-  }
-  if (b < Floc) gdelta[b] = gb - ex;
-  __syncthreads();
-  if (!EXTRA && next_row0 < next_rend)
-    shuffle_load<KeyT, PASS2>(keys, next_row0, next_rend, cm, reg_col, pw, rid_in, kv, pv, rv, kfirst, klast);
-
-  // 5. write-out
-  KeyT *kdst = (KeyT *)cm.dst[cm.key_index];
-  for (uint32_t i = threadIdx.x; i < rows; i += kShNT) {
-    const ulonglong2 r = rec[i];
-    const uint32_t m = meta[i];
-    KeyT k;
-    memcpy(&k, &r.x, sizeof(KeyT));
-    const uint32_t lb = PASS2 ? sub_bucket_of(fmix64(key_bits(k)), bs) - lb0 : (m & 0x3FFu);
-    const uint32_t d = i + gdelta[lb];
-    kdst[d] = k;
-    if (pw == 8) ((uint64_t *)cm.dst[reg_col])[d] = r.y;
-    if (pw == 4) ((uint32_t *)cm.dst[reg_col])[d] = (uint32_t)r.y;
-    if (rid_out) rid_out[d] = PASS2 ? m : row0 + (m >> 10);
-  }
-
-  // 6. further columns, one at a time through the payload half of the stage
-  if (EXTRA) {
+  for (uint32_t i0 = threadIdx.x & ~31u; i0 < rows; i0 += kShNT) {
+    const uint32_t i = i0 + lane;
+    const bool valid = i < rows;
+    const KeyT k = valid ? skey[i] : KeyT(0);
+    const uint32_t fb = valid ? sub_bucket_of(fmix64(key_bits(k)), bs) : 0xFFFFFFFFu;
+    const uint32_t peers = __match_any_sync(0xffffffffu, fb);
+    const int leader = __ffs(peers) - 1;
+    uint32_t base = 0;
+    if (valid && lane == leader) base = atomicAdd(&cursors[fb], (uint32_t)__popc(peers));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (!valid) continue;
+    const uint32_t pos = base + __popc(peers & lanemask_lt());
+    const size_t r = (size_t)row0 + i;
     for (int j = 0; j < cm.n; j++) {
-      if (j == cm.key_index || j == reg_col) continue;
-      const int w = cm.width[j];
-      uint64_t val[kRPL];
-#pragma unroll
-      for (int c = 0; c < kRPL; c++) {
-        const uint32_t r = row0 + wl0 + c * 32 + lane;
-        val[c] = 0;
-        if (r < rend) val[c] = w == 8 ? ((const uint64_t *)cm.src[j])[r] : ((const uint32_t *)cm.src[j])[r];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int c = 0; c < kRPL; c++)
-        if (pk[c] != 0xFFFFFFFFu) rec[lst[pk[c] >> 16] + (pk[c] & 0xFFFFu)].y = val[c];
-      __syncthreads();
-      for (uint32_t i = threadIdx.x; i < rows; i += kShNT) {
-        const ulonglong2 r = rec[i];
-        KeyT k;
-        memcpy(&k, &r.x, sizeof(KeyT));
-        const uint32_t lb = PASS2 ? sub_bucket_of(fmix64(key_bits(k)), bs) - lb0 : (meta[i] & 0x3FFu);
-        const uint32_t d = i + gdelta[lb];
-        if (w == 8)
-          ((uint64_t *)cm.dst[j])[d] = r.y;
-        else
-          ((uint32_t *)cm.dst[j])[d] = (uint32_t)r.y;
-      }
+      if (cm.width[j] == 8)
+        ((uint64_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint64_t)k : ((const uint64_t *)cm.src[j])[r];
+      else
+        ((uint32_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint32_t)k : ((const uint32_t *)cm.src[j])[r];
     }
-    if (next_row0 < next_rend)
-      shuffle_load<KeyT, PASS2>(keys, next_row0, next_rend, cm, reg_col, pw, rid_in, kv, pv, rv, kfirst, klast);
+    rid_out[pos] = srid[i];
   }
 }
 
-// Clears both counter buffers of shuffle_tile (block-wide, no barrier).
-__device__ __forceinline__ void shuffle_clear_counters(unsigned char *smem) {
-  uint32_t *cnt = (uint32_t *)(smem + ShLayout::cnt);
-  for (uint32_t i = threadIdx.x; i < 2 * kShSpan; i += kShNT) cnt[i] = 0;
+// One column of the staged tile to its destinations: consecutive threads
+// store consecutive rows of one run.
+template <typename V>
+__device__ __forceinline__ void write_column(V *__restrict__ dst, const V *stage, const uint32_t *perm,
+                                             const uint32_t *gdelta, uint32_t rows) {
+#pragma unroll 4
+  for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
+    const uint32_t m = perm[p];
+    dst[p + gdelta[m >> 16]] = stage[m & 0xFFFFu];
+  }
 }
 
 }  // namespace

@@ -1,0 +1,81 @@
+"""The merge's shuffle at the edges of its tiles: ragged sizes, columns that
+start off a 16-byte boundary, several columns, and pass-2 tiles that touch
+many pass-1 buckets.  Every result against the oracle, bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from joinhelp import assert_same_result, gpu_result_np
+from paper_2101_08878_gb300 import datagen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def _shifted(cols, shift):
+    """Device copies of `cols` that start `shift` elements into their allocations."""
+    out = []
+    for c in cols:
+        t = torch.empty(c.size + shift, dtype=torch.from_numpy(c).dtype, device=DEV)
+        t[shift:] = torch.from_numpy(c).to(DEV)
+        out.append(t[shift:])
+    return out
+
+
+def _check(left, right, P, shift=0):
+    from paper_2101_08878_gb300 import mdj
+    res = mdj.mdj_merge(_shifted(left, shift), _shifted(right, shift), P)
+    torch.cuda.synchronize()
+    assert_same_result(gpu_result_np(res), oracle.merge_table(left, right, 0, 0))
+
+
+def _tables(nl, nr, kd, pd, seed):
+    rng = np.random.default_rng(seed)
+    span = max(2, 2 * max(nl, nr))
+    lk = rng.permutation(span)[:nl].astype(kd)
+    rk = rng.integers(0, span, nr).astype(kd)
+    return [lk, datagen.uniform_payload(rng, nl, pd)], [rk, datagen.uniform_payload(rng, nr, pd)]
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 17, 5167, 5168, 5169, 5695, 5696, 5697, 6143, 6144, 6145, 12_289])
+@pytest.mark.parametrize("kd,pd", [(np.int64, np.float64), (np.int32, np.float32)])
+def test_tile_edges(n, kd, pd):
+    left, right = _tables(n, n + 1, kd, pd, n)
+    for P in (2, 128, 1000):
+        _check(left, right, P)
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("kd,pd", [(np.int64, np.float64), (np.int32, np.float32), (np.int64, np.float32),
+                                   (np.int32, np.float64)])
+def test_unaligned_columns(shift, kd, pd):
+    left, right = _tables(40_003, 50_001, kd, pd, shift)
+    _check(left, right, 8, shift)
+
+
+@pytest.mark.parametrize("ncols", [0, 1, 2, 4])
+def test_column_counts(ncols):
+    rng = np.random.default_rng(ncols)
+    left, right = _tables(30_011, 20_013, np.int64, np.float64, 9)
+    kinds = [np.float32, np.float64, np.float32, np.float64]
+    left = left[:1] + [datagen.uniform_payload(rng, 30_011, k) for k in kinds[:ncols]]
+    right = right[:1] + [datagen.uniform_payload(rng, 20_013, k) for k in kinds[:ncols]]
+    _check(left, right, 8, 1)
+
+
+@pytest.mark.parametrize("nr", [3, 1000, 60_001, 400_003])
+def test_two_level_plan_small_probe_side(nr):
+    # the plan follows the 4M-row build side, so a small probe side's pass-1
+    # buckets are shorter than a tile
+    left, right = _tables(4_000_003, nr, np.int64, np.float64, 5)
+    _check(left, right, 8, 1)
+
+
+def test_two_level_plan_few_distinct_keys():
+    # rows of a handful of pass-1 buckets far apart: tiles go direct
+    rng = np.random.default_rng(6)
+    left, _ = _tables(4_000_000, 1, np.int32, np.float32, 7)
+    rk = rng.choice(left[0][:5], 30_000)
+    _check(left, [rk, datagen.uniform_payload(rng, rk.size, np.float32)], 8)
