@@ -79,3 +79,25 @@ def test_two_level_plan_few_distinct_keys():
     left, _ = _tables(4_000_000, 1, np.int32, np.float32, 7)
     rk = rng.choice(left[0][:5], 30_000)
     _check(left, [rk, datagen.uniform_payload(rng, rk.size, np.float32)], 8)
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("kd,pd", [(np.int64, np.float64), (np.int32, np.float32)])
+def test_batch_segments_of_ragged_sizes(kd, pd, shift):
+    # segments start at any row, hold less than a tile or several, and differ in bucket counts
+    from paper_2101_08878_gb300 import mdj
+    nl = [1, 0, 5, 5183, 5184, 12_345, 3, 40_001, 700_001]
+    nr = [2, 7, 0, 5185, 11_111, 1, 8192, 90_003, 50_001]
+    P = [1, 8, 3, 32, 1, 1000, 8, 7, 1]
+    pairs = [_tables(a, b, kd, pd, 100 + i) for i, (a, b) in enumerate(zip(nl, nr))]
+    left = [np.concatenate([p[0][c] for p in pairs]) for c in (0, 1)]
+    right = [np.concatenate([p[1][c] for p in pairs]) for c in (0, 1)]
+    lo, ro = np.concatenate([[0], np.cumsum(nl)]), np.concatenate([[0], np.cumsum(nr)])
+    res, offs = mdj.mdj_merge_batch(_shifted(left, shift), _shifted(right, shift), lo, ro, P)
+    torch.cuda.synchronize()
+    for i, (l, r) in enumerate(pairs):
+        a, b = offs[i], offs[i + 1]
+        part = mdj.JoinResult(b - a, res.key[a:b], res.left_row.view(torch.int32)[a:b] - int(lo[i]),
+                              res.right_row.view(torch.int32)[a:b] - int(ro[i]), [c[a:b] for c in res.left_cols],
+                              [c[a:b] for c in res.right_cols])
+        assert_same_result(gpu_result_np(part), oracle.merge_table(l, r, 0, 0))
