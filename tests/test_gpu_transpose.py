@@ -68,3 +68,19 @@ def test_transpose_add_paper_size_20e3():
     x = _random(20_000, np.float64, seed=20)
     y = _mdj().transpose_add(torch.from_numpy(x).to(DEV))
     assert np.array_equal(_bits(y.cpu().numpy()), _bits(oracle.transpose_add(x)))
+
+
+@pytest.mark.parametrize("n", [4, 60, 252, 776])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32, np.int64, np.int32])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_transpose_add_words_and_single_elements(n, dtype, shift):
+    # rows on 16-byte boundaries (shift 0) and off them, out of place and in place
+    x = _random(n, dtype, seed=n + shift)
+    want = _bits(oracle.transpose_add(x))
+    flat = torch.empty(n * n + shift, dtype=torch.from_numpy(x).dtype, device=DEV)
+    t = flat[shift:].view(n, n)
+    t.copy_(torch.from_numpy(x))
+    y = _mdj().transpose_add(t)
+    assert np.array_equal(_bits(y.cpu().numpy()), want)
+    _mdj().transpose_add(t, out=t)
+    assert np.array_equal(_bits(t.cpu().numpy()), want)
