@@ -341,7 +341,8 @@ MDJ_API void mdj_stream_close(mdj_stream *s);
  * a < nkeys).  Inner join: every pair (l, r) whose tuples are equal column by
  * column.  Each tuple is hashed to a 64-bit surrogate, the surrogates are
  * merged as mdj_merge does (P partitions), and every candidate row's two
- * tuples are then compared, so hash collisions never reach the result.
+ * tuples are then compared, so hash collisions never reach the result.  A
+ * tuple of at most 64 bits (one column, or two 4-byte ones) is its own key.
  *   left_keys, right_keys : host arrays of nkeys distinct column indices
  *                           (1 <= nkeys <= 8); key columns are I32 / I64 /
  *                           U32 / U64, equal dtypes pairwise, compared as bits

@@ -7,6 +7,11 @@
 // collisions) are dropped.  Equal tuples always have equal surrogates, so no
 // pair is lost, and the comparison removes every false one: the result is
 // exactly the inner equi-join on all key columns.
+//
+// A tuple of at most 64 bits (two 4-byte columns, or one column) needs no
+// surrogate: its bits are the merge's key, the key columns are not carried
+// and nothing is compared afterwards.  Two int32 key columns, 2e7 x 2e7 rows:
+// kernels 1.69 -> 1.05 ms.
 #include <stdlib.h>
 #include <string.h>
 
@@ -43,6 +48,40 @@ __global__ void k_tuple_hash(const __grid_constant__ KeyCols K, uint64_t n, int 
     }
     out[i] = h;
   }
+}
+
+// Two 4-byte key columns as one 64-bit key and back: a in the low half.
+// Four rows per step where every array starts on a 16-byte boundary.
+// Streaming: 16 bytes per row.
+__global__ void k_tuple_pack(const uint32_t *__restrict__ a, const uint32_t *__restrict__ b, uint64_t n, int vec,
+                             uint64_t *__restrict__ out) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t nv = vec ? n / 4 : 0;
+  for (uint64_t i = t0; i < nv; i += stride) {
+    const uint4 x = ((const uint4 *)a)[i], y = ((const uint4 *)b)[i];
+    ((uint4 *)out)[2 * i] = make_uint4(x.x, y.x, x.y, y.y);
+    ((uint4 *)out)[2 * i + 1] = make_uint4(x.z, y.z, x.w, y.w);
+  }
+  for (uint64_t i = nv * 4 + t0; i < n; i += stride) out[i] = a[i] | (uint64_t)b[i] << 32;
+}
+
+__global__ void k_tuple_unpack(const uint64_t *__restrict__ in, uint64_t n, int vec, uint32_t *__restrict__ a,
+                               uint32_t *__restrict__ b) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t nv = vec ? n / 4 : 0;
+  for (uint64_t i = t0; i < nv; i += stride) {
+    const uint4 x = ((const uint4 *)in)[2 * i], y = ((const uint4 *)in)[2 * i + 1];
+    ((uint4 *)a)[i] = make_uint4(x.x, x.z, y.x, y.z);
+    ((uint4 *)b)[i] = make_uint4(x.y, x.w, y.y, y.w);
+  }
+  for (uint64_t i = nv * 4 + t0; i < n; i += stride) {
+    a[i] = (uint32_t)in[i];
+    b[i] = (uint32_t)(in[i] >> 32);
+  }
+}
+
+int aligned16(const void *a, const void *b, const void *c) {
+  return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15) == 0;
 }
 
 // keep[i] = 1 if candidate row i's left and right key tuples are equal;
@@ -114,6 +153,81 @@ bool is_key(const int32_t *keys, int32_t nkeys, int j) {
   return false;
 }
 
+// The merge on tuples whose bits are the key: one key column, or two 4-byte ones.
+int merge_packed(const mdj_table *left, const int32_t *lkeys, const mdj_table *right, const int32_t *rkeys,
+                 int32_t nkeys, uint32_t P, const mdj_allocator *alloc, void *stream, mdj_result *out) {
+  cudaStream_t s = (cudaStream_t)stream;
+  Workspace ws(alloc, s);
+  mdj_col cols[2][MDJ_MAX_COLS];
+  const mdj_table *sides[2] = {left, right};
+  const int32_t *keys[2] = {lkeys, rkeys};
+  mdj_table tabs[2];
+  for (int side = 0; side < 2; side++) {
+    const mdj_table *t = sides[side];
+    const mdj_col k0 = t->cols[keys[side][0]];
+    int c = 0;
+    if (nkeys == 1) {
+      cols[side][c++] = {k0.data, dtype_width(k0.dtype) == 8 ? MDJ_I64 : MDJ_I32};
+    } else {
+      const mdj_col k1 = t->cols[keys[side][1]];
+      uint64_t *packed = (uint64_t *)ws.get((size_t)(t->nrows ? t->nrows : 1) * 8);
+      if (!packed) return MDJ_ERR_OOM;
+      if (t->nrows) {
+        TraceScope tr("tuple_pack", s);
+        k_tuple_pack<<<grid_of(t->nrows), 256, 0, s>>>((const uint32_t *)k0.data, (const uint32_t *)k1.data, t->nrows,
+                                                       aligned16(k0.data, k1.data, packed), packed);
+      }
+      MDJ_LAUNCH_CHECK();
+      cols[side][c++] = {packed, MDJ_I64};
+    }
+    for (int j = 0; j < t->ncols; j++)
+      if (!is_key(keys[side], nkeys, j)) cols[side][c++] = t->cols[j];
+    tabs[side] = {cols[side], c, t->nrows};
+  }
+  mdj_result in;
+  MDJ_TRY(mdj_merge(&tabs[0], 0, &tabs[1], 0, P, alloc, stream, &in));
+  const uint64_t m = in.nrows;
+  mdj_result r = in;
+  r.key = nullptr;
+  r.key_dtype = 0;
+  r.n_left_cols = in.n_left_cols + nkeys;
+  for (int a = 0; a < nkeys; a++) {
+    r.left_dtypes[a] = left->cols[lkeys[a]].dtype;
+    r.left_cols[a] = nullptr;
+  }
+  for (int j = 0; j < in.n_left_cols; j++) {
+    r.left_dtypes[nkeys + j] = in.left_dtypes[j];
+    r.left_cols[nkeys + j] = in.left_cols[j];
+  }
+  if (nkeys == 1) {
+    r.left_cols[0] = in.key;
+  } else if (m) {
+    int rc = MDJ_OK;
+    for (int a = 0; a < 2; a++)
+      if (!(r.left_cols[a] = ws.get_owned_by_caller((size_t)m * 4))) rc = MDJ_ERR_OOM;
+    if (rc == MDJ_OK) {
+      TraceScope tr("tuple_unpack", s);
+      k_tuple_unpack<<<grid_of(m), 256, 0, s>>>((const uint64_t *)in.key, m,
+                                                aligned16(in.key, r.left_cols[0], r.left_cols[1]),
+                                                (uint32_t *)r.left_cols[0], (uint32_t *)r.left_cols[1]);
+      rc = cuda_status(cudaGetLastError());
+    }
+    ws.release_caller(in.key);
+    if (rc != MDJ_OK) {
+      mdj_result_release(&r, alloc, stream);
+      return rc;
+    }
+  }
+  // the result is complete on return, as where the tuples are compared
+  const int rc = cuda_status(cudaStreamSynchronize(s));
+  if (rc != MDJ_OK) {
+    mdj_result_release(&r, alloc, stream);
+    return rc;
+  }
+  *out = r;
+  return MDJ_OK;
+}
+
 int merge_multi_impl(const mdj_table *left, const int32_t *lkeys, const mdj_table *right, const int32_t *rkeys,
                      int32_t nkeys, uint32_t P, const mdj_allocator *alloc, void *stream, mdj_result *out) {
   if (!out || !lkeys || !rkeys || nkeys < 1 || nkeys > kMaxKeys) return MDJ_ERR_INVALID_ARG;
@@ -123,6 +237,11 @@ int merge_multi_impl(const mdj_table *left, const int32_t *lkeys, const mdj_tabl
   for (int a = 0; a < nkeys; a++)
     if (left->cols[lkeys[a]].dtype != right->cols[rkeys[a]].dtype) return MDJ_ERR_INVALID_ARG;
   if (P < 1 || P > MDJ_MAX_PARTITIONS) return MDJ_ERR_INVALID_ARG;
+  const int weak = weak_hash_for_tests();
+  const bool two_words = nkeys == 2 && dtype_width(left->cols[lkeys[0]].dtype) == 4 &&
+                         dtype_width(left->cols[lkeys[1]].dtype) == 4;
+  if (!weak && (nkeys == 1 || two_words))
+    return merge_packed(left, lkeys, right, rkeys, nkeys, P, alloc, stream, out);
   cudaStream_t s = (cudaStream_t)stream;
   Workspace ws(alloc, s);
 
@@ -132,7 +251,6 @@ int merge_multi_impl(const mdj_table *left, const int32_t *lkeys, const mdj_tabl
   const int32_t *keys[2] = {lkeys, rkeys};
   mdj_col *cols[2] = {lc, rc};
   mdj_table tabs[2];
-  const int weak = weak_hash_for_tests();
   for (int side = 0; side < 2; side++) {
     const mdj_table *t = sides[side];
     uint64_t *sur = (uint64_t *)ws.get((size_t)(t->nrows ? t->nrows : 1) * 8);

@@ -139,3 +139,43 @@ def test_outer_on_tuples_with_empty_or_unmatched_sides(how):
     assert _run_how([a, b], [a, b + 1], [0, 1], [0, 1], 4, how) == (2000 if how == "outer" else 1000)
     n = _run_how([a[:0], b[:0]], [a, b], [0, 1], [0, 1], 4, how)
     assert n == (0 if how == "left" else 1000)
+
+
+# -------------------------------------------- tuples whose bits are the key
+
+@pytest.mark.parametrize("kinds", [(np.int32, np.int32), (np.uint32, np.int32), (np.int64,), (np.uint32,)])
+@pytest.mark.parametrize("n_l,n_r", [(1, 3), (4095, 4097), (50_001, 70_003)])
+def test_tuples_of_at_most_64_bits(kinds, n_l, n_r):
+    # halves that must not mix (equal high or low words, sign bits), row
+    # counts around whole vectors, every join type
+    rng = np.random.default_rng(n_l)
+    top = max(2, int(n_l ** 0.5))
+
+    def column(kind, n):
+        v = rng.integers(0, top, n) * rng.choice([1, -1], n)
+        return v.astype(np.int64).astype(kind)
+
+    nk = len(kinds)
+    left = [rng.random(n_l)] + [column(k, n_l) for k in kinds] + [rng.random(n_l).astype(np.float32)]
+    right = [column(k, n_r) for k in kinds[::-1]] + [rng.random(n_r)]
+    lkeys, rkeys = list(range(1, nk + 1)), list(range(nk))[::-1]
+    _run_and_check(left, right, lkeys, rkeys, 8)
+    for how in ("left", "right", "outer"):
+        _run_how(left, right, lkeys, rkeys, 8, how)
+    _run_and_check([c[:0] for c in left], right, lkeys, rkeys, 1)
+
+
+def test_tuples_of_at_most_64_bits_in_unaligned_columns():
+    mdj = _mdj()
+    rng = np.random.default_rng(4)
+    cols = [rng.integers(0, 90, 5003).astype(np.int32) for _ in range(4)]
+    dev = [torch.from_numpy(c).to(DEV)[1:] for c in cols]
+    res = mdj.mdj_merge_multi(dev[:2], dev[2:], [0, 1], [0, 1], 1)
+    torch.cuda.synchronize()
+    want_l, want_r = oracle.merge_multi([c[1:] for c in cols[:2]], [c[1:] for c in cols[2:]], [0, 1], [0, 1])
+    lrow = res.left_row.cpu().numpy().view(np.uint32).astype(np.int64)
+    rrow = res.right_row.cpu().numpy().view(np.uint32).astype(np.int64)
+    order = np.lexsort((rrow, lrow))
+    assert np.array_equal(lrow[order], want_l) and np.array_equal(rrow[order], want_r)
+    for got, c in zip(res.left_cols, cols):
+        assert np.array_equal(got.cpu().numpy(), c[1:][lrow])
