@@ -25,6 +25,7 @@ constexpr uint32_t kMaxFanout = 1024;     // buckets of one stable scatter pass
 // 28.7K sub-buckets: 1.39 ms with 128, 1.41 with 160, 1.40 with 192; with
 // 14.4K sub-buckets (250M rows): 3.28 ms with 128, 3.42 with 192.
 constexpr uint32_t kMergeFanout = 128;
+constexpr uint32_t kMinBucketRows = 512;  // build rows a sub-bucket is planned for at least
 constexpr uint32_t kMaxSubBuckets = 49152;  // final buckets of a two-pass plan
 constexpr uint32_t kPass2SpanMax = 1024;  // local buckets of one pass-2 tile
 
@@ -318,6 +319,17 @@ Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition)
 // freshly allocated workspace buffers; fills `out` (offsets per final bucket).
 int partition_side(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan,
                    Side *out);
+
+// Both sides of a plan that needs one pass (or none), in shared launches, in
+// three steps so that the caller's kernel can turn the counts into offsets
+// and cursors between them: count_both adds every sub-bucket's rows to the
+// zeroed totL / totR; shuffle_both partitions both sides by the cursors and
+// fills L and R (an unpartitioned plan: the input tables themselves).
+bool plan_fits_one_launch(const Plan &plan);
+int count_both(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk, const Plan &plan,
+               uint32_t *totL, uint32_t *totR);
+int shuffle_both(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk,
+                 const Plan &plan, uint32_t *offL, uint32_t *offR, uint32_t *curL, uint32_t *curR, Side *L, Side *R);
 
 // Segmented partition of a batch: segment i = rows [seg_off[i], seg_off[i+1])
 // (host array) is split into seg_nb[i] = P_i * S_i buckets numbered from

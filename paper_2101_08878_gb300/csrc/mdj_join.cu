@@ -84,6 +84,68 @@ __global__ void k_expand(const uint32_t *__restrict__ offL, const uint32_t *__re
   }
 }
 
+// Everything between the counts and the shuffle of a plan of at most 1024
+// sub-buckets, in one block: offsets (scans of the counts), cursors, items
+// and their descriptors, and the join's counters cleared.  tot: rows per
+// sub-bucket, left then right; NULL: one bucket of nL and nR rows.  Eight
+// launches of the general path (two scans, two cursor kernels, items, their
+// scan, descriptors, and one count and one shuffle per side instead of both
+// in one) become one of about 6 us.
+constexpr int kPlanThreads = 1024;
+static_assert(kMaxFanout <= kPlanThreads, "one sub-bucket per thread");
+__global__ void __launch_bounds__(kPlanThreads)
+    k_merge_plan(const uint32_t *__restrict__ tot, uint32_t nL, uint32_t nR, uint32_t nb, uint32_t cap, uint32_t rch,
+                 uint32_t ulim, uint32_t *__restrict__ offL, uint32_t *__restrict__ offR, uint32_t *__restrict__ curL,
+                 uint32_t *__restrict__ curR, Item *__restrict__ desc, uint64_t *__restrict__ nitems,
+                 unsigned long long *__restrict__ tail) {
+  __shared__ uint32_t scratch[33], s_l[kPlanThreads + 1], s_r[kPlanThreads + 1], s_item[kPlanThreads + 1];
+  __shared__ uint64_t scratch64[33];
+  const uint32_t b = threadIdx.x;
+  const uint32_t cl = b < nb ? (tot ? tot[b] : nL) : 0u, cr = b < nb ? (tot ? tot[nb + b] : nR) : 0u;
+  uint32_t sum;
+  const uint32_t l = block_exclusive_scan<uint32_t>(cl, scratch, &sum);
+  const uint32_t r = block_exclusive_scan<uint32_t>(cr, scratch, &sum);
+  const uint64_t mine = cl && cr ? (uint64_t)((cl - 1) / cap + 1) * ((cr - 1) / rch + 1) : 0ull;
+  uint64_t total;
+  const uint64_t at = block_exclusive_scan<uint64_t>(mine, scratch64, &total);
+  if (b < nb) {
+    offL[b] = curL[b] = l;
+    offR[b] = curR[b] = r;
+    s_l[b] = l;
+    s_r[b] = r;
+    s_item[b] = (uint32_t)at;
+    if (b == nb - 1) {
+      offL[nb] = s_l[nb] = l + cl;
+      offR[nb] = s_r[nb] = r + cr;
+    }
+  }
+  if (b == 0) {
+    for (int w = 0; w < 5; w++) tail[w] = 0;
+    if (total > ulim) ((int *)(tail + 2))[FLAG_ITEMS] = 1;
+    *nitems = total;
+  }
+  __syncthreads();
+  if (total > ulim) return;
+  for (uint32_t it = b; it < (uint32_t)total; it += kPlanThreads) {
+    uint32_t lo = 0, hi = nb - 1;  // last bucket with s_item <= it
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) / 2;
+      if (s_item[mid] <= it)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const uint32_t nl = s_l[lo + 1] - s_l[lo], nr = s_r[lo + 1] - s_r[lo], nrc = (nr - 1) / rch + 1;
+    const uint32_t lc = (it - s_item[lo]) / nrc, rc = (it - s_item[lo]) % nrc;
+    Item d;
+    d.lbeg = s_l[lo] + lc * cap;
+    d.nl = min(cap, nl - lc * cap);
+    d.rbeg = s_r[lo] + rc * rch;
+    d.nr = min(rch, nr - rc * rch);
+    desc[it] = d;
+  }
+}
+
 // bulk: the build side's staged columns (key, row ids, first payload) have
 // 16-byte-aligned bases, so items stage them by bulk copies.  The item count
 // is read from *nitems_dev (no work when it exceeds `ulim`: k_expand has set
@@ -282,12 +344,37 @@ int read_tail(const unsigned long long *tail, cudaStream_t s, unsigned long long
   return MDJ_OK;
 }
 
+// A join's working arrays for at most `ulim` items, in one allocation:
+// state[ulim] | item_off[ulim] | total | ticket | flags (2 words) | item
+// count, and the descriptors.
+struct JoinArrays {
+  uint32_t ulim = 0;
+  unsigned long long *state = nullptr;
+  uint64_t *item_off = nullptr;
+  unsigned long long *total = nullptr;
+  Item *desc = nullptr;
+  const uint64_t *nitems = nullptr;  // device: the item count
+};
+int alloc_join_arrays(Workspace &ws, uint32_t ulim, JoinArrays *a) {
+  a->ulim = ulim;
+  a->state = (unsigned long long *)ws.get((2 * (size_t)ulim + 5) * 8);
+  if (!a->state) return MDJ_ERR_OOM;
+  a->item_off = (uint64_t *)(a->state + ulim);
+  a->total = a->state + 2 * (size_t)ulim;
+  return MDJ_OK;
+}
+
+// ready: arrays whose items and counters a kernel on the stream prepares
+// (k_merge_plan); NULL: prepared here.
 template <typename KeyT, int NT>
 int run_join_t(Workspace &ws, const Side &Ls, const Side &Rs, const Plan &plan, mdj_result *res,
-               bool force_ordered = false, ItemMap *map = nullptr, uint32_t exact_items = 0) {
+               bool force_ordered = false, ItemMap *map = nullptr, uint32_t exact_items = 0,
+               const JoinArrays *ready = nullptr) {
   cudaStream_t s = ws.stream();
   const uint32_t rch = (uint32_t)kWPF * NT;
-  const uint32_t ulim = exact_items ? exact_items : item_bound(plan.nbuckets, Ls.nrows, Rs.nrows, plan.cap, rch);
+  const uint32_t ulim = ready ? ready->ulim
+                        : exact_items ? exact_items
+                                      : item_bound(plan.nbuckets, Ls.nrows, Rs.nrows, plan.cap, rch);
   const int ordered = force_ordered || ordered_output() ? 1 : 0;
   // the optimistic output buffer (none for two-pass output); nothing below
   // waits for the device until the join has run
@@ -295,24 +382,27 @@ int run_join_t(Workspace &ws, const Side &Ls, const Side &Rs, const Plan &plan, 
   mdj_result r;
   JOut o;
   MDJ_TRY(alloc_result(ws, Ls, Rs, sizeof(KeyT), cap_rows, &r, &o));
-  // state[ulim] | item_off[ulim] | total | ticket | flags (2 words) | item count
-  const size_t words = 2 * (size_t)ulim + 5;
-  unsigned long long *state = (unsigned long long *)ws.get(words * 8);
-  int rc = state ? MDJ_OK : MDJ_ERR_OOM;
-  uint64_t *item_off = state ? (uint64_t *)(state + ulim) : nullptr;
-  unsigned long long *total = state ? state + 2 * (size_t)ulim : nullptr;
+  JoinArrays ja;
+  int rc = MDJ_OK;
+  if (ready)
+    ja = *ready;
+  else
+    rc = alloc_join_arrays(ws, ulim, &ja);
+  unsigned long long *state = ja.state, *total = ja.total;
+  uint64_t *item_off = ja.item_off;
   uint32_t *ticket = (uint32_t *)(total + 1);
   int *flags = (int *)(total + 2);
   // the look-back slots start empty (ordered); k_items clears the counters
   if (rc == MDJ_OK && ordered) rc = cuda_status(cudaMemsetAsync(state, 0, (size_t)ulim * 8, s));
-  Item *desc = nullptr;
+  Item *desc = ja.desc;
   uint64_t *bucket_items = nullptr;
-  if (rc == MDJ_OK) rc = make_items(ws, Ls, Rs, plan.nbuckets, plan.cap, rch, ulim, total, &desc, &bucket_items);
+  if (rc == MDJ_OK && !ready)
+    rc = make_items(ws, Ls, Rs, plan.nbuckets, plan.cap, rch, ulim, total, &desc, &bucket_items);
   if (rc != MDJ_OK) {
     mdj_result_release(&r, ws.allocator(), (void *)s);
     return rc;
   }
-  const uint64_t *nitems_dev = bucket_items + plan.nbuckets;
+  const uint64_t *nitems_dev = ready ? ready->nitems : bucket_items + plan.nbuckets;
 
   const size_t sm = WriteLayout<KeyT>(plan.cap).total;  // ~105 KB at cap 4096: two blocks per SM
   if (force_ordered) {
@@ -478,6 +568,39 @@ uint32_t cap_from_env() {
   return cap;
 }
 
+// The merge of a plan that needs one partition pass or none: both sides share
+// every launch.  Four launches (count, plan, shuffle, join) instead of
+// twelve; they are most of a small merge's time.
+int merge_one_pass(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk,
+                   const Plan &plan, mdj_result *out) {
+  cudaStream_t s = ws.stream();
+  const uint32_t nb = plan.nbuckets, rch = (uint32_t)kWPF * kWT;
+  // tot[2 nb] | offL[nb + 1] | offR[nb + 1] | curL[nb] | curR[nb]
+  uint32_t *w = (uint32_t *)ws.get((6 * (size_t)nb + 2) * 4);
+  uint64_t *nitems = (uint64_t *)ws.get(8);
+  JoinArrays ja;
+  MDJ_TRY(alloc_join_arrays(ws, item_bound(nb, left->nrows, right->nrows, plan.cap, rch), &ja));
+  ja.desc = (Item *)ws.get((size_t)ja.ulim * sizeof(Item));
+  ja.nitems = nitems;
+  if (!w || !nitems || !ja.desc) return MDJ_ERR_OOM;
+  uint32_t *offL = w + 2 * (size_t)nb, *offR = offL + nb + 1, *curL = offR + nb + 1, *curR = curL + nb;
+  if (plan.partition) {
+    MDJ_CUDA_TRY(cudaMemsetAsync(w, 0, 2 * (size_t)nb * 4, s));
+    MDJ_TRY(count_both(ws, left, lk, right, rk, plan, w, w + nb));
+  }
+  {
+    TraceScope tr("merge_plan", s);
+    k_merge_plan<<<1, kPlanThreads, 0, s>>>(plan.partition ? w : nullptr, (uint32_t)left->nrows,
+                                            (uint32_t)right->nrows, nb, plan.cap, rch, ja.ulim, offL, offR, curL, curR,
+                                            ja.desc, nitems, ja.total);
+  }
+  MDJ_LAUNCH_CHECK();
+  Side L, R;
+  MDJ_TRY(shuffle_both(ws, left, lk, right, rk, plan, offL, offR, curL, curR, &L, &R));
+  return left->cols[lk].dtype == MDJ_I64 ? run_join_t<int64_t, kWT>(ws, L, R, plan, out, false, nullptr, 0, &ja)
+                                         : run_join_t<int32_t, kWT>(ws, L, R, plan, out, false, nullptr, 0, &ja);
+}
+
 }  // namespace
 
 // The merge's steps; `after_left` (if set) runs once the left side's
@@ -496,6 +619,7 @@ int merge_steps(const mdj_table *left, int32_t lk, const mdj_table *right, int32
   // ordered output is deterministic only over stable partition passes
   plan.stable = ordered_output() != 0;
   const bool k64 = left->cols[lk].dtype == MDJ_I64;
+  if (!after_left && plan_fits_one_launch(plan) && !ordered_output()) return merge_one_pass(ws, left, lk, right, rk, plan, out);
   Side L, R;
   MDJ_TRY(partition_side(ws, left, lk, plan, &L));
   if (after_left) MDJ_TRY(after_left(ctx));

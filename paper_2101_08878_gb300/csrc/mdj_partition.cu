@@ -270,15 +270,27 @@ __device__ __forceinline__ void tot_load(const KeyT *__restrict__ keys, uint64_t
   }
 }
 
-// tot[sb] += rows of sub-bucket sb (spec bs, nsub = P * S).
+// One side of a count: `blocks` blocks add its rows per sub-bucket to tot.
+struct TotSide {
+  const void *keys;
+  uint32_t *tot;
+  uint32_t n, blocks;
+};
+
+// tot[sb] += rows of sub-bucket sb (spec bs, nsub = P * S), for one side or
+// for both in one launch (the first A.blocks blocks take side A).
 template <typename KeyT>
-__global__ void __launch_bounds__(kTotThreads) k_tot(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
-                                                     uint32_t nsub, uint32_t *__restrict__ tot) {
+__global__ void __launch_bounds__(kTotThreads) k_tot(const TotSide A, const TotSide B, BucketSpec bs, uint32_t nsub) {
   extern __shared__ uint32_t cnt[];
+  const bool first = blockIdx.x < A.blocks;
+  const KeyT *__restrict__ keys = (const KeyT *)(first ? A.keys : B.keys);
+  uint32_t *__restrict__ tot = first ? A.tot : B.tot;
+  const uint32_t n = first ? A.n : B.n, nblk = first ? A.blocks : B.blocks;
+  const uint32_t blk = first ? blockIdx.x : blockIdx.x - A.blocks;
   for (uint32_t i = threadIdx.x; i < nsub; i += kTotThreads) cnt[i] = 0;
   __syncthreads();
-  const uint64_t chunk = (uint64_t)kTotThreads * kTotU, stride = chunk * gridDim.x;
-  uint64_t base = chunk * blockIdx.x;
+  const uint64_t chunk = (uint64_t)kTotThreads * kTotU, stride = chunk * nblk;
+  uint64_t base = chunk * blk;
   KeyT cur[kTotU], nxt[kTotU];
   tot_load<KeyT>(keys, base, n, cur);
   for (; base < n; base += stride) {
@@ -313,7 +325,25 @@ struct SegArgs {
   const uint32_t *base, *nb, *P, *S;
 };
 
-// Persistent: block b takes tiles b, b + gridDim.x, ...  Per tile:
+// One table side of a shuffle pass: `ntiles` tiles of its n rows, run
+// destinations reserved on `cursors`, row ids to rid_out (read from rid_in in
+// pass 2, else the row's index).  `reg_col`: the first non-key column (-1:
+// none).
+struct ShSide {
+  const void *keys;
+  const uint32_t *rid_in;
+  uint32_t *rid_out;
+  uint32_t *cursors;
+  ColMove cm;
+  int32_t reg_col;
+  uint32_t n, ntiles;
+};
+struct ShSides {
+  ShSide s[2];
+};
+
+// Persistent: block b takes tiles b, b + gridDim.x, ... (side 0's tiles
+// first; only pass 1 has a side 1).  Per tile:
 //   1. load: keys, then payload and row ids, by asynchronous copies;
 //   2. rank: a row's rank in its bucket is a shared-memory atomicAdd;
 //   3. counts: local starts by a block scan; each (tile, bucket) run's
@@ -321,17 +351,14 @@ struct SegArgs {
 //      needed only at write-out;
 //   4. perm: each row's number goes to its bucket-ordered position;
 //   5. write-out: the columns are gathered through perm and leave as runs.
-// `reg_col`: the first non-key column (-1: none).  EXTRA: further columns,
-// one at a time through the payload's place.
+// `pay_width`: bytes of a row's place in the payload area.  EXTRA: further
+// columns, one at a time through that area.
 template <typename KeyT, int MODE, bool EXTRA>
 __global__ void __launch_bounds__(kShNT, kShBlocks)
-    k_shuffle(const KeyT *__restrict__ keys, uint32_t n, uint32_t tile, uint32_t ntiles, const __grid_constant__ BucketSpec bs,
-              uint32_t F, uint32_t F2, uint32_t span, uint32_t *__restrict__ cursors,
-              const __grid_constant__ ColMove cm, int reg_col, const uint32_t *__restrict__ rid_in,
-              uint32_t *__restrict__ rid_out, const SegArgs sg) {
+    k_shuffle(const __grid_constant__ ShSides sides, uint32_t tile, uint32_t ntiles, uint32_t pay_width,
+              const __grid_constant__ BucketSpec bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs sg) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int pw = reg_col >= 0 ? cm.width[reg_col] : 0;
-  const ShLayout lay(tile, sizeof(KeyT), EXTRA ? 8 : pw, MODE == SH_PASS2, span);
+  const ShLayout lay(tile, sizeof(KeyT), pay_width, MODE == SH_PASS2, span);
   KeyT *skey = (KeyT *)smem;
   unsigned char *spay = smem + lay.pay;
   uint32_t *srid = (uint32_t *)(smem + lay.rid);
@@ -341,20 +368,26 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
   uint32_t *gdelta = lst + span;
   uint32_t *wsum = gdelta + span;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  KeyT *kdst = (KeyT *)cm.dst[cm.key_index];
   for (uint32_t i = threadIdx.x; i < span; i += kShNT) cnt[i] = 0;
   __syncthreads();
 
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const uint32_t second = MODE == SH_PASS1 && t >= sides.s[0].ntiles ? 1u : 0u;
+    const ShSide &sd = sides.s[second];
+    const ColMove &cm = sd.cm;
+    const int reg_col = sd.reg_col;
+    const int pw = reg_col >= 0 ? cm.width[reg_col] : 0;
+    const KeyT *__restrict__ keys = (const KeyT *)sd.keys;
+    uint32_t *__restrict__ cursors = sd.cursors;
     SegTile td = {0, 0, 0};
     if (MODE == SH_SEG) td = sg.tiles[t];
-    const uint32_t row0 = MODE == SH_SEG ? td.row0 : t * tile;
-    const uint32_t rows = MODE == SH_SEG ? td.rows : min(tile, n - row0);
+    const uint32_t row0 = MODE == SH_SEG ? td.row0 : (second ? t - sides.s[0].ntiles : t) * tile;
+    const uint32_t rows = MODE == SH_SEG ? td.rows : min(tile, sd.n - row0);
     // 1. load
     load_key_pairs<KeyT>(skey, keys + row0, rows);
     cp_async_commit();
     if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
-    if (MODE == SH_PASS2) load_column<4>((unsigned char *)srid, (const unsigned char *)(rid_in + row0), rows);
+    if (MODE == SH_PASS2) load_column<4>((unsigned char *)srid, (const unsigned char *)(sd.rid_in + row0), rows);
     cp_async_commit();
     uint32_t lb0 = 0, Floc = F;
     BucketSpec sp;
@@ -372,7 +405,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
       if (Floc > span) {  // uniform over the block
         cp_async_wait<0>();
         __syncthreads();
-        shuffle_direct<KeyT>(skey, srid, row0, rows, bs, cursors, cm, rid_out);
+        shuffle_direct<KeyT>(skey, srid, row0, rows, bs, cursors, cm, sd.rid_out);
         __syncthreads();
         continue;
       }
@@ -383,8 +416,9 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 #pragma unroll
     for (int k = 0; k < kShPairs; k++) {
       const uint32_t r = 2 * (threadIdx.x + k * kShNT);
-      KeyT kv[2];
-      if (sizeof(KeyT) == 8) {
+      KeyT kv[2] = {KeyT(0), KeyT(0)};
+      if (r >= rows) {  // past the tile: nothing there to read
+      } else if (sizeof(KeyT) == 8) {
         const longlong2 v = *(const longlong2 *)(skey + r);
         kv[0] = (KeyT)v.x, kv[1] = (KeyT)v.y;
       } else {
@@ -449,13 +483,16 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     cp_async_wait<0>();
     __syncthreads();
     // 5. write-out
+    KeyT *__restrict__ kdst = (KeyT *)cm.dst[cm.key_index];
+    void *pdst = pw ? cm.dst[reg_col] : nullptr;
+    uint32_t *__restrict__ rid_out = sd.rid_out;
 #pragma unroll 4
     for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
       const uint32_t m = perm[p], i = m & 0xFFFFu;
       const uint32_t d = p + gdelta[m >> 16];
       kdst[d] = skey[i];
-      if (pw == 8) ((uint64_t *)cm.dst[reg_col])[d] = ((const uint64_t *)spay)[i];
-      if (pw == 4) ((uint32_t *)cm.dst[reg_col])[d] = ((const uint32_t *)spay)[i];
+      if (pw == 8) ((uint64_t *)pdst)[d] = ((const uint64_t *)spay)[i];
+      if (pw == 4) ((uint32_t *)pdst)[d] = ((const uint32_t *)spay)[i];
       rid_out[d] = MODE == SH_PASS2 ? srid[i] : row0 + i;
     }
     __syncthreads();
@@ -669,29 +706,75 @@ uint32_t shuffle_pay_width(const mdj_table *t, int32_t key_col) {
   return t->ncols < 2 ? 0u : (uint32_t)dtype_width(t->cols[1 - key_col].dtype);
 }
 
-// One unstable shuffle pass (see k_shuffle) of n rows in tiles of `tile`
-// rows, with run cursors `cur` (pass 1: one per pass-1 bucket; pass 2 and
-// segments: one per sub-bucket).
+// One side of a pass; ntiles is set by shuffle_pass.
+ShSide shuffle_side(const mdj_table *t, int32_t key_col, const void *const *src, void *const *dst,
+                    const uint32_t *rid_in, uint32_t *rid_out, uint32_t *cursors) {
+  ShSide sd;
+  memset(&sd, 0, sizeof sd);
+  sd.cm = make_move(t, key_col, src, dst);
+  sd.keys = src[key_col];
+  sd.rid_in = rid_in;
+  sd.rid_out = rid_out;
+  sd.cursors = cursors;
+  sd.reg_col = t->ncols < 2 ? -1 : (key_col == 0 ? 1 : 0);
+  sd.n = (uint32_t)t->nrows;
+  return sd;
+}
+
+// One unstable shuffle pass (see k_shuffle) in tiles of `tile` rows; cursors:
+// pass 1 one per pass-1 bucket, pass 2 and segments one per sub-bucket.  With
+// segments the tiles are sg's (ntiles of them), else the sides' (both may
+// have rows in pass 1 only).
 template <typename KeyT>
-int shuffle_pass(Workspace &ws, int mode, const KeyT *keys, uint32_t n, uint32_t tile, uint32_t ntiles,
-                 const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, uint32_t *cur, const ColMove &cm,
-                 const uint32_t *rid_in, uint32_t *rid_out, const SegArgs &sg) {
+int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_t pay_width, uint32_t ntiles,
+                 const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs &sg) {
+  bool extra = false;
+  for (ShSide &sd : sides.s) {
+    sd.ntiles = (uint32_t)(((uint64_t)sd.n + tile - 1) / tile);
+    if (mode != SH_SEG) ntiles += sd.ntiles;
+    extra = extra || sd.cm.n > 2;
+  }
   if (ntiles == 0) return MDJ_OK;
-  int reg_col = -1;
-  for (int j = 0; j < cm.n && reg_col < 0; j++)
-    if (j != cm.key_index) reg_col = j;
-  const bool extra = cm.n > 2;
-  const uint32_t pw = extra ? 8u : (reg_col >= 0 ? (uint32_t)cm.width[reg_col] : 0u);
-  const uint32_t sm = ShLayout(tile, sizeof(KeyT), pw, mode == SH_PASS2, span).total;
+  const uint32_t sm = ShLayout(tile, sizeof(KeyT), pay_width, mode == SH_PASS2, span).total;
   const uint32_t most = (uint32_t)num_sms() * kShBlocks;
   TraceScope tr(mode == SH_SEG ? "seg_scatter" : (mode == SH_PASS2 ? "shuffle_pass2" : "shuffle_pass1"), ws.stream());
-  shuffle_kernel<KeyT>(mode, extra)<<<std::min(ntiles, most), kShNT, sm, ws.stream()>>>(
-      keys, n, tile, ntiles, bs, F, F2, span, cur, cm, reg_col, rid_in, rid_out, sg);
+  shuffle_kernel<KeyT>(mode, extra)<<<std::min(ntiles, most), kShNT, sm, ws.stream()>>>(sides, tile, ntiles, pay_width,
+                                                                                        bs, F, F2, span, sg);
   MDJ_LAUNCH_CHECK();
   return MDJ_OK;
 }
 
-uint32_t tiles_of(uint32_t n, uint32_t tile) { return (uint32_t)(((uint64_t)n + tile - 1) / tile); }
+// Tile rows of a pass over n rows: the largest tile, or, where that leaves the
+// last wave of blocks part empty, the same number of waves of equal tiles
+// (1024 rows at least: a tile has fixed costs of its own).
+uint32_t balanced_tile(uint64_t n, uint32_t largest) {
+  const uint64_t slots = (uint64_t)num_sms() * kShBlocks;
+  const uint64_t waves = std::max<uint64_t>(1, (n + slots * largest - 1) / (slots * largest));
+  const uint64_t even = ((n + slots * waves - 1) / (slots * waves) + 15) / 16 * 16;
+  return (uint32_t)std::min<uint64_t>(largest, std::max<uint64_t>(even, 1024));
+}
+
+// Rows per sub-bucket of one or both sides (n = 0: none) added to their tot.
+template <typename KeyT>
+int count_rows(Workspace &ws, TotSide A, TotSide B, const BucketSpec &bs, uint32_t nsub) {
+  const size_t smem = (size_t)nsub * 4;
+  int per_sm = 0;
+  MDJ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tot<KeyT>, kTotThreads, smem));
+  const uint64_t full = (uint64_t)num_sms() * std::max(per_sm, 1);
+  const uint64_t chunk = (uint64_t)kTotThreads * kTotU;
+  const uint64_t ca = (A.n + chunk - 1) / chunk, cb = (B.n + chunk - 1) / chunk;
+  if (ca + cb == 0) return MDJ_OK;
+  A.blocks = (uint32_t)ca;
+  B.blocks = (uint32_t)cb;
+  if (ca + cb > full) {  // resident blocks, split by rows
+    A.blocks = cb ? (uint32_t)std::min(full - 1, std::max<uint64_t>(ca ? 1 : 0, full * ca / (ca + cb))) : (uint32_t)full;
+    B.blocks = (uint32_t)full - A.blocks;
+  }
+  TraceScope tr("hist", ws.stream());
+  k_tot<KeyT><<<A.blocks + B.blocks, kTotThreads, smem, ws.stream()>>>(A, B, bs, nsub);
+  MDJ_LAUNCH_CHECK();
+  return MDJ_OK;
+}
 
 // The merge's partition of one side with the unstable passes, first half:
 // count the final sub-buckets, scan them into `off`, then the only pass
@@ -717,18 +800,7 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   uint32_t *cur = (uint32_t *)ws.get((size_t)(nsub + 1) * 4);
   if (!cur) return MDJ_ERR_OOM;
   if (cur2 && !(*cur2 = (uint32_t *)ws.get((size_t)(nsub + 1) * 4))) return MDJ_ERR_OOM;
-  {
-    const size_t smem = (size_t)nsub * 4;
-    int per_sm = 0;
-    MDJ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tot<KeyT>, kTotThreads, smem));
-    if (per_sm < 1) per_sm = 1;
-    const uint64_t chunks = ((uint64_t)n + (uint64_t)kTotThreads * kTotU - 1) / ((uint64_t)kTotThreads * kTotU);
-    const uint64_t full = (uint64_t)num_sms() * per_sm;
-    const unsigned grid = (unsigned)(chunks < full ? chunks : full);
-    TraceScope tr("hist", s);
-    k_tot<KeyT><<<grid, kTotThreads, smem, s>>>(keys, n, sub, nsub, off);
-  }
-  MDJ_LAUNCH_CHECK();
+  MDJ_TRY(count_rows<KeyT>(ws, TotSide{keys, off, n, 0}, TotSide{nullptr, nullptr, 0, 0}, sub, nsub));
   MDJ_TRY(exclusive_scan_u32(ws, off, off, (size_t)nsub + 1));
   {
     // pass-1 cursors: the first row of every pass-1 bucket
@@ -737,11 +809,13 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
     k_pass1_cursors<<<(nk + 255) / 256, 256, 0, s>>>(off, F1, plan.F2, cur, cur2 ? *cur2 : nullptr, nsub);
   }
   MDJ_LAUNCH_CHECK();
-  ColMove cm = make_move(t, key_col, src, out->cols);
   const BucketSpec spec1 = plan.F2 == 1 ? sub : make_spec(plan.P, plan.S, plan.F2);
-  const uint32_t tile = shuffle_tile_rows(sizeof(KeyT), shuffle_pay_width(t, key_col), false, F1);
-  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS1, keys, n, tile, tiles_of(n, tile), spec1, F1, plan.F2, F1, cur, cm, nullptr,
-                             out->rid, SegArgs{}));
+  const uint32_t pw = shuffle_pay_width(t, key_col);
+  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, false, F1));
+  ShSides sides;
+  memset(&sides, 0, sizeof sides);
+  sides.s[0] = shuffle_side(t, key_col, src, out->cols, nullptr, out->rid, cur);
+  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}));
   ws.give_back(cur);
   return MDJ_OK;
 }
@@ -754,14 +828,17 @@ int shuffle_pass2_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Pl
   const uint32_t n = (uint32_t)t->nrows;
   MDJ_TRY(alloc_table_bufs(ws, t, fin, true));
   if (n == 0) return MDJ_OK;
-  ColMove cm2 = make_move(t, key_col, p1.cols, fin->cols);
   // local buckets of a tile: the pass-1 buckets it is expected to touch (two
   // at least); a tile that touches more (a run of small ones) goes direct
   const uint64_t touched = 2 + (uint64_t)kShMaxTile * plan.F1 / n;
   const uint32_t span = (uint32_t)std::min<uint64_t>(touched * plan.F2, kPass2SpanMax);
-  const uint32_t tile = shuffle_tile_rows(sizeof(KeyT), shuffle_pay_width(t, key_col), true, span);
-  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS2, (const KeyT *)p1.cols[key_col], n, tile, tiles_of(n, tile),
-                             make_spec(plan.P, plan.S, 1), 0, plan.F2, span, cur, cm2, p1.rid, fin->rid, SegArgs{}));
+  const uint32_t pw = shuffle_pay_width(t, key_col);
+  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, true, span));
+  ShSides sides;
+  memset(&sides, 0, sizeof sides);
+  sides.s[0] = shuffle_side(t, key_col, p1.cols, fin->cols, p1.rid, fin->rid, cur);
+  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS2, sides, tile, pw, 0, make_spec(plan.P, plan.S, 1), 0, plan.F2, span,
+                             SegArgs{}));
   ws.give_back(cur);
   return MDJ_OK;
 }
@@ -776,6 +853,24 @@ int shuffle_side_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Pla
   MDJ_TRY(shuffle_pass2_t<KeyT>(ws, t, key_col, plan, cur2, p1, fin));
   release_table_bufs(ws, t, &p1);
   return MDJ_OK;
+}
+
+// Both sides of a single-pass plan: the shuffle in one launch.
+template <typename KeyT>
+int shuffle_both_t(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk,
+                   const Plan &plan, uint32_t *curL, uint32_t *curR, TableBufs *fl, TableBufs *fr) {
+  MDJ_TRY(set_shuffle_attrs<KeyT>());
+  MDJ_TRY(alloc_table_bufs(ws, left, fl, true));
+  MDJ_TRY(alloc_table_bufs(ws, right, fr, true));
+  const void *src[2][MDJ_MAX_COLS];
+  for (int j = 0; j < left->ncols; j++) src[0][j] = left->cols[j].data;
+  for (int j = 0; j < right->ncols; j++) src[1][j] = right->cols[j].data;
+  const uint32_t F = plan.nbuckets, pw = std::max(shuffle_pay_width(left, lk), shuffle_pay_width(right, rk));
+  const uint32_t tile = balanced_tile(left->nrows + right->nrows, shuffle_tile_rows(sizeof(KeyT), pw, false, F));
+  ShSides sides;
+  sides.s[0] = shuffle_side(left, lk, src[0], fl->cols, nullptr, fl->rid, curL);
+  sides.s[1] = shuffle_side(right, rk, src[1], fr->cols, nullptr, fr->rid, curR);
+  return shuffle_pass<KeyT>(ws, SH_PASS1, sides, tile, pw, 0, make_spec(plan.P, plan.S, 1), F, 1, F, SegArgs{});
 }
 
 // Stable partition by p with P > kMaxFanout: two stable LSD digit passes
@@ -928,7 +1023,12 @@ Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition)
   pl.cap = cap;
   // target mean build rows per sub-bucket: ~85% of a table, so that hash
   // variance rarely overflows one table
-  const uint64_t target = (uint64_t)cap * 85 / 100;
+  uint64_t target = (uint64_t)cap * 85 / 100;
+  // small build sides: enough sub-buckets for every resident join block (two
+  // per SM), of at least kMinBucketRows rows; a side that fits one table
+  // still stays whole
+  if (n_build > target)
+    target = std::min(target, std::max<uint64_t>(kMinBucketRows, n_build / (2 * (uint64_t)num_sms()) + 1));
   uint64_t need = (n_build + target - 1) / target;
   if (need < 1) need = 1;
   if (P > kMaxFanout) {
@@ -991,6 +1091,36 @@ void fill_side(const mdj_table *t, int32_t key_col, const TableBufs &b, uint32_t
   out->nrows = t->nrows;
 }
 }  // namespace
+
+bool plan_fits_one_launch(const Plan &plan) {
+  return !plan.partition || (!plan.lsd && !plan.stable && plan.F2 == 1 && fast_shuffle_enabled());
+}
+
+int count_both(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk, const Plan &plan,
+               uint32_t *totL, uint32_t *totR) {
+  const TotSide A = {left->cols[lk].data, totL, (uint32_t)left->nrows, 0};
+  const TotSide B = {right->cols[rk].data, totR, (uint32_t)right->nrows, 0};
+  const BucketSpec bs = make_spec(plan.P, plan.S, 1);
+  return left->cols[lk].dtype == MDJ_I64 ? count_rows<int64_t>(ws, A, B, bs, plan.nbuckets)
+                                         : count_rows<int32_t>(ws, A, B, bs, plan.nbuckets);
+}
+
+int shuffle_both(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk,
+                 const Plan &plan, uint32_t *offL, uint32_t *offR, uint32_t *curL, uint32_t *curR, Side *L, Side *R) {
+  TableBufs fl, fr;
+  if (plan.partition) {
+    MDJ_TRY(left->cols[lk].dtype == MDJ_I64
+                ? shuffle_both_t<int64_t>(ws, left, lk, right, rk, plan, curL, curR, &fl, &fr)
+                : shuffle_both_t<int32_t>(ws, left, lk, right, rk, plan, curL, curR, &fl, &fr));
+  } else {
+    for (int j = 0; j < left->ncols; j++) fl.cols[j] = (void *)left->cols[j].data;
+    for (int j = 0; j < right->ncols; j++) fr.cols[j] = (void *)right->cols[j].data;
+    fl.rid = fr.rid = nullptr;
+  }
+  fill_side(left, lk, fl, offL, L);
+  fill_side(right, rk, fr, offR, R);
+  return MDJ_OK;
+}
 
 int stable_partition(Workspace &ws, const mdj_table *t, int32_t key_col, uint32_t P, void *const *out_cols,
                      uint32_t *out_rid, int64_t *out_offsets) {
@@ -1171,9 +1301,11 @@ int seg_partition_t(Workspace &ws, const mdj_table *t, int32_t key_col, const ui
     MDJ_TRY(exclusive_scan_u32(ws, off, off, nb + 1));
     MDJ_CUDA_TRY(cudaMemcpyAsync(cur, off, (size_t)nb * 4, cudaMemcpyDeviceToDevice, s));
     MDJ_TRY(alloc_table_bufs(ws, t, &fin, true));
-    ColMove cm = make_move(t, key_col, src, fin.cols);
-    MDJ_TRY(shuffle_pass<KeyT>(ws, SH_SEG, (const KeyT *)key, n, tile, ntiles, make_spec(1, 1, 1), 0, 1, smax, cur, cm,
-                               nullptr, fin.rid, sg));
+    ShSides sides;
+    memset(&sides, 0, sizeof sides);
+    sides.s[0] = shuffle_side(t, key_col, src, fin.cols, nullptr, fin.rid, cur);
+    MDJ_TRY(shuffle_pass<KeyT>(ws, SH_SEG, sides, tile, shuffle_pay_width(t, key_col), ntiles, make_spec(1, 1, 1), 0, 1,
+                               smax, sg));
     key = fin.cols[key_col];
     cols = fin.cols;
     rid = fin.rid;
