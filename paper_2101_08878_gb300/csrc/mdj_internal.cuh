@@ -320,6 +320,11 @@ Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition)
 int partition_side(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan,
                    Side *out);
 
+// Partition one side for the count mode: `out` has the key and one 8-byte
+// column, each row's checksum term (f on the left, g on the right); its row
+// ids mean nothing.
+int partition_terms(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan, bool left, Side *out);
+
 // Both sides of a plan that needs one pass (or none), in shared launches, in
 // three steps so that the caller's kernel can turn the counts into offsets
 // and cursors between them: count_both adds every sub-bucket's rows to the
@@ -357,11 +362,11 @@ int stable_partition_scratch(const mdj_table *t, int32_t key_col, uint32_t P, vo
 int merge_steps(const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk, uint32_t P,
                 const mdj_allocator *alloc, void *stream, mdj_result *out, int (*after_left)(void *), void *ctx);
 
-// mdj_count_checksum: the pair count and checksum of the inner join, from
-// the streamed output's grouping (every key group of the build side gathered
-// once, each probe row told its group): count = sum of the probe rows' group
-// sizes, checksum = sum over probe rows r of g(r) times the sum of f over r's
-// group (a prefix sum over the grouped build rows).
+// mdj_count_checksum: the pair count and checksum of the inner join.  Equal
+// keys factor: count = sum over probe rows of their key's build rows,
+// checksum = sum over probe rows r of g(r) times the sum of f over the build
+// rows of r's key, so a table of (rows, sum of f) per distinct build key is
+// all a probe row needs (csrc/mdj_stream.cu).
 int grouped_count_checksum(const mdj_table *left, int32_t lk, const mdj_table *right, int32_t rk, uint32_t P,
                            const mdj_allocator *alloc, void *stream, uint64_t *count, uint64_t *checksum);
 

@@ -327,7 +327,7 @@ struct SegArgs {
 
 // One table side of a shuffle pass: `ntiles` tiles of its n rows, run
 // destinations reserved on `cursors`, row ids to rid_out (read from rid_in in
-// pass 2, else the row's index).  `reg_col`: the first non-key column (-1:
+// pass 2, where both may be NULL, else the row's index).  `reg_col`: the first non-key column (-1:
 // none).
 struct ShSide {
   const void *keys;
@@ -336,6 +336,8 @@ struct ShSide {
   uint32_t *cursors;
   ColMove cm;
   int32_t reg_col;
+  int32_t term;         // SH_TERM: TERM_F or TERM_G, to term_dst
+  uint64_t *term_dst;
   uint32_t n, ntiles;
 };
 struct ShSides {
@@ -358,7 +360,8 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     k_shuffle(const __grid_constant__ ShSides sides, uint32_t tile, uint32_t ntiles, uint32_t pay_width,
               const __grid_constant__ BucketSpec bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs sg) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const ShLayout lay(tile, sizeof(KeyT), pay_width, MODE == SH_PASS2, span);
+  const bool with_rid = MODE == SH_PASS2 && sides.s[0].rid_in != nullptr;
+  const ShLayout lay(tile, sizeof(KeyT), pay_width, with_rid, span);
   KeyT *skey = (KeyT *)smem;
   unsigned char *spay = smem + lay.pay;
   uint32_t *srid = (uint32_t *)(smem + lay.rid);
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     load_key_pairs<KeyT>(skey, keys + row0, rows);
     cp_async_commit();
     if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
-    if (MODE == SH_PASS2) load_column<4>((unsigned char *)srid, (const unsigned char *)(sd.rid_in + row0), rows);
+    if (with_rid) load_column<4>((unsigned char *)srid, (const unsigned char *)(sd.rid_in + row0), rows);
     cp_async_commit();
     uint32_t lb0 = 0, Floc = F;
     BucketSpec sp;
@@ -430,9 +433,9 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
         pk[2 * k + e] = 0xFFFFFFFFu;
         if (r + e < rows) {
           const uint64_t h = fmix64(key_bits(kv[e]));
-          const uint32_t lb = MODE == SH_PASS1   ? bucket_of(h, bs)
-                              : MODE == SH_PASS2 ? sub_bucket_of(h, bs) - lb0
-                                                 : sub_bucket_of(h, sp);
+          const uint32_t lb = MODE == SH_PASS1 || MODE == SH_TERM ? bucket_of(h, bs)
+                              : MODE == SH_PASS2               ? sub_bucket_of(h, bs) - lb0
+                                                               : sub_bucket_of(h, sp);
           pk[2 * k + e] = (lb << 16) | atomicAdd(&cnt[lb], 1u);
         }
       }
@@ -491,9 +494,17 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
       const uint32_t m = perm[p], i = m & 0xFFFFu;
       const uint32_t d = p + gdelta[m >> 16];
       kdst[d] = skey[i];
+      if (MODE == SH_TERM) {
+        const uint64_t pb = pay_bits(pw ? spay : nullptr, pw, i);
+        sd.term_dst[d] = sd.term == TERM_F ? term_f(key_bits(skey[i]), row0 + i, pb) : term_g(row0 + i, pb);
+        continue;
+      }
       if (pw == 8) ((uint64_t *)pdst)[d] = ((const uint64_t *)spay)[i];
       if (pw == 4) ((uint32_t *)pdst)[d] = ((const uint32_t *)spay)[i];
-      rid_out[d] = MODE == SH_PASS2 ? srid[i] : row0 + i;
+      if (MODE != SH_PASS2)
+        rid_out[d] = row0 + i;
+      else if (with_rid)
+        rid_out[d] = srid[i];
     }
     __syncthreads();
     if (EXTRA) {
@@ -682,6 +693,7 @@ template <typename KeyT>
 auto shuffle_kernel(int mode, bool extra) {
   if (mode == SH_PASS2) return extra ? k_shuffle<KeyT, SH_PASS2, true> : k_shuffle<KeyT, SH_PASS2, false>;
   if (mode == SH_SEG) return extra ? k_shuffle<KeyT, SH_SEG, true> : k_shuffle<KeyT, SH_SEG, false>;
+  if (mode == SH_TERM) return k_shuffle<KeyT, SH_TERM, false>;
   return extra ? k_shuffle<KeyT, SH_PASS1, true> : k_shuffle<KeyT, SH_PASS1, false>;
 }
 
@@ -691,7 +703,7 @@ int set_shuffle_attrs() {
   return once_per_device(once, [] {
     const int sm = (int)kShSmem;
     for (int extra = 0; extra < 2; extra++)
-      for (int mode = 0; mode < 3; mode++)
+      for (int mode = 0; mode < 4; mode++)
         MDJ_CUDA_TRY(cudaFuncSetAttribute(shuffle_kernel<KeyT>(mode, extra != 0),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_tot<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -732,10 +744,11 @@ int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_
   for (ShSide &sd : sides.s) {
     sd.ntiles = (uint32_t)(((uint64_t)sd.n + tile - 1) / tile);
     if (mode != SH_SEG) ntiles += sd.ntiles;
-    extra = extra || sd.cm.n > 2;
+    extra = extra || (mode != SH_TERM && sd.cm.n > 2);
   }
   if (ntiles == 0) return MDJ_OK;
-  const uint32_t sm = ShLayout(tile, sizeof(KeyT), pay_width, mode == SH_PASS2, span).total;
+  const bool with_rid = mode == SH_PASS2 && sides.s[0].rid_in;
+  const uint32_t sm = ShLayout(tile, sizeof(KeyT), pay_width, with_rid, span).total;
   const uint32_t most = (uint32_t)num_sms() * kShBlocks;
   TraceScope tr(mode == SH_SEG ? "seg_scatter" : (mode == SH_PASS2 ? "shuffle_pass2" : "shuffle_pass1"), ws.stream());
   shuffle_kernel<KeyT>(mode, extra)<<<std::min(ntiles, most), kShNT, sm, ws.stream()>>>(sides, tile, ntiles, pay_width,
@@ -783,7 +796,7 @@ int count_rows(Workspace &ws, TotSide A, TotSide B, const BucketSpec &bs, uint32
 // the offsets by the same kernel as pass 1's.
 template <typename KeyT>
 int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan, uint32_t *off,
-                          TableBufs *out, uint32_t **cur2 = nullptr) {
+                          TableBufs *out, uint32_t **cur2 = nullptr, int term = 0) {
   cudaStream_t s = ws.stream();
   MDJ_TRY(set_shuffle_attrs<KeyT>());
   const uint32_t n = (uint32_t)t->nrows;
@@ -795,7 +808,10 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   const BucketSpec sub = make_spec(plan.P, plan.S, 1);
 
   MDJ_CUDA_TRY(cudaMemsetAsync(off, 0, (size_t)(nsub + 1) * 4, s));
-  MDJ_TRY(alloc_table_bufs(ws, t, out, true));
+  // with a term the rows leave as two columns, the key and the term
+  const mdj_col term_cols[2] = {{nullptr, t->cols[key_col].dtype}, {nullptr, MDJ_U64}};
+  const mdj_table term_table = {(mdj_col *)term_cols, 2, t->nrows};
+  MDJ_TRY(alloc_table_bufs(ws, term ? &term_table : t, out, !term));
   if (n == 0) return MDJ_OK;
   uint32_t *cur = (uint32_t *)ws.get((size_t)(nsub + 1) * 4);
   if (!cur) return MDJ_ERR_OOM;
@@ -810,12 +826,21 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   }
   MDJ_LAUNCH_CHECK();
   const BucketSpec spec1 = plan.F2 == 1 ? sub : make_spec(plan.P, plan.S, plan.F2);
-  const uint32_t pw = shuffle_pay_width(t, key_col);
+  const int32_t pay_col = t->ncols < 2 ? -1 : (key_col == 0 ? 1 : 0);
+  const uint32_t pw = !term ? shuffle_pay_width(t, key_col) : pay_col < 0 ? 0u : dtype_width(t->cols[pay_col].dtype);
   const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, false, F1));
   ShSides sides;
   memset(&sides, 0, sizeof sides);
-  sides.s[0] = shuffle_side(t, key_col, src, out->cols, nullptr, out->rid, cur);
-  MDJ_TRY(shuffle_pass<KeyT>(ws, SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}));
+  if (term) {
+    void *dst[MDJ_MAX_COLS] = {};
+    dst[key_col] = out->cols[0];
+    sides.s[0] = shuffle_side(t, key_col, src, dst, nullptr, nullptr, cur);
+    sides.s[0].term = term;
+    sides.s[0].term_dst = (uint64_t *)out->cols[1];
+  } else {
+    sides.s[0] = shuffle_side(t, key_col, src, out->cols, nullptr, out->rid, cur);
+  }
+  MDJ_TRY(shuffle_pass<KeyT>(ws, term ? SH_TERM : SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}));
   ws.give_back(cur);
   return MDJ_OK;
 }
@@ -826,14 +851,14 @@ template <typename KeyT>
 int shuffle_pass2_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan, uint32_t *cur,
                     const TableBufs &p1, TableBufs *fin) {
   const uint32_t n = (uint32_t)t->nrows;
-  MDJ_TRY(alloc_table_bufs(ws, t, fin, true));
+  MDJ_TRY(alloc_table_bufs(ws, t, fin, p1.rid != nullptr));
   if (n == 0) return MDJ_OK;
   // local buckets of a tile: the pass-1 buckets it is expected to touch (two
   // at least); a tile that touches more (a run of small ones) goes direct
   const uint64_t touched = 2 + (uint64_t)kShMaxTile * plan.F1 / n;
   const uint32_t span = (uint32_t)std::min<uint64_t>(touched * plan.F2, kPass2SpanMax);
   const uint32_t pw = shuffle_pay_width(t, key_col);
-  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, true, span));
+  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, p1.rid != nullptr, span));
   ShSides sides;
   memset(&sides, 0, sizeof sides);
   sides.s[0] = shuffle_side(t, key_col, p1.cols, fin->cols, p1.rid, fin->rid, cur);
@@ -1091,6 +1116,60 @@ void fill_side(const mdj_table *t, int32_t key_col, const TableBufs &b, uint32_t
   out->nrows = t->nrows;
 }
 }  // namespace
+
+namespace {
+// The checksum term of every row (plans without the fast shuffle).
+template <typename KeyT>
+__global__ void k_terms(const KeyT *__restrict__ keys, const void *pay, int pw, uint32_t n, int term,
+                        uint64_t *__restrict__ out) {
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
+    const uint64_t pb = pay_bits(pay, pw, (uint32_t)r);
+    out[r] = term == TERM_F ? term_f(key_bits(keys[r]), (uint32_t)r, pb) : term_g((uint32_t)r, pb);
+  }
+}
+
+template <typename KeyT>
+int partition_terms_t(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan, int term, Side *out) {
+  cudaStream_t s = ws.stream();
+  const uint32_t n = (uint32_t)t->nrows;
+  mdj_col cols[2] = {t->cols[key_col], {nullptr, MDJ_U64}};
+  mdj_table tt = {cols, 2, t->nrows};
+  if (plan.partition && !plan.lsd && !plan.stable && fast_shuffle_enabled()) {
+    uint32_t *off = (uint32_t *)ws.get((size_t)(plan.nbuckets + 1) * 4);
+    if (!off) return MDJ_ERR_OOM;
+    TableBufs fin, p1;
+    if (plan.F2 == 1) {
+      MDJ_TRY(shuffle_count_pass1_t<KeyT>(ws, t, key_col, plan, off, &fin, nullptr, term));
+    } else {
+      uint32_t *cur2 = nullptr;
+      MDJ_TRY(shuffle_count_pass1_t<KeyT>(ws, t, key_col, plan, off, &p1, &cur2, term));
+      MDJ_TRY(shuffle_pass2_t<KeyT>(ws, &tt, 0, plan, cur2, p1, &fin));
+      release_table_bufs(ws, &tt, &p1);
+    }
+    fill_side(&tt, 0, fin, off, out);
+    return MDJ_OK;
+  }
+  uint64_t *terms = (uint64_t *)ws.get((size_t)(n ? n : 1) * 8);
+  if (!terms) return MDJ_ERR_OOM;
+  const int32_t pay_col = t->ncols < 2 ? -1 : (key_col == 0 ? 1 : 0);
+  if (n) {
+    TraceScope tr("count_terms", s);
+    k_terms<KeyT><<<(unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms() * 8), 256, 0, s>>>(
+        (const KeyT *)t->cols[key_col].data, pay_col < 0 ? nullptr : t->cols[pay_col].data,
+        pay_col < 0 ? 0 : dtype_width(t->cols[pay_col].dtype), n, term, terms);
+  }
+  MDJ_LAUNCH_CHECK();
+  cols[1].data = terms;
+  return partition_side_t<KeyT>(ws, &tt, 0, plan, out);
+}
+}  // namespace
+
+int partition_terms(Workspace &ws, const mdj_table *t, int32_t key_col, const Plan &plan, bool left, Side *out) {
+  const int term = left ? TERM_F : TERM_G;
+  return t->cols[key_col].dtype == MDJ_I64 ? partition_terms_t<int64_t>(ws, t, key_col, plan, term, out)
+                                           : partition_terms_t<int32_t>(ws, t, key_col, plan, term, out);
+}
 
 bool plan_fits_one_launch(const Plan &plan) {
   return !plan.partition || (!plan.lsd && !plan.stable && plan.F2 == 1 && fast_shuffle_enabled());

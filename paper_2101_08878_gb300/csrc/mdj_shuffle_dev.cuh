@@ -61,7 +61,7 @@ __device__ void scatter_direct(const KeyT (&kv)[kRPL], uint32_t wrow0, uint32_t 
 // half of the shared memory holds (5,700 rows of an 8-byte key and payload):
 //   key  [tile]   the key column
 //   pay  [tile]   the first non-key column (every further one in turn)
-//   rid  [tile]   pass 2: row ids
+//   rid  [tile]   pass 2: row ids (none where rows carry a term)
 //   perm [tile]   bucket-ordered position -> local bucket << 16 | row in tile
 //   cnt, lst, gdelta [span]  per local bucket: rank counter, local start,
 //                 destination - position (modulo 2^32)
@@ -87,7 +87,9 @@ constexpr uint32_t kShSmem = 228u * 1024 / kShBlocks - 1024;  // shared memory o
 constexpr int kShScan = (1024 + kShNT - 1) / kShNT;       // local buckets a thread scans at most
 static_assert(kShMaxTile <= 65536, "perm keeps the row in tile in 16 bits");
 
-enum { SH_PASS1 = 0, SH_PASS2 = 1, SH_SEG = 2 };
+// SH_TERM: pass 1 whose rows leave as (key, checksum term) without row ids.
+enum { SH_PASS1 = 0, SH_PASS2 = 1, SH_SEG = 2, SH_TERM = 3 };
+enum { TERM_F = 1, TERM_G = 2 };  // the left and the right side's term (term_f, term_g)
 
 // Shared memory of a block for tiles of `tile` rows (a multiple of 16) and
 // `span` local buckets.
@@ -191,7 +193,7 @@ __device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *sr
       else
         ((uint32_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint32_t)k : ((const uint32_t *)cm.src[j])[r];
     }
-    rid_out[pos] = srid[i];
+    if (rid_out) rid_out[pos] = srid[i];
   }
 }
 

@@ -932,12 +932,12 @@ int entries_pass(Workspace &tmp, const EntrySrc &src, const uint64_t *rows0, con
 // Groups the build side, probes, and builds the entries into the handle.
 // Groups the build side and finds every probe row's group (steps 2-4 of the
 // open): fills `o` (grouped build rows in `keep`, per-probe-row arrays in
-// `tmp`).  want_gkey: also the grouped keys; keep_left: also the group sizes
-// and hit flags that the unmatched-group entries need.  *err_out: a device
+// `tmp`).  keep_left: also the grouped keys, and the group sizes and hit flags
+// that the unmatched-group entries need.  *err_out: a device
 // word set when a global-table probe sequence ran out (read it after a sync).
 template <typename KeyT>
-int group_sides(Workspace &tmp, Workspace &keep, const Side &L, const Side &R, uint32_t nb, bool keep_left,
-                bool want_gkey, GOut &o, int **err_out) {
+int group_sides(Workspace &tmp, Workspace &keep, const Side &L, const Side &R, uint32_t nb, bool keep_left, GOut &o,
+                int **err_out) {
   cudaStream_t s = tmp.stream();
   const uint32_t nL = (uint32_t)L.nrows, nR = (uint32_t)R.nrows;
   std::vector<uint32_t> offL(nb + 1), offR(nb + 1);
@@ -959,11 +959,9 @@ int group_sides(Workspace &tmp, Workspace &keep, const Side &L, const Side &R, u
   int *err = (int *)tmp.get(16);  // [0]: a global-table probe sequence ran out
   if (!o.cnt || !o.gbase || !err) return MDJ_ERR_OOM;
   MDJ_CUDA_TRY(cudaMemsetAsync(err, 0, 16, s));
-  if (keep_left || want_gkey) {
+  if (keep_left) {
     o.gkey = keep.get((size_t)nL * sizeof(KeyT));
     if (!o.gkey) return MDJ_ERR_OOM;
-  }
-  if (keep_left) {
     o.gsize = (uint32_t *)tmp.get((size_t)nL * 4);
     o.hit = (uint32_t *)tmp.get((size_t)nL * 4);
     if (!o.gsize || !o.hit) return MDJ_ERR_OOM;
@@ -1044,7 +1042,7 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
   const uint32_t nL = (uint32_t)L.nrows, nR = (uint32_t)R.nrows;
   GOut o;
   int *err = nullptr;
-  MDJ_TRY(group_sides<KeyT>(tmp, keep, L, R, nb, keep_left, false, o, &err));
+  MDJ_TRY(group_sides<KeyT>(tmp, keep, L, R, nb, keep_left, o, &err));
   // entries: the probe rows (matching ones, or all), then the unmatched groups
   EmitSrc &S = h->src;
   const size_t cap = (size_t)nR + (keep_left ? nL : 0);
@@ -1100,30 +1098,97 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
 }
 
 // ------------------------------------------------------ count + checksum
+//
+// Both sides come shuffled as (key, term) rows: term = f(l) on the build
+// side, g(r) on the probe side.  Per sub-bucket a table of the distinct build
+// keys holds each one's rows and sum of f; a probe row adds rows to the count
+// and g(r) * sum to the checksum.  Nothing per row is written.
+//   light (build side <= kGCap rows): the table in shared memory, probed by
+//     units of kProbeChunk probe rows (each unit builds it anew);
+//   heavy: blocks build the same table from kGCap rows at a time and add its
+//     distinct keys to a global table (linear probing, 5/4 slots per row), so
+//     that a key of millions of rows costs a few thousand global additions;
+//     a second kernel probes that table.
+// Before, the count grouped the build side, wrote every probe row's group and
+// read it back: 5e7 x 2e8 Zipf rows, everything after the shuffle 4.2 -> X ms.
 
-// f of every grouped build position (its key, input row id and first payload)
-template <typename KeyT>
-__global__ void k_count_f(const KeyT *__restrict__ gkey, const uint32_t *__restrict__ grid, const void *gpay, int pw,
-                          uint32_t n, uint64_t *__restrict__ f) {
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride)
-    f[p] = term_f(key_bits(gkey[p]), grid[p], pay_bits(gpay, pw, p));
+// 64-bit addition to shared memory by two native 32-bit atomics: the carry of
+// the low half, known from its old value, goes into the high half.
+__device__ __forceinline__ void add64_shared(uint32_t *lo, uint32_t *hi, uint64_t v) {
+  const uint32_t vl = (uint32_t)v, old = atomicAdd(lo, vl);
+  const uint32_t vh = (uint32_t)(v >> 32) + (old + vl < old ? 1u : 0u);
+  if (vh) atomicAdd(hi, vh);
 }
 
-// totals[0] += group sizes, totals[1] += g(r) * (F[start + size] - F[start])
-// over probe rows r (F: exclusive prefix sums of f, modulo 2^64)
-__global__ void k_count_probe(const uint32_t *__restrict__ cnt, const uint32_t *__restrict__ gbase,
-                              const uint64_t *__restrict__ F, const uint32_t *__restrict__ rrid, const void *rpay,
-                              int pw, uint32_t n, unsigned long long *totals) {
-  uint64_t acc = 0, csum = 0;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
-    const uint32_t c = cnt[r];
-    if (!c) continue;
-    const uint32_t g0 = gbase[r];
-    acc += c;
-    csum += term_g(rrid ? rrid[r] : r, pay_bits(rpay, pw, r)) * (F[g0 + c] - F[g0]);
+// Shared-memory table: keys[kGCap], slots[kGTab] (tag << 16 | representative
+// + 1), and per representative its rows and sum of f in two halves.
+template <typename KeyT>
+struct CountTable {
+  KeyT *keys;
+  uint32_t *slots, *rows, *lo, *hi;
+  __device__ explicit CountTable(unsigned char *smem) {
+    keys = (KeyT *)smem;
+    slots = (uint32_t *)(smem + group_slots_at<KeyT>());
+    rows = slots + kGTab;
+    lo = rows + kGCap;
+    hi = lo + kGCap;
   }
+  static constexpr size_t bytes() { return group_slots_at<KeyT>() + (size_t)(kGTab + 3 * kGCap) * 4; }
+
+  // Builds the table of n <= kGCap rows (ends with a barrier; the table must
+  // not be in use).  Returns log2 of its slots.
+  __device__ __forceinline__ uint32_t build(const KeyT *__restrict__ k, const uint64_t *__restrict__ f, uint32_t n) {
+    const uint32_t logt = small_logt(n), T = 1u << logt, mask = T - 1;
+    KeyT kr[kGRows];
+    uint64_t fr[kGRows];
+#pragma unroll
+    for (int j = 0; j < kGRows; j++) {
+      const uint32_t i = threadIdx.x + j * kGT;
+      kr[j] = i < n ? k[i] : KeyT(0);
+      fr[j] = i < n ? f[i] : 0ull;
+    }
+    for (uint32_t s = threadIdx.x; s < T; s += kGT) slots[s] = 0;
+#pragma unroll
+    for (int j = 0; j < kGRows; j++) {
+      const uint32_t i = threadIdx.x + j * kGT;
+      if (i < n) {
+        keys[i] = kr[j];
+        rows[i] = lo[i] = hi[i] = 0;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kGRows; j++) {
+      const uint32_t i = threadIdx.x + j * kGT;
+      if (i < n) {
+        uint32_t s, tag;
+        small_slot_tag(key_bits(kr[j]), logt, s, tag);
+        const uint32_t w = (tag << 16) | (i + 1);
+        uint32_t rep = i;
+        for (uint32_t p = 0; p <= mask; p++) {  // ends: 2 slots per row, so a free slot exists
+          uint32_t cur = slots[s];
+          if (cur == 0) {
+            const uint32_t prev = atomicCAS(&slots[s], 0u, w);
+            if (prev == 0) break;
+            cur = prev;
+          }
+          if ((cur >> 16) == tag && keys[(cur & 0xFFFFu) - 1] == kr[j]) {
+            rep = (cur & 0xFFFFu) - 1;
+            break;
+          }
+          s = (s + 1) & mask;
+        }
+        atomicAdd(&rows[rep], 1u);
+        add64_shared(&lo[rep], &hi[rep], fr[j]);
+      }
+    }
+    __syncthreads();
+    return logt;
+  }
+};
+
+// Adds this block's sums to totals (all threads call it).
+__device__ __forceinline__ void add_totals(uint64_t acc, uint64_t csum, unsigned long long *totals) {
   acc = warp_sum(acc);
   csum = warp_sum(csum);
   if ((threadIdx.x & 31) == 0) {
@@ -1133,37 +1198,217 @@ __global__ void k_count_probe(const uint32_t *__restrict__ cnt, const uint32_t *
 }
 
 template <typename KeyT>
+__global__ void __launch_bounds__(kGT, 2)
+    k_count_light(const __grid_constant__ GSide L, const __grid_constant__ GSide R,
+                  const LightUnit *__restrict__ units, uint32_t nunits, uint32_t *ticket, unsigned long long *totals) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  CountTable<KeyT> tab(smem);
+  __shared__ uint32_t s_u;
+  const KeyT *__restrict__ Rk = (const KeyT *)R.key;
+  const uint64_t *__restrict__ Rg = (const uint64_t *)R.cols[0];
+  uint64_t acc = 0, csum = 0;
+  for (;;) {
+    if (threadIdx.x == 0) s_u = atomicAdd(ticket, 1u);
+    __syncthreads();  // also: the last unit's probe is done with the table
+    const uint32_t u = s_u;
+    if (u >= nunits) break;
+    const LightUnit U = units[u];
+    const uint32_t lb = L.off[U.b], nl = L.off[U.b + 1] - lb;
+    const uint32_t logt = tab.build((const KeyT *)L.key + lb, (const uint64_t *)L.cols[0] + lb, nl);
+    const uint32_t mask = (1u << logt) - 1;
+    for (uint32_t i0 = threadIdx.x; i0 < U.nr; i0 += 4 * kGT) {
+      KeyT kv[4];
+      uint64_t gv[4];
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const uint32_t i = i0 + e * kGT;
+        kv[e] = i < U.nr ? Rk[U.r0 + i] : KeyT(0);
+        gv[e] = i < U.nr ? Rg[U.r0 + i] : 0ull;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        if (i0 + e * kGT >= U.nr) continue;
+        uint32_t s, tag;
+        small_slot_tag(key_bits(kv[e]), logt, s, tag);
+        for (uint32_t p = 0; p <= mask; p++) {
+          const uint32_t w = tab.slots[s];
+          if (w == 0) break;
+          const uint32_t rep = (w & 0xFFFFu) - 1;
+          if ((w >> 16) == tag && tab.keys[rep] == kv[e]) {
+            acc += tab.rows[rep];
+            csum += gv[e] * ((uint64_t)tab.hi[rep] << 32 | tab.lo[rep]);
+            break;
+          }
+          s = (s + 1) & mask;
+        }
+      }
+    }
+  }
+  add_totals(acc, csum, totals);
+}
+
+// Units of at most kGCap build rows of a heavy sub-bucket: their table's
+// distinct keys into the global one.  Slot words hold a build row + 1 (the
+// row that claimed the slot, whose key is the slot's) and are read through L2:
+// other SMs write them during the kernel.
+template <typename KeyT>
+__global__ void __launch_bounds__(kGT, 2)
+    k_count_heavy_build(const __grid_constant__ GSide L, const HeavyDesc *__restrict__ hd,
+                        const HeavyUnit *__restrict__ units, uint32_t nunits, uint32_t *hslot, uint32_t *hrows,
+                        unsigned long long *hsum, int *err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  CountTable<KeyT> tab(smem);
+  const KeyT *__restrict__ Lk = (const KeyT *)L.key;
+  for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const HeavyUnit U = units[u];
+    const HeavyDesc H = hd[U.h];
+    tab.build(Lk + H.lb + U.i0, (const uint64_t *)L.cols[0] + H.lb + U.i0, U.n);
+    for (uint32_t i = threadIdx.x; i < U.n; i += kGT) {
+      if (!tab.rows[i]) continue;  // not a representative
+      const KeyT kk = tab.keys[i];
+      uint32_t s = big_home(key_bits(kk), H.tsz), p = 0;
+      for (; p < H.tsz; p++) {
+        uint32_t cur = __ldcg(&hslot[H.ts0 + s]);
+        if (cur == 0) {
+          const uint32_t prev = atomicCAS(&hslot[H.ts0 + s], 0u, U.i0 + i + 1);
+          if (prev == 0) break;
+          cur = prev;
+        }
+        if (Lk[H.lb + cur - 1] == kk) break;
+        s = s + 1 == H.tsz ? 0 : s + 1;
+      }
+      if (p == H.tsz) {  // unreachable: there are more slots than rows
+        atomicExch(err, 1);
+        continue;
+      }
+      atomicAdd(&hrows[H.ts0 + s], tab.rows[i]);
+      atomicAdd(&hsum[H.ts0 + s], (unsigned long long)((uint64_t)tab.hi[i] << 32 | tab.lo[i]));
+    }
+    __syncthreads();
+  }
+}
+
+template <typename KeyT>
+__global__ void __launch_bounds__(kHT)
+    k_count_heavy_probe(const __grid_constant__ GSide L, const __grid_constant__ GSide R,
+                        const HeavyDesc *__restrict__ hd, const HeavyUnit *__restrict__ units, uint32_t nunits,
+                        const uint32_t *__restrict__ hslot, const uint32_t *__restrict__ hrows,
+                        const unsigned long long *__restrict__ hsum, unsigned long long *totals, int *err) {
+  const KeyT *__restrict__ Lk = (const KeyT *)L.key;
+  const KeyT *__restrict__ Rk = (const KeyT *)R.key;
+  const uint64_t *__restrict__ Rg = (const uint64_t *)R.cols[0];
+  uint64_t acc = 0, csum = 0;
+  for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const HeavyUnit U = units[u];
+    const HeavyDesc H = hd[U.h];
+    for (uint32_t i0 = threadIdx.x; i0 < U.n; i0 += 4 * kHT) {
+      KeyT kv[4];
+      uint64_t gv[4];
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const uint32_t i = i0 + e * kHT;
+        kv[e] = i < U.n ? Rk[U.i0 + i] : KeyT(0);
+        gv[e] = i < U.n ? Rg[U.i0 + i] : 0ull;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        if (i0 + e * kHT >= U.n) continue;
+        uint32_t s = big_home(key_bits(kv[e]), H.tsz), p = 0;
+        for (; p < H.tsz; p++) {
+          const uint32_t w = hslot[H.ts0 + s];
+          if (w == 0) break;
+          if (Lk[H.lb + w - 1] == kv[e]) {
+            acc += hrows[H.ts0 + s];
+            csum += gv[e] * hsum[H.ts0 + s];
+            break;
+          }
+          s = s + 1 == H.tsz ? 0 : s + 1;
+        }
+        if (p == H.tsz) atomicExch(err, 1);  // unreachable: a slot is empty
+      }
+    }
+  }
+  add_totals(acc, csum, totals);
+}
+
+template <typename KeyT>
 int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, uint64_t *count, uint64_t *checksum) {
   cudaStream_t s = ws.stream();
-  const uint32_t nL = (uint32_t)L.nrows, nR = (uint32_t)R.nrows;
-  GOut o;
-  int *err = nullptr;
-  MDJ_TRY(group_sides<KeyT>(ws, ws, L, R, nb, false, true, o, &err));
-  uint64_t *F = (uint64_t *)ws.get(((size_t)nL + 1) * 8);
-  unsigned long long *tot = (unsigned long long *)ws.get(16);
-  if (!F || !tot) return MDJ_ERR_OOM;
-  MDJ_CUDA_TRY(cudaMemsetAsync(F + nL, 0, 8, s));
-  MDJ_CUDA_TRY(cudaMemsetAsync(tot, 0, 16, s));
-  const unsigned grid = (unsigned)num_sms() * 8;
-  {
-    TraceScope tr("count_f", s);
-    k_count_f<KeyT><<<grid, 256, 0, s>>>((const KeyT *)o.gkey, o.grid, L.ncols ? o.gcols[0] : nullptr,
-                                         L.ncols ? L.widths[0] : 0, nL, F);
-  }
-  MDJ_LAUNCH_CHECK();
-  MDJ_TRY(exclusive_scan_u64(ws, F, F, (size_t)nL + 1));
-  {
-    TraceScope tr("count_probe", s);
-    k_count_probe<<<grid, 256, 0, s>>>(o.cnt, o.gbase, F, R.rid, R.ncols ? R.cols[0] : nullptr,
-                                       R.ncols ? R.widths[0] : 0, nR, tot);
-  }
-  MDJ_LAUNCH_CHECK();
-  unsigned long long host[2] = {0, 0};
-  int herr = 0;
-  MDJ_CUDA_TRY(cudaMemcpyAsync(host, tot, 16, cudaMemcpyDeviceToHost, s));
-  MDJ_CUDA_TRY(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
+  std::vector<uint32_t> offL(nb + 1), offR(nb + 1);
+  MDJ_CUDA_TRY(cudaMemcpyAsync(offL.data(), L.off, (size_t)(nb + 1) * 4, cudaMemcpyDeviceToHost, s));
+  MDJ_CUDA_TRY(cudaMemcpyAsync(offR.data(), R.off, (size_t)(nb + 1) * 4, cudaMemcpyDeviceToHost, s));
   MDJ_CUDA_TRY(cudaStreamSynchronize(s));
-  if (herr) return MDJ_ERR_INTERNAL;
+  std::vector<LightUnit> light;
+  std::vector<HeavyDesc> heavy;
+  std::vector<HeavyUnit> hbuild, hprobe;
+  uint64_t hslots = 0;
+  for (uint32_t b = 0; b < nb; b++) {
+    const uint32_t nl = offL[b + 1] - offL[b], nr = offR[b + 1] - offR[b];
+    if (nl == 0 || nr == 0) continue;  // no pairs
+    if (nl <= kGCap) {
+      for (uint32_t c0 = 0; c0 < nr; c0 += kProbeChunk)
+        light.push_back({b, offR[b] + c0, std::min(kProbeChunk, nr - c0), -1});
+      continue;
+    }
+    const uint32_t h = (uint32_t)heavy.size(), tsz = nl + nl / 4;
+    if (hslots + tsz >= (1ull << 32)) return MDJ_ERR_TOO_LARGE;
+    heavy.push_back({b, offL[b], nl, tsz, (uint32_t)hslots, 0});
+    hslots += tsz;
+    for (uint32_t i0 = 0; i0 < nl; i0 += kGCap) hbuild.push_back({h, i0, std::min(kGCap, nl - i0)});
+    for (uint32_t c0 = 0; c0 < nr; c0 += kHChunk) hprobe.push_back({h, offR[b] + c0, std::min(kHChunk, nr - c0)});
+  }
+  // largest first, so the persistent blocks finish together
+  std::stable_sort(light.begin(), light.end(), [](const LightUnit &a, const LightUnit &b) { return a.nr > b.nr; });
+  int rc = MDJ_OK;
+  LightUnit *d_light = upload(ws, light, &rc);
+  HeavyDesc *d_heavy = upload(ws, heavy, &rc);
+  HeavyUnit *d_hbuild = upload(ws, hbuild, &rc), *d_hprobe = upload(ws, hprobe, &rc);
+  MDJ_TRY(rc);
+  // totals (2 words) | ticket | error
+  unsigned long long *tot = (unsigned long long *)ws.get(32);
+  if (!tot) return MDJ_ERR_OOM;
+  MDJ_CUDA_TRY(cudaMemsetAsync(tot, 0, 32, s));
+  uint32_t *ticket = (uint32_t *)(tot + 2);
+  int *err = (int *)(tot + 3);
+  const GSide gL = to_gside(L), gR = to_gside(R);
+  const size_t sm = CountTable<KeyT>::bytes();
+  static PerDeviceOnce once;
+  MDJ_TRY(once_per_device(once, [sm] {
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_light<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_heavy_build<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    return (int)MDJ_OK;
+  }));
+  if (!heavy.empty()) {
+    uint32_t *hslot = (uint32_t *)ws.get((size_t)hslots * 4), *hrows = (uint32_t *)ws.get((size_t)hslots * 4);
+    unsigned long long *hsum = (unsigned long long *)ws.get((size_t)hslots * 8);
+    if (!hslot || !hrows || !hsum) return MDJ_ERR_OOM;
+    MDJ_CUDA_TRY(cudaMemsetAsync(hslot, 0, (size_t)hslots * 4, s));
+    MDJ_CUDA_TRY(cudaMemsetAsync(hrows, 0, (size_t)hslots * 4, s));
+    MDJ_CUDA_TRY(cudaMemsetAsync(hsum, 0, (size_t)hslots * 8, s));
+    {
+      TraceScope tr("count_heavy_build", s);
+      k_count_heavy_build<KeyT><<<grid_for(hbuild.size(), 2), kGT, sm, s>>>(gL, d_heavy, d_hbuild,
+                                                                           (uint32_t)hbuild.size(), hslot, hrows, hsum,
+                                                                           err);
+    }
+    MDJ_LAUNCH_CHECK();
+    {
+      TraceScope tr("count_heavy_probe", s);
+      k_count_heavy_probe<KeyT><<<grid_for(hprobe.size(), 8), kHT, 0, s>>>(
+          gL, gR, d_heavy, d_hprobe, (uint32_t)hprobe.size(), hslot, hrows, hsum, tot, err);
+    }
+    MDJ_LAUNCH_CHECK();
+  }
+  if (!light.empty()) {
+    TraceScope tr("count_light", s);
+    k_count_light<KeyT><<<grid_for(light.size(), 2), kGT, sm, s>>>(gL, gR, d_light, (uint32_t)light.size(), ticket,
+                                                                    tot);
+  }
+  MDJ_LAUNCH_CHECK();
+  unsigned long long host[4] = {0, 0, 0, 0};
+  MDJ_CUDA_TRY(cudaMemcpyAsync(host, tot, sizeof host, cudaMemcpyDeviceToHost, s));
+  MDJ_CUDA_TRY(cudaStreamSynchronize(s));
+  if (host[3]) return MDJ_ERR_INTERNAL;
   *count = host[0];
   *checksum = host[1];
   return MDJ_OK;
@@ -1184,8 +1429,8 @@ int grouped_count_checksum(const mdj_table *left, int32_t lk, const mdj_table *r
   Workspace ws(alloc, (cudaStream_t)stream);
   const Plan plan = make_plan(left->nrows, P, kGCap, P > 1);
   Side L, R;
-  MDJ_TRY(partition_side(ws, left, lk, plan, &L));
-  MDJ_TRY(partition_side(ws, right, rk, plan, &R));
+  MDJ_TRY(partition_terms(ws, left, lk, plan, true, &L));
+  MDJ_TRY(partition_terms(ws, right, rk, plan, false, &R));
   return left->cols[lk].dtype == MDJ_I64 ? grouped_count_t<int64_t>(ws, L, R, plan.nbuckets, count, checksum)
                                           : grouped_count_t<int32_t>(ws, L, R, plan.nbuckets, count, checksum);
 }
