@@ -1110,7 +1110,7 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
 //     that a key of millions of rows costs a few thousand global additions;
 //     a second kernel probes that table.
 // Before, the count grouped the build side, wrote every probe row's group and
-// read it back: 5e7 x 2e8 Zipf rows, everything after the shuffle 4.2 -> X ms.
+// read it back: 5e7 x 2e8 Zipf rows, everything after the shuffle 4.2 -> 1.3 ms.
 
 // 64-bit addition to shared memory by two native 32-bit atomics: the carry of
 // the low half, known from its old value, goes into the high half.
@@ -1136,7 +1136,10 @@ struct CountTable {
   static constexpr size_t bytes() { return group_slots_at<KeyT>() + (size_t)(kGTab + 3 * kGCap) * 4; }
 
   // Builds the table of n <= kGCap rows (ends with a barrier; the table must
-  // not be in use).  Returns log2 of its slots.
+  // not be in use).  Returns log2 of its slots.  HOT: a few keys may hold most
+  // rows, so a warp adds its most frequent key's rows in one go (a chunk of
+  // one key otherwise waits on 4096 additions to one address).
+  template <bool HOT>
   __device__ __forceinline__ uint32_t build(const KeyT *__restrict__ k, const uint64_t *__restrict__ f, uint32_t n) {
     const uint32_t logt = small_logt(n), T = 1u << logt, mask = T - 1;
     KeyT kr[kGRows];
@@ -1160,11 +1163,12 @@ struct CountTable {
 #pragma unroll
     for (int j = 0; j < kGRows; j++) {
       const uint32_t i = threadIdx.x + j * kGT;
+      uint32_t rep = 0xFFFFFFFFu;
       if (i < n) {
         uint32_t s, tag;
         small_slot_tag(key_bits(kr[j]), logt, s, tag);
         const uint32_t w = (tag << 16) | (i + 1);
-        uint32_t rep = i;
+        rep = i;
         for (uint32_t p = 0; p <= mask; p++) {  // ends: 2 slots per row, so a free slot exists
           uint32_t cur = slots[s];
           if (cur == 0) {
@@ -1178,8 +1182,27 @@ struct CountTable {
           }
           s = (s + 1) & mask;
         }
-        atomicAdd(&rows[rep], 1u);
-        add64_shared(&lo[rep], &hi[rep], fr[j]);
+      }
+      uint64_t v = fr[j];
+      uint32_t c = rep != 0xFFFFFFFFu ? 1u : 0u;
+      if (HOT) {
+        const uint32_t lane = threadIdx.x & 31, peers = __match_any_sync(0xffffffffu, rep);
+        const uint32_t top = __reduce_max_sync(0xffffffffu, c ? (uint32_t)__popc(peers) << 5 | lane : 0u);
+        if ((top >> 5) >= 4) {  // uniform over the warp: lane `top & 31` adds for its peers
+          const uint32_t group = __shfl_sync(0xffffffffu, peers, top & 31);
+          const bool in = group >> lane & 1;
+          const uint64_t sum = warp_sum(in ? v : 0ull);
+          if (lane == (top & 31)) {
+            v = sum;
+            c = (uint32_t)__popc(group);
+          } else if (in) {
+            c = 0;
+          }
+        }
+      }
+      if (c) {
+        atomicAdd(&rows[rep], c);
+        add64_shared(&lo[rep], &hi[rep], v);
       }
     }
     __syncthreads();
@@ -1214,7 +1237,7 @@ __global__ void __launch_bounds__(kGT, 2)
     if (u >= nunits) break;
     const LightUnit U = units[u];
     const uint32_t lb = L.off[U.b], nl = L.off[U.b + 1] - lb;
-    const uint32_t logt = tab.build((const KeyT *)L.key + lb, (const uint64_t *)L.cols[0] + lb, nl);
+    const uint32_t logt = tab.template build<false>((const KeyT *)L.key + lb, (const uint64_t *)L.cols[0] + lb, nl);
     const uint32_t mask = (1u << logt) - 1;
     for (uint32_t i0 = threadIdx.x; i0 < U.nr; i0 += 4 * kGT) {
       KeyT kv[4];
@@ -1247,13 +1270,65 @@ __global__ void __launch_bounds__(kGT, 2)
   add_totals(acc, csum, totals);
 }
 
+// Per sub-bucket, packed for two scans: light units << 32 | heavy build units,
+// and heavy probe units << 40 | global-table slots (entry nb: 0).
+__host__ __device__ constexpr uint32_t count_slots(uint32_t nl) {
+  return nl / 4 < 0xFFFFFFFFu - nl ? nl + nl / 4 : 0xFFFFFFFFu;
+}
+constexpr uint64_t kSlotMask = (1ull << 40) - 1;
+__global__ void k_count_sizes(const uint32_t *__restrict__ offL, const uint32_t *__restrict__ offR, uint32_t nb,
+                              uint64_t *__restrict__ a, uint64_t *__restrict__ b) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i > nb) return;
+  uint64_t va = 0, vb = 0;
+  if (i < nb) {
+    const uint32_t nl = offL[i + 1] - offL[i], nr = offR[i + 1] - offR[i];
+    if (nl && nr && nl <= kGCap) va = (uint64_t)((nr - 1) / kProbeChunk + 1) << 32;
+    if (nr && nl > kGCap) {
+      va = (nl - 1) / kGCap + 1;
+      vb = (uint64_t)((nr - 1) / kHChunk + 1) << 40 | count_slots(nl);
+    }
+  }
+  a[i] = va;
+  b[i] = vb;
+}
+
+// The units of every sub-bucket, one warp per sub-bucket.
+__global__ void k_count_expand(const uint32_t *__restrict__ offL, const uint32_t *__restrict__ offR, uint32_t nb,
+                               const uint64_t *__restrict__ a, const uint64_t *__restrict__ b,
+                               LightUnit *__restrict__ light, HeavyUnit *__restrict__ hbuild,
+                               HeavyUnit *__restrict__ hprobe) {
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nb) return;
+  const uint32_t nl = offL[i + 1] - offL[i], r0 = offR[i], nr = offR[i + 1] - r0;
+  if (!nl || !nr) return;
+  if (nl <= kGCap) {
+    const uint32_t u0 = (uint32_t)(a[i] >> 32), nu = (nr - 1) / kProbeChunk + 1;
+    for (uint32_t u = lane; u < nu; u += 32)
+      light[u0 + u] = {i, r0 + u * kProbeChunk, min(kProbeChunk, nr - u * kProbeChunk), -1};
+    return;
+  }
+  const uint32_t b0 = (uint32_t)a[i], nbu = (nl - 1) / kGCap + 1;
+  for (uint32_t u = lane; u < nbu; u += 32) hbuild[b0 + u] = {i, u * kGCap, min(kGCap, nl - u * kGCap)};
+  const uint32_t p0 = (uint32_t)(b[i] >> 40), npu = (nr - 1) / kHChunk + 1;
+  for (uint32_t u = lane; u < npu; u += 32) hprobe[p0 + u] = {i, r0 + u * kHChunk, min(kHChunk, nr - u * kHChunk)};
+}
+
+// The global table of a heavy sub-bucket.
+struct HeavyTable {
+  uint32_t lb, nl, tsz;
+  uint64_t ts0;
+  __device__ HeavyTable(const uint32_t *off, const uint64_t *slots, uint32_t b)
+      : lb(off[b]), nl(off[b + 1] - off[b]), tsz(count_slots(nl)), ts0(slots[b] & kSlotMask) {}
+};
+
 // Units of at most kGCap build rows of a heavy sub-bucket: their table's
 // distinct keys into the global one.  Slot words hold a build row + 1 (the
 // row that claimed the slot, whose key is the slot's) and are read through L2:
 // other SMs write them during the kernel.
 template <typename KeyT>
 __global__ void __launch_bounds__(kGT, 2)
-    k_count_heavy_build(const __grid_constant__ GSide L, const HeavyDesc *__restrict__ hd,
+    k_count_heavy_build(const __grid_constant__ GSide L, const uint64_t *__restrict__ slots,
                         const HeavyUnit *__restrict__ units, uint32_t nunits, uint32_t *hslot, uint32_t *hrows,
                         unsigned long long *hsum, int *err) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1261,8 +1336,8 @@ __global__ void __launch_bounds__(kGT, 2)
   const KeyT *__restrict__ Lk = (const KeyT *)L.key;
   for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
     const HeavyUnit U = units[u];
-    const HeavyDesc H = hd[U.h];
-    tab.build(Lk + H.lb + U.i0, (const uint64_t *)L.cols[0] + H.lb + U.i0, U.n);
+    const HeavyTable H(L.off, slots, U.h);
+    tab.template build<true>(Lk + H.lb + U.i0, (const uint64_t *)L.cols[0] + H.lb + U.i0, U.n);
     for (uint32_t i = threadIdx.x; i < U.n; i += kGT) {
       if (!tab.rows[i]) continue;  // not a representative
       const KeyT kk = tab.keys[i];
@@ -1291,7 +1366,7 @@ __global__ void __launch_bounds__(kGT, 2)
 template <typename KeyT>
 __global__ void __launch_bounds__(kHT)
     k_count_heavy_probe(const __grid_constant__ GSide L, const __grid_constant__ GSide R,
-                        const HeavyDesc *__restrict__ hd, const HeavyUnit *__restrict__ units, uint32_t nunits,
+                        const uint64_t *__restrict__ slots, const HeavyUnit *__restrict__ units, uint32_t nunits,
                         const uint32_t *__restrict__ hslot, const uint32_t *__restrict__ hrows,
                         const unsigned long long *__restrict__ hsum, unsigned long long *totals, int *err) {
   const KeyT *__restrict__ Lk = (const KeyT *)L.key;
@@ -1300,7 +1375,7 @@ __global__ void __launch_bounds__(kHT)
   uint64_t acc = 0, csum = 0;
   for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
     const HeavyUnit U = units[u];
-    const HeavyDesc H = hd[U.h];
+    const HeavyTable H(L.off, slots, U.h);
     for (uint32_t i0 = threadIdx.x; i0 < U.n; i0 += 4 * kHT) {
       KeyT kv[4];
       uint64_t gv[4];
@@ -1334,36 +1409,32 @@ __global__ void __launch_bounds__(kHT)
 template <typename KeyT>
 int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, uint64_t *count, uint64_t *checksum) {
   cudaStream_t s = ws.stream();
-  std::vector<uint32_t> offL(nb + 1), offR(nb + 1);
-  MDJ_CUDA_TRY(cudaMemcpyAsync(offL.data(), L.off, (size_t)(nb + 1) * 4, cudaMemcpyDeviceToHost, s));
-  MDJ_CUDA_TRY(cudaMemcpyAsync(offR.data(), R.off, (size_t)(nb + 1) * 4, cudaMemcpyDeviceToHost, s));
-  MDJ_CUDA_TRY(cudaStreamSynchronize(s));
-  std::vector<LightUnit> light;
-  std::vector<HeavyDesc> heavy;
-  std::vector<HeavyUnit> hbuild, hprobe;
-  uint64_t hslots = 0;
-  for (uint32_t b = 0; b < nb; b++) {
-    const uint32_t nl = offL[b + 1] - offL[b], nr = offR[b + 1] - offR[b];
-    if (nl == 0 || nr == 0) continue;  // no pairs
-    if (nl <= kGCap) {
-      for (uint32_t c0 = 0; c0 < nr; c0 += kProbeChunk)
-        light.push_back({b, offR[b] + c0, std::min(kProbeChunk, nr - c0), -1});
-      continue;
-    }
-    const uint32_t h = (uint32_t)heavy.size(), tsz = nl + nl / 4;
-    if (hslots + tsz >= (1ull << 32)) return MDJ_ERR_TOO_LARGE;
-    heavy.push_back({b, offL[b], nl, tsz, (uint32_t)hslots, 0});
-    hslots += tsz;
-    for (uint32_t i0 = 0; i0 < nl; i0 += kGCap) hbuild.push_back({h, i0, std::min(kGCap, nl - i0)});
-    for (uint32_t c0 = 0; c0 < nr; c0 += kHChunk) hprobe.push_back({h, offR[b] + c0, std::min(kHChunk, nr - c0)});
+  // the units, planned on the device: only their numbers and the slots come back
+  uint64_t *pa = (uint64_t *)ws.get((size_t)(nb + 1) * 8), *pb = (uint64_t *)ws.get((size_t)(nb + 1) * 8);
+  if (!pa || !pb) return MDJ_ERR_OOM;
+  {
+    TraceScope tr("count_sizes", s);
+    k_count_sizes<<<(nb + 256) / 256, 256, 0, s>>>(L.off, R.off, nb, pa, pb);
   }
-  // largest first, so the persistent blocks finish together
-  std::stable_sort(light.begin(), light.end(), [](const LightUnit &a, const LightUnit &b) { return a.nr > b.nr; });
-  int rc = MDJ_OK;
-  LightUnit *d_light = upload(ws, light, &rc);
-  HeavyDesc *d_heavy = upload(ws, heavy, &rc);
-  HeavyUnit *d_hbuild = upload(ws, hbuild, &rc), *d_hprobe = upload(ws, hprobe, &rc);
-  MDJ_TRY(rc);
+  MDJ_LAUNCH_CHECK();
+  MDJ_TRY(exclusive_scan_u64(ws, pa, pa, (size_t)nb + 1));
+  MDJ_TRY(exclusive_scan_u64(ws, pb, pb, (size_t)nb + 1));
+  uint64_t na = 0, nbp = 0;
+  MDJ_CUDA_TRY(cudaMemcpyAsync(&na, pa + nb, 8, cudaMemcpyDeviceToHost, s));
+  MDJ_CUDA_TRY(cudaMemcpyAsync(&nbp, pb + nb, 8, cudaMemcpyDeviceToHost, s));
+  MDJ_CUDA_TRY(cudaStreamSynchronize(s));
+  const uint32_t nlight = (uint32_t)(na >> 32), nhb = (uint32_t)na, nhp = (uint32_t)(nbp >> 40);
+  const uint64_t hslots = nbp & kSlotMask;
+  LightUnit *d_light = (LightUnit *)ws.get((size_t)nlight * sizeof(LightUnit));
+  HeavyUnit *d_hbuild = (HeavyUnit *)ws.get((size_t)nhb * sizeof(HeavyUnit));
+  HeavyUnit *d_hprobe = (HeavyUnit *)ws.get((size_t)nhp * sizeof(HeavyUnit));
+  if (!d_light || !d_hbuild || !d_hprobe) return MDJ_ERR_OOM;
+  {
+    TraceScope tr("count_expand", s);
+    k_count_expand<<<(unsigned)(((uint64_t)nb * 32 + 255) / 256), 256, 0, s>>>(L.off, R.off, nb, pa, pb, d_light,
+                                                                              d_hbuild, d_hprobe);
+  }
+  MDJ_LAUNCH_CHECK();
   // totals (2 words) | ticket | error
   unsigned long long *tot = (unsigned long long *)ws.get(32);
   if (!tot) return MDJ_ERR_OOM;
@@ -1378,7 +1449,7 @@ int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, ui
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_heavy_build<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     return (int)MDJ_OK;
   }));
-  if (!heavy.empty()) {
+  if (nhb) {
     uint32_t *hslot = (uint32_t *)ws.get((size_t)hslots * 4), *hrows = (uint32_t *)ws.get((size_t)hslots * 4);
     unsigned long long *hsum = (unsigned long long *)ws.get((size_t)hslots * 8);
     if (!hslot || !hrows || !hsum) return MDJ_ERR_OOM;
@@ -1387,22 +1458,19 @@ int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, ui
     MDJ_CUDA_TRY(cudaMemsetAsync(hsum, 0, (size_t)hslots * 8, s));
     {
       TraceScope tr("count_heavy_build", s);
-      k_count_heavy_build<KeyT><<<grid_for(hbuild.size(), 2), kGT, sm, s>>>(gL, d_heavy, d_hbuild,
-                                                                           (uint32_t)hbuild.size(), hslot, hrows, hsum,
-                                                                           err);
+      k_count_heavy_build<KeyT><<<grid_for(nhb, 2), kGT, sm, s>>>(gL, pb, d_hbuild, nhb, hslot, hrows, hsum, err);
     }
     MDJ_LAUNCH_CHECK();
     {
       TraceScope tr("count_heavy_probe", s);
-      k_count_heavy_probe<KeyT><<<grid_for(hprobe.size(), 8), kHT, 0, s>>>(
-          gL, gR, d_heavy, d_hprobe, (uint32_t)hprobe.size(), hslot, hrows, hsum, tot, err);
+      k_count_heavy_probe<KeyT><<<grid_for(nhp, 8), kHT, 0, s>>>(gL, gR, pb, d_hprobe, nhp, hslot, hrows, hsum, tot,
+                                                                 err);
     }
     MDJ_LAUNCH_CHECK();
   }
-  if (!light.empty()) {
+  if (nlight) {
     TraceScope tr("count_light", s);
-    k_count_light<KeyT><<<grid_for(light.size(), 2), kGT, sm, s>>>(gL, gR, d_light, (uint32_t)light.size(), ticket,
-                                                                    tot);
+    k_count_light<KeyT><<<grid_for(nlight, 2), kGT, sm, s>>>(gL, gR, d_light, nlight, ticket, tot);
   }
   MDJ_LAUNCH_CHECK();
   unsigned long long host[4] = {0, 0, 0, 0};
