@@ -5,15 +5,16 @@
 // On one GPU that exchange is a scatter: partition p's region of the output
 // plays worker p's receive buffer.  Kernels:
 //
-//   k_hist       per-tile bucket histogram (warp match_any + shared counters);
-//                optionally also the per-sub-bucket totals of a two-level plan
+//   k_hist       per-tile bucket histogram (shared counters); optionally also
+//                the per-sub-bucket totals of a two-level plan
 //   (scan)       exclusive scan of the bucket-major (bucket, tile) histogram
 //                matrix = the global base of every (bucket, tile) run
-//   k_scatter    stable local counting sort of a tile in shared memory, then
-//                every column leaves as coalesced runs (one per bucket)
-//                RESERVE variant (pass 2): rows already grouped by pass-1
-//                bucket are split further; each tile reserves its runs with
-//                one atomicAdd per (tile, bucket) - not stable, coalesced
+//   k_partition  stable local counting sort of a tile in shared memory; the
+//                columns leave as coalesced runs (one per bucket)
+//   k_scatter    the same for many buckets, in smaller tiles; RESERVE variant
+//                (pass 2 of the stable two-level plans): rows already grouped
+//                by pass-1 bucket are split further; each tile reserves its
+//                runs with one atomicAdd per (tile, bucket)
 //
 // Every kernel is bandwidth-bound: no tensor cores, integer hashing only.
 #include <stdlib.h>
@@ -36,48 +37,60 @@ size_t scatter_smem_bytes(uint32_t FL) {
   return (size_t)kTile * 8 + (size_t)kTile * 4 + align16((size_t)kNW * FL * 2) + (size_t)FL * 8 + 40 * 4;
 }
 
-// ------------------------------------------------------------------ k_hist
+constexpr int kHistU = 8;  // keys per thread in flight
 
+// ------------------------------------------------------------------ k_hist
+//
+// hist[b * ntiles + t] = rows of bucket b in tile t.  With few buckets the
+// lanes of a warp would add to the same few counters, so each counter has
+// `copies` (a power of two) neighbouring copies, one per group of lanes.
 template <typename KeyT>
-__global__ void __launch_bounds__(kHistThreads) k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
-                                                       uint32_t F, uint32_t tile, uint32_t ntiles,
+__global__ void __launch_bounds__(kHistThreads, 4) k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
+                                                       uint32_t F, uint32_t copies, uint32_t tile, uint32_t ntiles,
                                                        uint32_t *__restrict__ hist, uint32_t *__restrict__ total2,
                                                        uint32_t nsub) {
   extern __shared__ uint32_t sh[];
   uint32_t *cnt = sh;
-  uint32_t *cnt2 = sh + F;
+  uint32_t *cnt2 = sh + F * copies;
+  const uint32_t mine = threadIdx.x & (copies - 1);
   if (total2)
     for (uint32_t i = threadIdx.x; i < nsub; i += blockDim.x) cnt2[i] = 0;
-  constexpr int U = 8;
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    for (uint32_t b = threadIdx.x; b < F; b += blockDim.x) cnt[b] = 0;
+    for (uint32_t b = threadIdx.x; b < F * copies; b += kHistThreads) cnt[b] = 0;
     __syncthreads();
     const uint32_t row0 = t * tile;
-    const uint32_t end = min(row0 + tile, n);
-    for (uint32_t base = row0; base < end; base += blockDim.x * U) {
-      KeyT kv[U];
+    const uint32_t end = row0 + min(tile, n - row0);
+    for (uint32_t base = row0; base < end; base += kHistThreads * kHistU) {
+      KeyT kv[kHistU];
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        uint32_t r = base + u * blockDim.x + threadIdx.x;
+      for (int u = 0; u < kHistU; u++) {
+        const uint32_t r = base + u * kHistThreads + threadIdx.x;
         kv[u] = r < end ? keys[r] : KeyT(0);
       }
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        uint32_t r = base + u * blockDim.x + threadIdx.x;
+      for (int u = 0; u < kHistU; u++) {
+        const uint32_t r = base + u * kHistThreads + threadIdx.x;
         if (r < end) {
           const uint64_t h = fmix64(key_bits(kv[u]));
           if (total2) {
             const uint32_t p = mod_p(h, bs), x = (uint32_t)(h >> 32);
-            atomicAdd(&cnt[p * bs.S1 + __umulhi(x, bs.S1)], 1u);
+            atomicAdd(&cnt[(p * bs.S1 + __umulhi(x, bs.S1)) * copies + mine], 1u);
             atomicAdd(&cnt2[p * bs.S + __umulhi(x, bs.S)], 1u);
           } else {
-            atomicAdd(&cnt[bucket_of(h, bs)], 1u);
+            atomicAdd(&cnt[bucket_of(h, bs) * copies + mine], 1u);
           }
         }
       }
     }
     __syncthreads();
-    for (uint32_t b = threadIdx.x; b < F; b += blockDim.x) hist[(size_t)b * ntiles + t] = cnt[b];
+    if (copies > 1) {  // F * copies <= kHistThreads: one copy per thread, neighbours summed
+      const uint32_t i = threadIdx.x, all = F * copies;
+      uint32_t v = i < all ? cnt[i] : 0u;
+      for (uint32_t o = copies / 2; o > 0; o /= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (i < all && mine == 0) hist[(size_t)(i / copies) * ntiles + t] = v;
+    } else {
+      for (uint32_t b = threadIdx.x; b < F; b += kHistThreads) hist[(size_t)b * ntiles + t] = cnt[b];
+    }
     __syncthreads();
   }
   if (total2) {
@@ -87,8 +100,20 @@ __global__ void __launch_bounds__(kHistThreads) k_hist(const KeyT *__restrict__ 
   }
 }
 
+// Copies of each counter: as many as one block can sum with one thread each,
+// for the few buckets of k_partition's passes.
+constexpr uint32_t kPartitionMaxF = 64;  // see launch_partition
+uint32_t hist_copies(uint32_t F) {
+  uint32_t c = F <= kPartitionMaxF ? 32 : 1;
+  while (c > 1 && F * c > kHistThreads) c /= 2;
+  return c;
+}
+
 // --------------------------------------------------------------- k_scatter
 
+// RESERVE (pass 2 of a two-level plan): the rows come grouped by pass-1 bucket
+// and runs are reserved on cursors; else runs start at the scanned histogram
+// entries and the scatter is stable.
 template <typename KeyT, bool RESERVE>
 __global__ void __launch_bounds__(kNW * 32, 2)
     k_scatter(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs, uint32_t F, uint32_t ntiles,
@@ -120,8 +145,8 @@ __global__ void __launch_bounds__(kNW * 32, 2)
 
   uint32_t Floc = F, lb0 = 0;
   if (RESERVE) {
-    uint32_t b1f = sub_bucket_of(fmix64(key_bits(keys[row0])), bs) / F2;
-    uint32_t b1l = sub_bucket_of(fmix64(key_bits(keys[rend - 1])), bs) / F2;
+    const uint32_t b1f = sub_bucket_of(fmix64(key_bits(keys[row0])), bs) / F2;
+    const uint32_t b1l = sub_bucket_of(fmix64(key_bits(keys[rend - 1])), bs) / F2;
     lb0 = b1f * F2;
     Floc = (b1l - b1f + 1) * F2;
     if (Floc > kPass2SpanMax) {
@@ -170,8 +195,8 @@ __global__ void __launch_bounds__(kNW * 32, 2)
     if (!RESERVE) {
       gbase[b] = tile_base[(size_t)b * ntiles + t];
     } else {
-      uint32_t e = b + 1 < Floc ? lstart[b + 1] : rows;
-      uint32_t cnt = e - lstart[b];
+      const uint32_t e = b + 1 < Floc ? lstart[b + 1] : rows;
+      const uint32_t cnt = e - lstart[b];
       gbase[b] = cnt ? atomicAdd(&cursors[lb0 + b], cnt) : 0u;
     }
   }
@@ -238,6 +263,162 @@ __global__ void __launch_bounds__(kNW * 32, 2)
       if (wrow0 + c * 32 + lane < rend) stage32[lp[c]] = v[c];
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < rows; i += blockDim.x) rid_out[dstmap[i]] = stage32[i];
+  }
+}
+
+// ------------------------------------------------------------- k_partition
+//
+// The stable scatter: persistent blocks, tiles staged in input order as in
+// k_shuffle (key, first payload and row ids by asynchronous copies, a 4-byte
+// permutation entry per row), two blocks per SM.  A row's stable rank: warp w
+// owns rows [w * tile / 16, (w + 1) * tile / 16) and walks them 32 at a time
+// (match_any among the 32, a shared counter per warp and bucket), then the
+// counters become offsets over the warps; the run of (tile, bucket) starts at
+// the scanned histogram entry.
+//
+// DRAM-bound for few buckets.  5e7 rows of 8 + 8 bytes, 8 buckets, with row
+// ids: 0.407 -> 0.306 ms (5.9 TB/s).
+constexpr int kPtGroups = (int)(kShMaxTile / kShNT);  // 32-row groups of a warp's rows at most
+constexpr int kPtWarps = kShNT / 32;
+
+struct PtLayout {
+  uint32_t pay, rid, perm, lst, whist, total;
+  __host__ __device__ PtLayout(uint32_t tile, uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F) {
+    pay = tile * key_width;
+    rid = pay + tile * pay_width;
+    perm = rid + (with_rid ? tile * 4 : 0u);
+    lst = perm + tile * 4;
+    whist = lst + (2 * F + 32) * 4;
+    total = whist + (kPtWarps * F * 2 + 15) / 16 * 16;
+  }
+};
+
+// Tile rows (a multiple of kShNT): the most that leave room for two blocks per
+// SM.
+uint32_t partition_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F) {
+  uint32_t tile = kShMaxTile;
+  while (PtLayout(tile, key_width, pay_width, with_rid, F).total > kShSmem) tile -= kShNT;
+  return tile;
+}
+
+template <typename KeyT, bool EXTRA>
+__global__ void __launch_bounds__(kShNT, kShBlocks)
+    k_partition(const KeyT *__restrict__ keys, uint32_t n, uint32_t tile, uint32_t ntiles, uint32_t pay_width,
+                const __grid_constant__ BucketSpec bs, uint32_t F, const uint32_t *__restrict__ tile_base,
+                const __grid_constant__ ColMove cm, int reg_col, const uint32_t *__restrict__ rid_in,
+                uint32_t *__restrict__ rid_out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const PtLayout lay(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F);
+  KeyT *skey = (KeyT *)smem;
+  unsigned char *spay = smem + lay.pay;
+  uint32_t *srid = (uint32_t *)(smem + lay.rid);
+  uint32_t *perm = (uint32_t *)(smem + lay.perm);
+  uint32_t *lst = (uint32_t *)(smem + lay.lst);
+  uint32_t *gdelta = lst + F;
+  uint32_t *wsum = gdelta + F;
+  uint16_t *whist = (uint16_t *)(smem + lay.whist);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint16_t *wh = whist + warp * F;
+  const int pw = reg_col >= 0 ? cm.width[reg_col] : 0;
+  KeyT *__restrict__ kdst = (KeyT *)cm.dst[cm.key_index];
+  void *pdst = pw ? cm.dst[reg_col] : nullptr;
+  const uint32_t wrows = tile / kPtWarps;  // rows of a warp, a multiple of 32
+
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const uint32_t row0 = t * tile, rows = min(tile, n - row0);
+    load_column<(int)sizeof(KeyT)>((unsigned char *)skey, (const unsigned char *)(keys + row0), rows);
+    cp_async_commit();
+    if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
+    if (rid_in) load_column<4>((unsigned char *)srid, (const unsigned char *)(rid_in + row0), rows);
+    cp_async_commit();
+    for (uint32_t i = lane; i < F; i += 32) wh[i] = 0;
+    cp_async_wait<1>();
+    __syncthreads();
+    // stable ranks inside the warp's rows
+    uint32_t pk[kPtGroups];
+#pragma unroll
+    for (int c = 0; c < kPtGroups; c++) {
+      pk[c] = 0xFFFFFFFFu;
+      if (c * 32u < wrows) {  // uniform over the block
+        const uint32_t i = warp * wrows + c * 32 + lane;
+        const bool valid = i < rows;
+        const uint32_t b = valid ? bucket_of(fmix64(key_bits(skey[i])), bs) : 0xFFFFFFFFu;
+        const uint32_t peers = __match_any_sync(0xffffffffu, b);
+        const uint32_t rank = __popc(peers & lanemask_lt());
+        const uint32_t old = valid ? wh[b] : 0u;
+        __syncwarp();
+        if (valid && rank == 0) wh[b] = (uint16_t)(old + __popc(peers));
+        __syncwarp();
+        if (valid) pk[c] = (b << 16) | (old + rank);
+      }
+    }
+    __syncthreads();
+    // per bucket: offsets over the warps, the local start, the destination
+    const uint32_t per = (F + kShNT - 1) / kShNT;
+    const uint32_t s0 = min(F, threadIdx.x * per), s1 = min(F, s0 + per);
+    uint32_t cb[kShScan], gb[kShScan], own = 0;
+#pragma unroll
+    for (int i = 0; i < kShScan; i++) {
+      cb[i] = gb[i] = 0;
+      if (s0 + i < s1) {
+        gb[i] = tile_base[(size_t)(s0 + i) * ntiles + t];
+#pragma unroll
+        for (int w = 0; w < kPtWarps; w++) {
+          const uint32_t c = whist[w * F + s0 + i];
+          whist[w * F + s0 + i] = (uint16_t)cb[i];
+          cb[i] += c;
+        }
+        own += cb[i];
+      }
+    }
+    const uint32_t inc = warp_inclusive_scan(own);
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    uint32_t ex = inc - own;
+#pragma unroll
+    for (int w = 0; w < kPtWarps; w++)
+      if (w < warp) ex += wsum[w];
+#pragma unroll
+    for (int i = 0; i < kShScan; i++)
+      if (s0 + i < s1) {
+        lst[s0 + i] = ex;
+        gdelta[s0 + i] = gb[i] - ex;
+        ex += cb[i];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kPtGroups; c++)
+      if (pk[c] != 0xFFFFFFFFu) {
+        const uint32_t b = pk[c] >> 16;
+        perm[lst[b] + wh[b] + (pk[c] & 0xFFFFu)] = (b << 16) | (warp * wrows + c * 32 + lane);
+      }
+    cp_async_wait<0>();
+    __syncthreads();
+#pragma unroll 4
+    for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
+      const uint32_t m = perm[p], i = m & 0xFFFFu;
+      const uint32_t d = p + gdelta[m >> 16];
+      kdst[d] = skey[i];
+      if (pw == 8) ((uint64_t *)pdst)[d] = ((const uint64_t *)spay)[i];
+      if (pw == 4) ((uint32_t *)pdst)[d] = ((const uint32_t *)spay)[i];
+      if (rid_out) rid_out[d] = rid_in ? srid[i] : row0 + i;
+    }
+    __syncthreads();
+    if (EXTRA) {
+#pragma unroll 1
+      for (int j = 0; j < cm.n; j++) {
+        if (j == cm.key_index || j == reg_col) continue;
+        load_payload(spay, cm.src[j], cm.width[j], row0, rows);
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+        if (cm.width[j] == 8)
+          write_column<uint64_t>((uint64_t *)cm.dst[j], (const uint64_t *)spay, perm, gdelta, rows);
+        else
+          write_column<uint32_t>((uint32_t *)cm.dst[j], (const uint32_t *)spay, perm, gdelta, rows);
+        __syncthreads();
+      }
+    }
   }
 }
 
@@ -527,8 +708,11 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 
 // ------------------------------------------------------------ small kernels
 
+// First row of every bucket, and n behind the last (as row numbers or as the
+// caller's 64-bit offsets).
+template <typename T>
 __global__ void k_bucket_starts(const uint32_t *__restrict__ hist, uint32_t F, uint32_t ntiles, uint32_t n,
-                                uint32_t *__restrict__ start) {
+                                T *__restrict__ start) {
   uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < F) start[b] = ntiles ? hist[(size_t)b * ntiles] : 0u;
   if (b == F) start[F] = n;
@@ -578,47 +762,93 @@ int set_smem_attrs() {
                                       (int)scatter_smem_bytes(kMaxFanout)));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_scatter<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)scatter_smem_bytes(kPass2SpanMax)));
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_partition<KeyT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_partition<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_hist<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)((kMaxFanout + kMaxSubBuckets) * 4)));
     return (int)MDJ_OK;
   });
 }
 
+// kPartitionMaxF: buckets up to which a stable pass runs as k_partition, above
+// as k_scatter.
+// 5e7 rows, k_partition against k_scatter (whole mdj_partition call, us):
+// 8 + 8 bytes: 32 buckets 499 / 568, 100 655 / 661, 256 693 / 688, 1000 1319 /
+// 1009; 4 + 4 bytes: 32 434 / 493, 100 571 / 601, 256 663 / 612; three columns:
+// 32 580 / 633, 100 748 / 732, 256 888 / 760.  Above, k_partition's counters
+// per warp and bucket shorten its tile, and with it the runs.
+uint32_t stable_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F) {
+  return F > kPartitionMaxF ? kTile : partition_tile_rows(key_width, pay_width, with_rid, F);
+}
+
+// Launches of a stable pass over n > 0 rows into F <= kMaxFanout buckets with
+// a given tile and histogram matrix: the histogram, then (the matrix scanned
+// in between) the scatter.
+template <typename KeyT>
+void launch_hist(const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32_t F, uint32_t tile, uint32_t ntiles,
+                 uint32_t *hist, uint32_t *total2, uint32_t nsub, cudaStream_t s) {
+  const uint32_t copies = hist_copies(F);
+  const size_t hsmem = (size_t)(F * copies + (total2 ? nsub : 0)) * 4;
+  TraceScope tr("hist", s);
+  const unsigned hgrid = (unsigned)(ntiles < (uint32_t)hist_grid(hsmem) ? ntiles : (uint32_t)hist_grid(hsmem));
+  k_hist<KeyT><<<hgrid, kHistThreads, hsmem, s>>>(keys, n, bs, F, copies, tile, ntiles, hist, total2, nsub);
+}
+
+template <typename KeyT>
+void launch_partition(const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32_t F, uint32_t tile, uint32_t ntiles,
+                      uint32_t pay_width, const uint32_t *hist, const ColMove &cm, const uint32_t *rid_in,
+                      uint32_t *rid_out, cudaStream_t s) {
+  TraceScope tr("scatter_stable", s);
+  if (F > kPartitionMaxF) {
+    k_scatter<KeyT, false><<<ntiles, kNW * 32, scatter_smem_bytes(F), s>>>(keys, n, bs, F, ntiles, hist, nullptr, 1, cm,
+                                                                           rid_in, rid_out);
+    return;
+  }
+  const uint32_t sm = PtLayout(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F).total;
+  const uint32_t most = (uint32_t)num_sms() * kShBlocks;
+  const int reg_col = cm.n < 2 ? -1 : (cm.key_index == 0 ? 1 : 0);
+  auto kernel = cm.n > 2 ? k_partition<KeyT, true> : k_partition<KeyT, false>;
+  kernel<<<std::min(ntiles, most), kShNT, sm, s>>>(keys, n, tile, ntiles, pay_width, bs, F, hist, cm, reg_col, rid_in,
+                                                   rid_out);
+}
+
+// Payload bytes a row takes in a tile of the columns of `cm`.
+uint32_t move_pay_width(const ColMove &cm) {
+  if (cm.n > 2) return 8;  // any column may pass through
+  return cm.n < 2 ? 0u : (uint32_t)cm.width[1 - cm.key_index];
+}
+
 // One stable scatter pass over n rows into F <= kMaxFanout buckets.  If
-// `start` is given it receives the F+1 bucket start positions.  If `total2` is
-// given, the pass also counts rows per sub-bucket (nsub entries, zeroed by the
-// caller) for a following RESERVE pass.
+// `start` (row numbers) or `start64` (64-bit offsets) is given it receives the
+// F+1 bucket start positions.  If `total2` is given, the pass also counts rows
+// per sub-bucket (nsub entries, zeroed by the caller) for a following RESERVE
+// pass.
 template <typename KeyT>
 int stable_pass(Workspace &ws, const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32_t F, const ColMove &cm,
-                const uint32_t *rid_in, uint32_t *rid_out, uint32_t *start, uint32_t *total2, uint32_t nsub) {
+                const uint32_t *rid_in, uint32_t *rid_out, uint32_t *start, int64_t *start64, uint32_t *total2,
+                uint32_t nsub) {
   cudaStream_t s = ws.stream();
   MDJ_TRY(set_smem_attrs<KeyT>());
-  const uint32_t tile = kTile;
-  const uint32_t ntiles = (n + tile - 1) / tile;
-  if (ntiles == 0) {
+  if (n == 0) {
     if (start) MDJ_CUDA_TRY(cudaMemsetAsync(start, 0, (size_t)(F + 1) * 4, s));
+    if (start64) MDJ_CUDA_TRY(cudaMemsetAsync(start64, 0, (size_t)(F + 1) * 8, s));
     return MDJ_OK;
   }
+  const uint32_t pw = move_pay_width(cm);
+  const uint32_t tile = stable_tile_rows(sizeof(KeyT), pw, rid_in != nullptr, F);
+  const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile - 1) / tile);
   uint32_t *hist = (uint32_t *)ws.get((size_t)F * ntiles * 4);
   if (!hist) return MDJ_ERR_OOM;
-  const size_t hsmem = (size_t)(F + (total2 ? nsub : 0)) * 4;
-  {
-    TraceScope tr("hist", s);
-    const unsigned hgrid = (unsigned)(ntiles < (uint32_t)hist_grid(hsmem) ? ntiles : (uint32_t)hist_grid(hsmem));
-    k_hist<KeyT><<<hgrid, kHistThreads, hsmem, s>>>(keys, n, bs, F, tile, ntiles, hist, total2, nsub);
-  }
+  launch_hist<KeyT>(keys, n, bs, F, tile, ntiles, hist, total2, nsub, s);
   MDJ_LAUNCH_CHECK();
   MDJ_TRY(exclusive_scan_u32(ws, hist, hist, (size_t)F * ntiles));
-  if (start) {
+  if (start || start64) {
     TraceScope tr("bucket_starts", s);
-    k_bucket_starts<<<(F + 1 + 255) / 256, 256, 0, s>>>(hist, F, ntiles, n, start);
+    if (start) k_bucket_starts<uint32_t><<<(F + 1 + 255) / 256, 256, 0, s>>>(hist, F, ntiles, n, start);
+    if (start64) k_bucket_starts<int64_t><<<(F + 1 + 255) / 256, 256, 0, s>>>(hist, F, ntiles, n, start64);
   }
   MDJ_LAUNCH_CHECK();
-  {
-    TraceScope tr("scatter_stable", s);
-    k_scatter<KeyT, false><<<ntiles, kNW * 32, scatter_smem_bytes(F), s>>>(
-        keys, n, bs, F, ntiles, hist, nullptr, 1, cm, rid_in, rid_out);
-  }
+  launch_partition<KeyT>(keys, n, bs, F, tile, ntiles, pw, hist, cm, rid_in, rid_out, s);
   MDJ_LAUNCH_CHECK();
   ws.give_back(hist);
   return MDJ_OK;
@@ -912,10 +1142,10 @@ int lsd_partition(Workspace &ws, const mdj_table *t, int32_t key_col, uint32_t P
   const uint32_t d0 = kMaxFanout, d1 = (P + kMaxFanout - 1) / kMaxFanout;
   ColMove cm0 = make_move(t, key_col, src, mid.cols);
   MDJ_TRY(stable_pass<KeyT>(ws, (const KeyT *)src[key_col], n, make_digit_spec(P, 1, d0), d0, cm0, nullptr, mid.rid,
-                            nullptr, nullptr, 0));
+                            nullptr, nullptr, nullptr, 0));
   ColMove cm1 = make_move(t, key_col, mid.cols, dst_cols);
   MDJ_TRY(stable_pass<KeyT>(ws, (const KeyT *)mid.cols[key_col], n, make_digit_spec(P, d0, d1), d1, cm1, mid.rid,
-                            dst_rid, nullptr, nullptr, 0));
+                            dst_rid, nullptr, nullptr, nullptr, 0));
   release_table_bufs(ws, t, &mid);
   {
     TraceScope tr("offsets_bsearch", ws.stream());
@@ -931,28 +1161,21 @@ int stable_partition_t(Workspace &ws, const mdj_table *t, int32_t key_col, uint3
                        uint32_t *out_rid, int64_t *out_offsets) {
   cudaStream_t s = ws.stream();
   const uint32_t n = (uint32_t)t->nrows;
-  uint32_t *off = (uint32_t *)ws.get((size_t)(P + 1) * 4);
-  if (!off) return MDJ_ERR_OOM;
-  uint32_t *rid = out_rid;
-  if (!rid && n > 0) {
-    // row ids are needed by the second LSD pass only; a single pass can skip them
-    if (P > kMaxFanout) {
-      rid = (uint32_t *)ws.get((size_t)n * 4);
-      if (!rid) return MDJ_ERR_OOM;
-    }
-  }
   if (P <= kMaxFanout) {
     const void *src[MDJ_MAX_COLS];
     for (int j = 0; j < t->ncols; j++) src[j] = t->cols[j].data;
     ColMove cm = make_move(t, key_col, src, out_cols);
-    MDJ_TRY(stable_pass<KeyT>(ws, (const KeyT *)src[key_col], n, make_spec(P, 1, 1), P, cm, nullptr, out_rid, off,
-                              nullptr, 0));
+    return stable_pass<KeyT>(ws, (const KeyT *)src[key_col], n, make_spec(P, 1, 1), P, cm, nullptr, out_rid, nullptr,
+                             out_offsets, nullptr, 0);
+  }
+  uint32_t *off = (uint32_t *)ws.get((size_t)(P + 1) * 4);
+  if (!off) return MDJ_ERR_OOM;
+  if (n == 0) {
+    MDJ_CUDA_TRY(cudaMemsetAsync(off, 0, (size_t)(P + 1) * 4, s));
   } else {
-    if (n == 0) {
-      MDJ_CUDA_TRY(cudaMemsetAsync(off, 0, (size_t)(P + 1) * 4, s));
-    } else {
-      MDJ_TRY(lsd_partition<KeyT>(ws, t, key_col, P, out_cols, rid, off));
-    }
+    uint32_t *rid = out_rid ? out_rid : (uint32_t *)ws.get((size_t)n * 4);
+    if (!rid) return MDJ_ERR_OOM;
+    MDJ_TRY(lsd_partition<KeyT>(ws, t, key_col, P, out_cols, rid, off));
   }
   {
     TraceScope tr("offsets_i64", s);
@@ -996,7 +1219,7 @@ int partition_side_t(Workspace &ws, const mdj_table *t, int32_t key_col, const P
     MDJ_TRY(alloc_table_bufs(ws, t, &fin, true));
     ColMove cm = make_move(t, key_col, src, fin.cols);
     MDJ_TRY(stable_pass<KeyT>(ws, (const KeyT *)key, n, make_spec(plan.P, plan.S, 1), plan.nbuckets, cm, nullptr,
-                              fin.rid, off, nullptr, 0));
+                              fin.rid, off, nullptr, nullptr, 0));
     key = fin.cols[key_col];
     cols = fin.cols;
     rid = fin.rid;
@@ -1009,7 +1232,7 @@ int partition_side_t(Workspace &ws, const mdj_table *t, int32_t key_col, const P
     MDJ_TRY(alloc_table_bufs(ws, t, &p1, true));
     ColMove cm1 = make_move(t, key_col, src, p1.cols);
     MDJ_TRY(stable_pass<KeyT>(ws, (const KeyT *)key, n, make_spec(plan.P, plan.S, plan.F2), plan.F1, cm1, nullptr,
-                              p1.rid, nullptr, off, plan.nbuckets));
+                              p1.rid, nullptr, nullptr, off, plan.nbuckets));
     MDJ_TRY(exclusive_scan_u32(ws, off, off, plan.nbuckets + 1));
     MDJ_CUDA_TRY(cudaMemcpyAsync(cur, off, (size_t)plan.nbuckets * 4, cudaMemcpyDeviceToDevice, s));
     // pass 2
@@ -1218,33 +1441,30 @@ int stable_partition_scratch_t(const mdj_table *t, int32_t key_col, uint32_t P, 
                                uint32_t *out_rid, int64_t *out_offsets, uint32_t *scratch, size_t scratch_words,
                                cudaStream_t s) {
   const uint32_t n = (uint32_t)t->nrows, F = P;
-  const uint32_t ntiles = (n + kTile - 1) / kTile;
-  const size_t nhist = (size_t)F * ntiles;
   if (stable_partition_scratch_words(n, P) > scratch_words) return MDJ_ERR_TOO_LARGE;
   MDJ_TRY(set_smem_attrs<KeyT>());
-  uint32_t *hist = scratch;
-  uint32_t *sums = hist + nhist;
-  uint32_t *start = sums + scan_scratch_words(nhist);
-  if (ntiles == 0) {
-    MDJ_CUDA_TRY(cudaMemsetAsync(start, 0, (size_t)(F + 1) * 4, s));
-  } else {
-    const BucketSpec bs = make_spec(P, 1, 1);
-    const size_t hsmem = (size_t)F * 4;
-    const unsigned hgrid = (unsigned)(ntiles < (uint32_t)hist_grid(hsmem) ? ntiles : (uint32_t)hist_grid(hsmem));
-    k_hist<KeyT><<<hgrid, kHistThreads, hsmem, s>>>((const KeyT *)t->cols[key_col].data, n, bs, F, kTile, ntiles,
-                                                   hist, nullptr, 0);
-    MDJ_LAUNCH_CHECK();
-    MDJ_TRY(exclusive_scan_u32_scratch(hist, hist, nhist, sums, s));
-    k_bucket_starts<<<(F + 1 + 255) / 256, 256, 0, s>>>(hist, F, ntiles, n, start);
-    MDJ_LAUNCH_CHECK();
-    const void *src[MDJ_MAX_COLS];
-    for (int j = 0; j < t->ncols; j++) src[j] = t->cols[j].data;
-    ColMove cm = make_move(t, key_col, src, out_cols);
-    k_scatter<KeyT, false><<<ntiles, kNW * 32, scatter_smem_bytes(F), s>>>(
-        (const KeyT *)src[key_col], n, bs, F, ntiles, hist, nullptr, 1, cm, nullptr, out_rid);
-    MDJ_LAUNCH_CHECK();
+  if (n == 0) {
+    MDJ_CUDA_TRY(cudaMemsetAsync(out_offsets, 0, (size_t)(F + 1) * 8, s));
+    return MDJ_OK;
   }
-  k_u32_to_i64<<<(P + 1 + 255) / 256, 256, 0, s>>>(start, out_offsets, P + 1);
+  const void *src[MDJ_MAX_COLS];
+  for (int j = 0; j < t->ncols; j++) src[j] = t->cols[j].data;
+  const KeyT *keys = (const KeyT *)src[key_col];
+  const ColMove cm = make_move(t, key_col, src, out_cols);
+  const BucketSpec bs = make_spec(P, 1, 1);
+  const uint32_t pw = move_pay_width(cm);
+  // (tiles have at least kTile rows here, so the matrix fits the scratch words
+  // counted for kTile-row tiles)
+  const uint32_t tile = stable_tile_rows(sizeof(KeyT), pw, false, F);
+  const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile - 1) / tile);
+  const size_t nhist = (size_t)F * ntiles;
+  uint32_t *hist = scratch, *sums = hist + nhist;
+  launch_hist<KeyT>(keys, n, bs, F, tile, ntiles, hist, nullptr, 0, s);
+  MDJ_LAUNCH_CHECK();
+  MDJ_TRY(exclusive_scan_u32_scratch(hist, hist, nhist, sums, s));
+  k_bucket_starts<int64_t><<<(F + 1 + 255) / 256, 256, 0, s>>>(hist, F, ntiles, n, out_offsets);
+  MDJ_LAUNCH_CHECK();
+  launch_partition<KeyT>(keys, n, bs, F, tile, ntiles, pw, hist, cm, nullptr, out_rid, s);
   MDJ_LAUNCH_CHECK();
   return MDJ_OK;
 }
@@ -1275,8 +1495,8 @@ namespace {
 // totals[seg_base + b] += rows of bucket b of each segment.  A block counts a
 // contiguous run of tiles and adds its counters to the totals only where the
 // segment changes (once per tile, one load in flight: 0.61 vs 0.42 ms for 246M rows in 512
-// segments); kHistU keys per thread are loaded before any is counted.
-constexpr int kHistU = 8;
+// segments); kSegHistU keys per thread are loaded before any is counted.
+constexpr int kSegHistU = 8;
 template <typename KeyT>
 __global__ void __launch_bounds__(kHistThreads) k_seg_hist(const KeyT *__restrict__ keys, const SegArgs sg,
                                                            uint32_t ntiles, uint32_t *__restrict__ totals) {
@@ -1301,15 +1521,15 @@ __global__ void __launch_bounds__(kHistThreads) k_seg_hist(const KeyT *__restric
       __syncthreads();
     }
     const KeyT *k = keys + td.row0;
-    for (uint32_t i0 = threadIdx.x; i0 < td.rows; i0 += kHistThreads * kHistU) {
-      KeyT kv[kHistU];
+    for (uint32_t i0 = threadIdx.x; i0 < td.rows; i0 += kHistThreads * kSegHistU) {
+      KeyT kv[kSegHistU];
 #pragma unroll
-      for (int u = 0; u < kHistU; u++) {
+      for (int u = 0; u < kSegHistU; u++) {
         const uint32_t i = i0 + u * kHistThreads;
         kv[u] = i < td.rows ? k[i] : KeyT(0);
       }
 #pragma unroll
-      for (int u = 0; u < kHistU; u++)
+      for (int u = 0; u < kSegHistU; u++)
         if (i0 + u * kHistThreads < td.rows) atomicAdd(&cnt[sub_bucket_of(fmix64(key_bits(kv[u])), sp)], 1u);
     }
   }

@@ -81,3 +81,29 @@ def test_partition_invalid_args():
     with pytest.raises(mdj.MdjError) as e:
         mdj.mdj_partition([k.double()], 0, 4)  # float key
     assert e.value.status == -2
+
+
+@pytest.mark.parametrize("P", [1, 63, 64, 65, 2000])
+@pytest.mark.parametrize("n", [31, 511, 512, 4609, 5631, 5632, 5633, 6143, 6144, 6145, 30_001])
+@pytest.mark.parametrize("layout", ["key", "wide", "narrow", "many"])
+def test_partition_tile_edges_and_unaligned_columns(P, n, layout):
+    # tiles of every size in use, columns that start one element off a 16-byte
+    # boundary, both scatter kernels, and (P = 2000) a second pass that reads row ids
+    mdj = _mdj()
+    key, f64, f32, i32 = _table(n, np.int32 if layout == "narrow" else np.int64, seed=n + P)
+    cols_np = {"key": [key], "wide": [f64, key], "narrow": [key, f32], "many": [f32, key, i32, f64]}[layout]
+    key_col = next(j for j, c in enumerate(cols_np) if c is key)
+    cols = []
+    for c in cols_np:
+        t = torch.empty(n + 1, dtype=torch.from_numpy(c).dtype, device="cuda:0")
+        t[1:] = torch.from_numpy(c)
+        cols.append(t[1:])
+    w_off, w_rid, w_cols = oracle.partition_table(cols_np, key_col, P)
+    for row_ids in (True, False):
+        off, rid, outs = mdj.mdj_partition(cols, key_col, P, row_ids=row_ids)
+        torch.cuda.synchronize()
+        assert np.array_equal(off.cpu().numpy(), w_off)
+        if row_ids:
+            assert np.array_equal(rid.cpu().numpy().view(np.uint32), w_rid)
+        for g, w in zip(outs, w_cols):
+            assert np.array_equal(g.cpu().numpy().view(np.uint8), w.view(np.uint8))
