@@ -652,6 +652,17 @@ __global__ void __launch_bounds__(kCT)
   for (uint32_t i = threadIdx.x; i < n; i += kCT) mg[ebase + i] = stage32[i];
 }
 
+// out = {total rows, entries, error}; moff[entries] = total rows.
+__global__ void k_stream_totals(const uint64_t *r1, const uint32_t *e1, const uint64_t *r2, const uint32_t *e2,
+                                const int *err, uint64_t *__restrict__ moff, unsigned long long *__restrict__ out) {
+  const uint64_t total = *r1 + (r2 ? *r2 : 0ull);
+  const uint32_t nm = *e1 + (e2 ? *e2 : 0u);
+  out[0] = total;
+  out[1] = nm;
+  out[2] = err[0] != 0;
+  moff[nm] = total;
+}
+
 // ------------------------------------------------------------------ emit
 //
 // Each block writes a contiguous range of tiles (kETile rows each).  The
@@ -885,9 +896,12 @@ void plan_units(const std::vector<uint32_t> &offL, const std::vector<uint32_t> &
     for (uint32_t i0 = 0; i0 < nl; i0 += kHChunk) u->hbuild.push_back({h, i0, std::min(kHChunk, nl - i0)});
     for (uint32_t c0 = 0; c0 < nr; c0 += kHChunk) u->hprobe.push_back({h, offR[b] + c0, std::min(kHChunk, nr - c0)});
   }
-  // largest probe chunks first, so the persistent blocks finish together
-  std::stable_sort(u->first.begin(), u->first.end(),
-                   [](const LightUnit &a, const LightUnit &b) { return a.nr > b.nr; });
+  // much larger probe chunks than the mean first, so the persistent blocks
+  // finish together (a full sort by size kept the GPU waiting)
+  uint64_t rows = 0;
+  for (const LightUnit &w : u->first) rows += w.nr;
+  const uint64_t large = u->first.empty() ? 0 : 2 * rows / u->first.size();
+  std::stable_partition(u->first.begin(), u->first.end(), [large](const LightUnit &w) { return w.nr > large; });
 }
 
 template <typename T>
@@ -1067,23 +1081,20 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
     const EntrySrc group_src = {o.gsize, o.hit, nL, SRC_UNMATCHED_GROUPS};
     MDJ_TRY(entries_pass(tmp, group_src, crows1 + c1, cents1 + c1, moff, mr, mg, &crows2, &cents2, &c2));
   }
-  uint64_t t1 = 0, t2 = 0;
-  uint32_t n1 = 0, n2 = 0;
-  int herr[4] = {0, 0, 0, 0};
-  MDJ_CUDA_TRY(cudaMemcpyAsync(&t1, crows1 + c1, 8, cudaMemcpyDeviceToHost, s));
-  MDJ_CUDA_TRY(cudaMemcpyAsync(&n1, cents1 + c1, 4, cudaMemcpyDeviceToHost, s));
-  if (keep_left) {
-    MDJ_CUDA_TRY(cudaMemcpyAsync(&t2, crows2 + c2, 8, cudaMemcpyDeviceToHost, s));
-    MDJ_CUDA_TRY(cudaMemcpyAsync(&n2, cents2 + c2, 4, cudaMemcpyDeviceToHost, s));
+  // the totals in one read; the search sentinel after the last entry
+  unsigned long long *dev = (unsigned long long *)tmp.get(24), host[3] = {0, 0, 0};
+  if (!dev) return MDJ_ERR_OOM;
+  {
+    TraceScope tr("stream_totals", s);
+    k_stream_totals<<<1, 1, 0, s>>>(crows1 + c1, cents1 + c1, keep_left ? crows2 + c2 : nullptr,
+                                    keep_left ? cents2 + c2 : nullptr, err, moff, dev);
   }
-  MDJ_CUDA_TRY(cudaMemcpyAsync(herr, err, 16, cudaMemcpyDeviceToHost, s));
+  MDJ_LAUNCH_CHECK();
+  MDJ_CUDA_TRY(cudaMemcpyAsync(host, dev, sizeof host, cudaMemcpyDeviceToHost, s));
   MDJ_CUDA_TRY(cudaStreamSynchronize(s));
-  if (herr[0]) return MDJ_ERR_INTERNAL;
-  const uint64_t total = t1 + t2;
-  const uint32_t nm = n1 + n2;
-  // the search sentinel after the last entry: moff[nm] = total rows
-  MDJ_CUDA_TRY(cudaMemcpyAsync(moff + nm, &total, 8, cudaMemcpyHostToDevice, s));
-  MDJ_CUDA_TRY(cudaStreamSynchronize(s));
+  if (host[2]) return MDJ_ERR_INTERNAL;
+  const uint64_t total = host[0];
+  const uint32_t nm = (uint32_t)host[1];
   h->total = total;
   S.moff = moff;
   S.mr = mr;
