@@ -101,3 +101,18 @@ def test_batch_segments_of_ragged_sizes(kd, pd, shift):
                               res.right_row.view(torch.int32)[a:b] - int(ro[i]), [c[a:b] for c in res.left_cols],
                               [c[a:b] for c in res.right_cols])
         assert_same_result(gpu_result_np(part), oracle.merge_table(l, r, 0, 0))
+
+
+@pytest.mark.parametrize("nl,P", [(3481, 1), (3482, 1), (3482, 7), (3_564_544, 1), (3_564_545, 1), (3_564_545, 1000)])
+def test_plan_boundaries(nl, P):
+    # unpartitioned / one pass, and one pass / two passes, at the sizes where the plan changes
+    left, right = _tables(nl, 12_289, np.int32, np.float32, nl % 1000)
+    _check(left, right, P)
+
+
+def test_one_pass_plan_with_many_items_per_bucket():
+    # 20 build rows of each key against probe chunks of several items, empty buckets in between
+    rng = np.random.default_rng(8)
+    lk = np.repeat(rng.permutation(10_000)[:400], 20).astype(np.int64)
+    rk = rng.choice(np.concatenate([lk[:40], rng.integers(0, 10_000, 300)]), 60_001)
+    _check([lk, datagen.uniform_payload(rng, lk.size)], [rk, datagen.uniform_payload(rng, rk.size)], 16)
