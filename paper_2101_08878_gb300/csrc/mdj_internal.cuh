@@ -24,7 +24,10 @@ constexpr uint32_t kMaxFanout = 1024;     // buckets of one stable scatter pass
 // Pass-1 buckets of a two-pass join plan.  Both passes of a 1e8-row side in
 // 28.7K sub-buckets: 1.39 ms with 128, 1.41 with 160, 1.40 with 192; with
 // 14.4K sub-buckets (250M rows): 3.28 ms with 128, 3.42 with 192.
+// The stable passes' smaller tiles do better with 256: ordered output of 1e8 x
+// 1e8 rows 7.15 ms, 7.57 with 128.
 constexpr uint32_t kMergeFanout = 128;
+constexpr uint32_t kStableFanout = 256;
 constexpr uint32_t kMinBucketRows = 512;  // build rows a sub-bucket is planned for at least
 constexpr uint32_t kMaxSubBuckets = 49152;  // final buckets of a two-pass plan
 constexpr uint32_t kPass2SpanMax = 1024;  // local buckets of one pass-2 tile
@@ -313,7 +316,8 @@ struct Plan {
   uint32_t join_threads = 512;  // threads of a join block (256 or 512); probe rows per item = 8x
 };
 
-Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition);
+// stable: the plan's passes will be the stable ones.
+Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition, bool stable = false);
 
 // Partition one side (key + every column + row ids) according to `plan` into
 // freshly allocated workspace buffers; fills `out` (offsets per final bucket).

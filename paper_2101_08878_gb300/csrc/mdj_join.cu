@@ -615,9 +615,8 @@ int merge_steps(const mdj_table *left, int32_t lk, const mdj_table *right, int32
   if (!out) return MDJ_ERR_INVALID_ARG;
   memset(out, 0, sizeof *out);
   Workspace ws(alloc, (cudaStream_t)stream);
-  Plan plan = make_plan(left->nrows, P, cap_from_env(), P > 1);
   // ordered output is deterministic only over stable partition passes
-  plan.stable = ordered_output() != 0;
+  const Plan plan = make_plan(left->nrows, P, cap_from_env(), P > 1, ordered_output() != 0);
   const bool k64 = left->cols[lk].dtype == MDJ_I64;
   if (!after_left && plan_fits_one_launch(plan) && !ordered_output()) return merge_one_pass(ws, left, lk, right, rk, plan, out);
   Side L, R;
