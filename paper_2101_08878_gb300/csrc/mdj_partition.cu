@@ -24,6 +24,7 @@
 
 #include "mdj_internal.cuh"
 #include "mdj_shuffle_dev.cuh"
+#include "mdj_sizes.h"
 
 namespace mdj {
 namespace {
@@ -60,19 +61,18 @@ __global__ void __launch_bounds__(kHistThreads, 4) k_hist(const KeyT *__restrict
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     for (uint32_t b = threadIdx.x; b < F * copies; b += kHistThreads) cnt[b] = 0;
     __syncthreads();
-    const uint32_t row0 = t * tile;
-    const uint32_t end = row0 + min(tile, n - row0);
-    for (uint32_t base = row0; base < end; base += kHistThreads * kHistU) {
+    const TileRows tr = tile_rows(n, tile, t);
+    for (uint32_t i0 = 0; i0 < tr.rows; i0 += kHistThreads * kHistU) {
       KeyT kv[kHistU];
 #pragma unroll
       for (int u = 0; u < kHistU; u++) {
-        const uint32_t r = base + u * kHistThreads + threadIdx.x;
-        kv[u] = r < end ? keys[r] : KeyT(0);
+        const uint32_t i = i0 + u * kHistThreads + threadIdx.x;
+        kv[u] = i < tr.rows ? keys[tr.row0 + i] : KeyT(0);
       }
 #pragma unroll
       for (int u = 0; u < kHistU; u++) {
-        const uint32_t r = base + u * kHistThreads + threadIdx.x;
-        if (r < end) {
+        const uint32_t i = i0 + u * kHistThreads + threadIdx.x;
+        if (i < tr.rows) {
           const uint64_t h = fmix64(key_bits(kv[u]));
           if (TWO) {
             const uint32_t p = mod_p(h, bs), x = (uint32_t)(h >> 32);

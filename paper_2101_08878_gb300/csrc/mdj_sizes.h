@@ -1,10 +1,27 @@
-// Size gates of the library's host code that a CPU test can check on its own
-// (plain C++, no CUDA headers).
+// Size gates and row arithmetic of the library that a CPU test can check on its
+// own (plain C++, no CUDA headers).
 #pragma once
 
 #include <stdint.h>
 
+#ifdef __CUDACC__
+#define MDJ_HD __host__ __device__ __forceinline__
+#else
+#define MDJ_HD inline
+#endif
+
 namespace mdj {
+
+// Tile t of n < 2^32 rows in tiles of `tile` rows: its first row and its rows.
+// Kernels step over a tile with row numbers relative to row0: an absolute
+// 32-bit row number wraps when a step passes 2^32, and a loop bounded by the
+// tile's end then starts again at row 0 and never leaves.
+struct TileRows {
+  uint32_t row0, rows;
+};
+MDJ_HD constexpr TileRows tile_rows(uint32_t n, uint32_t tile, uint32_t t) {
+  return {t * tile, n - t * tile < tile ? n - t * tile : tile};
+}
 
 // Output positions of a compaction over m candidate rows come from an
 // exclusive scan of m + 1 keep flags; its last entry (the kept total) must

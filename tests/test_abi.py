@@ -229,6 +229,44 @@ def test_compaction_position_width_gate(tmp_path):
     assert out == ["0", "0", "0", "0", "1", "1"]
 
 
+def _run_sizes_program(tmp_path, body):
+    # a program over mdj_sizes.h (plain C++), compiled with the host compiler; its words of output
+    import shutil
+    import subprocess
+    if not shutil.which("g++"):
+        pytest.skip("no host C++ compiler")
+    src = tmp_path / "sizes.cc"
+    src.write_text('#include "mdj_sizes.h"\n#include <stdio.h>\n#include <algorithm>\n'
+                   'int main() {\n' + body + '  return 0;\n}\n')
+    exe = tmp_path / "sizes"
+    csrc = os.path.join(ROOT, "paper_2101_08878_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-I", csrc, str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_tile_rows_up_to_the_largest_table(tmp_path):
+    # Tiles cover all rows of the largest tables (nrows < 2^32) and a tile's
+    # rows are numbered from its first one, so a step past its end stays far
+    # from 2^32 (tile rows <= 6144, steps of 4096 rows).
+    out = _run_sizes_program(tmp_path, '''
+  const unsigned tiles[] = {4096, 4608, 5632, 6144};
+  const unsigned rows[] = {1u, 4096u, 4097u, 6144u, 1u << 31, 4294963201u, 4294967295u - 4096u, 4294967295u};
+  for (unsigned tile : tiles)
+    for (unsigned n : rows) {
+      const unsigned m = (unsigned)(((unsigned long long)n + tile - 1) / tile);
+      unsigned long long next = 0, most = 0;
+      for (unsigned t = 0; t < m; t++) {
+        const mdj::TileRows r = mdj::tile_rows(n, tile, t);
+        if (r.row0 != next || r.rows < 1) { printf("bad\\n"); return 1; }
+        next += r.rows;
+        most = std::max(most, (unsigned long long)r.rows);
+      }
+      printf("%d\\n", next == n && most <= tile);
+    }
+''')
+    assert out == ["1"] * 32
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and

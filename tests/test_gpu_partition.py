@@ -107,3 +107,46 @@ def test_partition_tile_edges_and_unaligned_columns(P, n, layout):
             assert np.array_equal(rid.cpu().numpy().view(np.uint32), w_rid)
         for g, w in zip(outs, w_cols):
             assert np.array_equal(g.cpu().numpy().view(np.uint8), w.view(np.uint8))
+
+
+def _fmix64(h):
+    # MurmurHash3's 64-bit finalizer on an int64 tensor (wraparound multiplies, logical shifts)
+    for mult in (0xff51afd7ed558ccd - 2**64, 0xc4ceb9fe1a85ec53 - 2**64):
+        h = (h ^ ((h >> 33) & 0x7FFFFFFF)) * mult
+    return h ^ ((h >> 33) & 0x7FFFFFFF)
+
+
+@pytest.mark.parametrize("P", [8, 256])
+def test_partition_of_the_largest_table(P):
+    # 2^32 - 1 rows of one 4-byte key column, the most a table may have; row
+    # i's key is i's bits, so the output checks itself: keys equal to the row
+    # ids, ascending in every partition, each in its hash's partition, all there
+    n = 2**32 - 1
+    mdj = _mdj()
+    dev = torch.device("cuda", 0)
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info(dev)[0] < 80 << 30:
+        pytest.skip("needs 80 GB of device memory")
+    step = 1 << 27
+    keys = torch.empty(n, dtype=torch.int32, device=dev)
+    for r0 in range(0, n, step):
+        keys[r0:r0 + step] = torch.arange(r0, min(n, r0 + step), device=dev)
+    off, rid, (out,) = mdj.mdj_partition([keys], 0, P)
+    assert torch.equal(rid.view(torch.int32), out)
+    del keys, rid
+    off = off.cpu().tolist()
+    assert off[0] == 0 and off[P] == n and sorted(off) == off
+    bounds = torch.tensor(off[1:P], device=dev)
+    starts = bounds[bounds < n]
+    for r0 in range(0, n, step):
+        k = out[r0:r0 + step].to(torch.int64)
+        at = torch.arange(r0, r0 + k.numel(), device=dev)
+        assert torch.equal(_fmix64(k) & (P - 1), torch.bucketize(at, bounds, right=True))
+        row = k & 0xFFFFFFFF
+        assert int(row.max()) < n
+        last = out[r0 - 1:r0].to(torch.int64) & 0xFFFFFFFF if r0 else row[:0]
+        up = torch.cat([last, row])
+        down = torch.nonzero(up[1:] <= up[:-1]).view(-1) + r0 + (0 if r0 else 1)
+        assert bool(torch.isin(down, starts).all())
+    del out
+    torch.cuda.empty_cache()
