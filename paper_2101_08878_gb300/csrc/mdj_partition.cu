@@ -839,7 +839,7 @@ int stable_pass(Workspace &ws, const KeyT *keys, uint32_t n, const BucketSpec &b
   }
   const uint32_t pw = move_pay_width(cm);
   const uint32_t tile = stable_tile_rows(sizeof(KeyT), pw, rid_in != nullptr, F);
-  const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile - 1) / tile);
+  const uint32_t ntiles = tile_count(n, tile);
   uint32_t *hist = (uint32_t *)ws.get((size_t)F * ntiles * 4);
   if (!hist) return MDJ_ERR_OOM;
   launch_hist<KeyT>(keys, n, bs, F, tile, ntiles, hist, total2, nsub, s);
@@ -864,7 +864,7 @@ int reserve_pass(Workspace &ws, const KeyT *keys, uint32_t n, const BucketSpec &
                  uint32_t *cursors, const ColMove &cm, const uint32_t *rid_in, uint32_t *rid_out) {
   cudaStream_t s = ws.stream();
   MDJ_TRY(set_smem_attrs<KeyT>());
-  const uint32_t ntiles = (n + kTile - 1) / kTile;
+  const uint32_t ntiles = tile_count(n, kTile);
   if (ntiles == 0) return MDJ_OK;
   {
     TraceScope tr("scatter_reserve", s);
@@ -975,7 +975,7 @@ int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_
                  const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs &sg) {
   bool extra = false;
   for (ShSide &sd : sides.s) {
-    sd.ntiles = (uint32_t)(((uint64_t)sd.n + tile - 1) / tile);
+    sd.ntiles = tile_count(sd.n, tile);
     if (mode != SH_SEG) ntiles += sd.ntiles;
     extra = extra || (mode != SH_TERM && sd.cm.n > 2);
   }
@@ -1462,7 +1462,7 @@ int stable_partition_scratch_t(const mdj_table *t, int32_t key_col, uint32_t P, 
   // (tiles have at least kTile rows here, so the matrix fits the scratch words
   // counted for kTile-row tiles)
   const uint32_t tile = stable_tile_rows(sizeof(KeyT), pw, false, F);
-  const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile - 1) / tile);
+  const uint32_t ntiles = tile_count(n, tile);
   const size_t nhist = (size_t)F * ntiles;
   uint32_t *hist = scratch, *sums = hist + nhist;
   launch_hist<KeyT>(keys, n, bs, F, tile, ntiles, hist, nullptr, 0, s);

@@ -12,6 +12,11 @@
 
 namespace mdj {
 
+// Tiles (or chunks, or blocks) of `tile` rows that n rows take.  In 64 bits: n
+// + tile - 1 passes 2^32 for the last sizes of a table (nrows < 2^32), and the
+// quotient would be 0.
+MDJ_HD constexpr uint32_t tile_count(uint64_t n, uint32_t tile) { return (uint32_t)((n + tile - 1) / tile); }
+
 // Tile t of n < 2^32 rows in tiles of `tile` rows: its first row and its rows.
 // Kernels step over a tile with row numbers relative to row0: an absolute
 // 32-bit row number wraps when a step passes 2^32, and a loop bounded by the

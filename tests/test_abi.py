@@ -253,7 +253,7 @@ def test_tile_rows_up_to_the_largest_table(tmp_path):
   const unsigned rows[] = {1u, 4096u, 4097u, 6144u, 1u << 31, 4294963201u, 4294967295u - 4096u, 4294967295u};
   for (unsigned tile : tiles)
     for (unsigned n : rows) {
-      const unsigned m = (unsigned)(((unsigned long long)n + tile - 1) / tile);
+      const unsigned m = mdj::tile_count(n, tile);
       unsigned long long next = 0, most = 0;
       for (unsigned t = 0; t < m; t++) {
         const mdj::TileRows r = mdj::tile_rows(n, tile, t);
@@ -265,6 +265,22 @@ def test_tile_rows_up_to_the_largest_table(tmp_path):
     }
 ''')
     assert out == ["1"] * 32
+
+
+def test_tile_count_of_the_largest_table(tmp_path):
+    # n + tile - 1 passes 2^32 for tables of nearly 2^32 rows: in 32 bits the
+    # second pass of a stable two-level plan got no tiles above 2^32 - 4096
+    # rows, and returned with its output unwritten.
+    out = _run_sizes_program(tmp_path, '''
+  const unsigned rows[] = {0u, 1u, 4294963200u, 4294963201u, 4294967295u};
+  for (unsigned n : rows) printf("%u\\n", mdj::tile_count(n, 4096));
+''')
+    assert [int(v) for v in out] == [0, 1, 1048575, 1048576, 1048576]
+    # no tile count of the partition passes is computed another way (the
+    # scratch words, from a 64-bit row count, are)
+    with open(os.path.join(ROOT, "paper_2101_08878_gb300", "csrc", "mdj_partition.cu")) as f:
+        passes = f.read().split("size_t stable_partition_scratch_words")[0]
+    assert "kTile - 1)" not in passes and "tile - 1)" not in passes
 
 
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
