@@ -1384,7 +1384,7 @@ int partition_terms_t(Workspace &ws, const mdj_table *t, int32_t key_col, const 
   const int32_t pay_col = t->ncols < 2 ? -1 : (key_col == 0 ? 1 : 0);
   if (n) {
     TraceScope tr("count_terms", s);
-    k_terms<KeyT><<<(unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms() * 8), 256, 0, s>>>(
+    k_terms<KeyT><<<std::min(tile_count(n, 256), (uint32_t)num_sms() * 8), 256, 0, s>>>(
         (const KeyT *)t->cols[key_col].data, pay_col < 0 ? nullptr : t->cols[pay_col].data,
         pay_col < 0 ? 0 : dtype_width(t->cols[pay_col].dtype), n, term, terms);
   }

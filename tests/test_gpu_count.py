@@ -57,3 +57,27 @@ def test_terms_under_the_stable_passes(monkeypatch):
     rng = np.random.default_rng(4)
     lk, rk = rng.integers(0, 5000, 60_000), rng.integers(0, 5000, 50_000)
     _check([lk, datagen.uniform_payload(rng, lk.size)], [rk, datagen.uniform_payload(rng, rk.size)], 8)
+
+
+def test_largest_probe_side_of_an_unpartitioned_plan():
+    # 2^32 - 1 probe rows, the most a table may have; row i's key is i's bits,
+    # so a build key's one probe row is the key's own bits (-1 has none)
+    from paper_2101_08878_gb300 import mdj
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info(DEV)[0] < 80 << 30:
+        pytest.skip("needs 80 GB of device memory")
+    n, step = 2**32 - 1, 1 << 27
+    rk = torch.empty(n, dtype=torch.int32, device=DEV)
+    for r0 in range(0, n, step):
+        rk[r0:r0 + step] = torch.arange(r0, min(n, r0 + step), device=DEV)
+    rng = np.random.default_rng(9)
+    lk = np.concatenate([rng.integers(-2**31, 2**31, 3000), [-1, -2, 0, -1, 5, 5]]).astype(np.int32)
+    hit = lk != -1
+    rows = lk.view(np.uint32).astype(np.uint64)
+    f, _ = oracle.checksum_terms(lk, np.zeros(lk.size, np.uint64), np.zeros(1, np.uint64))
+    with np.errstate(over="ignore"):
+        g = oracle.fmix64(np.uint64(0xC2B2AE3D27D4EB4F) * (rows + np.uint64(1)))
+        want = int((f * g)[hit].sum(dtype=np.uint64))
+    assert mdj.mdj_count_checksum([torch.from_numpy(lk).to(DEV)], [rk], 1) == (int(hit.sum()), want)
+    del rk
+    torch.cuda.empty_cache()
