@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "mdj_internal.cuh"
+#include "mdj_sizes.h"
 
 namespace mdj {
 
@@ -288,9 +289,9 @@ __global__ void __launch_bounds__(kGT, 2)
     const LightUnit U = units[u];
     const uint32_t lb = L.off[U.b], nl = L.off[U.b + 1] - lb;
     if (nl == 0) {
-      for (uint32_t r = U.r0 + threadIdx.x; r < U.r0 + U.nr; r += kGT) {
-        o.cnt[r] = 0;
-        o.gbase[r] = 0;
+      for (uint32_t i = threadIdx.x; i < U.nr; i += kGT) {
+        o.cnt[U.r0 + i] = 0;
+        o.gbase[U.r0 + i] = 0;
       }
       continue;
     }
@@ -473,7 +474,8 @@ __global__ void __launch_bounds__(kHT)
   for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
     const HeavyUnit U = units[u];
     const HeavyDesc H = hd[U.h];
-    for (uint32_t i = U.i0 + threadIdx.x; i < U.i0 + U.n; i += kHT) {
+    for (uint32_t k = threadIdx.x; k < U.n; k += kHT) {
+      const uint32_t i = U.i0 + k;
       const uint32_t s = H.ts0 + hs[H.hr0 + i], rank = hrank[H.hr0 + i];
       const uint32_t pos = H.lb + (hbase[s] - H.hr0) + rank;
       const uint32_t src = H.lb + i;
@@ -493,7 +495,8 @@ __global__ void __launch_bounds__(kHT)
   for (uint32_t u = blockIdx.x; u < nunits; u += gridDim.x) {
     const HeavyUnit U = units[u];
     const HeavyDesc H = hd[U.h];
-    for (uint32_t r = U.i0 + threadIdx.x; r < U.i0 + U.n; r += kHT) {
+    for (uint32_t k = threadIdx.x; k < U.n; k += kHT) {
+      const uint32_t r = U.i0 + k;
       const KeyT kk = Rk[r];
       uint32_t s = big_home(key_bits(kk), H.tsz);
       bool found = false;
@@ -544,7 +547,7 @@ struct EntrySrc {
 };
 
 __device__ __forceinline__ void load8(const uint32_t *__restrict__ a, uint32_t n, uint32_t r0, uint32_t (&v)[kCRows]) {
-  if (r0 + kCRows <= n) {
+  if (r0 < n && n - r0 >= kCRows) {
     const uint4 x = *(const uint4 *)(a + r0), y = *(const uint4 *)(a + r0 + 4);
     v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w, v[4] = y.x, v[5] = y.y, v[6] = y.z, v[7] = y.w;
   } else {
@@ -878,23 +881,33 @@ void plan_units(const std::vector<uint32_t> &offL, const std::vector<uint32_t> &
     const uint32_t nl = offL[b + 1] - offL[b], nr = offR[b + 1] - offR[b];
     if (nr == 0 && !(keep_left && nl > 0)) continue;  // nothing of this sub-bucket is ever read
     if (nl == 0) {
-      for (uint32_t c0 = 0; c0 < nr; c0 += kProbeChunk)
-        u->first.push_back({b, offR[b] + c0, std::min(kProbeChunk, nr - c0), -1});
+      for (uint32_t c = 0, m = tile_count(nr, kProbeChunk); c < m; c++) {
+        const TileRows t = tile_rows(nr, kProbeChunk, c);
+        u->first.push_back({b, offR[b] + t.row0, t.rows, -1});
+      }
       continue;
     }
     if (nl <= kGCap) {  // nr may be 0 (keep_left): the unit groups and probes nothing
       const int32_t dump = nr > kProbeChunk ? (int32_t)u->ndump++ : -1;
       u->first.push_back({b, offR[b], std::min(kProbeChunk, nr), dump});
-      for (uint32_t c0 = kProbeChunk; c0 < nr; c0 += kProbeChunk)
-        u->later.push_back({b, offR[b] + c0, std::min(kProbeChunk, nr - c0), dump});
+      for (uint32_t c = 1, m = tile_count(nr, kProbeChunk); c < m; c++) {
+        const TileRows t = tile_rows(nr, kProbeChunk, c);
+        u->later.push_back({b, offR[b] + t.row0, t.rows, dump});
+      }
       continue;
     }
     const uint32_t h = (uint32_t)u->heavy.size();
     u->heavy.push_back({b, offL[b], nl, 2 * nl, (uint32_t)u->hslots, (uint32_t)u->hrows});
     u->hslots += 2ull * nl;
     u->hrows += nl;
-    for (uint32_t i0 = 0; i0 < nl; i0 += kHChunk) u->hbuild.push_back({h, i0, std::min(kHChunk, nl - i0)});
-    for (uint32_t c0 = 0; c0 < nr; c0 += kHChunk) u->hprobe.push_back({h, offR[b] + c0, std::min(kHChunk, nr - c0)});
+    for (uint32_t c = 0, m = tile_count(nl, kHChunk); c < m; c++) {
+      const TileRows t = tile_rows(nl, kHChunk, c);
+      u->hbuild.push_back({h, t.row0, t.rows});
+    }
+    for (uint32_t c = 0, m = tile_count(nr, kHChunk); c < m; c++) {
+      const TileRows t = tile_rows(nr, kHChunk, c);
+      u->hprobe.push_back({h, offR[b] + t.row0, t.rows});
+    }
   }
   // much larger probe chunks than the mean first, so the persistent blocks
   // finish together (a full sort by size kept the GPU waiting)

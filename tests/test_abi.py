@@ -283,6 +283,22 @@ def test_tile_count_of_the_largest_table(tmp_path):
     assert "kTile - 1)" not in passes and "tile - 1)" not in passes
 
 
+def test_probe_chunks_of_the_largest_table(tmp_path):
+    # the grouping's units (65536 and 8192 rows) cover a sub-bucket of nearly
+    # 2^32 rows: a 32-bit loop over their first rows wrapped and never ended
+    out = _run_sizes_program(tmp_path, '''
+  for (unsigned chunk : {65536u, 8192u})
+    for (unsigned n : {0u, 1u, 65536u, 4294901761u, 4294967295u}) {
+      unsigned long long sum = 0;
+      const unsigned m = mdj::tile_count(n, chunk);
+      for (unsigned c = 0; c < m; c++) sum += mdj::tile_rows(n, chunk, c).rows;
+      printf("%u %d\\n", m, sum == n && (m == 0 || mdj::tile_rows(n, chunk, m - 1).row0 < n));
+    }
+''')
+    assert [int(v) for v in out[::2]] == [0, 1, 1, 65536, 65536, 0, 1, 8, 524281, 524288]
+    assert out[1::2] == ["1"] * 10
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and

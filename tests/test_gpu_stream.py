@@ -342,3 +342,35 @@ def test_stream_tiny_tables_and_more_partitions_than_rows(nl, nr, P):
     right = [rk, np.arange(nr, dtype=np.float64)]
     for how in ("inner", "outer"):
         _check(left, right, P, window=1, how=how)
+
+
+def _largest_right(n):
+    """A right table of n rows whose row i has the key i's bits, in bounded steps."""
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info(DEV)[0] < 180 << 30:
+        pytest.skip("needs 180 GB of device memory")
+    step = 1 << 27
+    rk = torch.empty(n, dtype=torch.int32, device=DEV)
+    for r0 in range(0, n, step):
+        rk[r0:r0 + step] = torch.arange(r0, min(n, r0 + step), device=DEV)
+    return rk
+
+
+def test_largest_probe_side_inner():
+    # 2^32 - 1 right rows, the most a table may have, in one sub-bucket; the
+    # left keys -1 have no right row, 5 has three left rows
+    mdj = _mdj()
+    n = 2**32 - 1
+    rk = _largest_right(n)
+    rng = np.random.default_rng(9)
+    lk = np.concatenate([rng.integers(-2**31, 2**31, 2000), [-1, -2, 0, -1, 5, 5, 5]]).astype(np.int32)
+    with mdj.MergeStream([torch.from_numpy(lk).to(DEV)], [rk], 1) as st:
+        res = st.emit(0, st.total_rows, st.buffers(st.total_rows))
+        got = [t.cpu().numpy() for t in (res.key, res.left_row.view(torch.int32), res.right_row.view(torch.int32))]
+    lrow = np.flatnonzero(lk != -1).astype(np.int32)
+    want = [lk[lrow], lrow, lk[lrow]]
+    order = [np.lexsort((c[1], c[0])) for c in (got, want)]
+    for g, w in zip(got, want):
+        assert np.array_equal(g[order[0]], w[order[1]])
+    del rk, st, res
+    torch.cuda.empty_cache()
