@@ -56,7 +56,7 @@ struct EmitSrc {
   const uint64_t *moff;  // [nm + 1], moff[nm] = total rows
   const uint32_t *mr;    // [nm] shuffled probe row
   const uint32_t *mg;    // [nm] first grouped build position of its group
-  uint32_t nm;
+  uint64_t nm;           // outer joins: up to n_L + n_R
   const void *rkey;
   const uint32_t *rrid;  // NULL: identity
   const void *rcols[MDJ_MAX_COLS];
@@ -585,7 +585,7 @@ __device__ __forceinline__ uint64_t packed_sum(const uint32_t (&v)[kCRows]) {
 
 // chunk c: rows[c], ents[c] (nchunks + 1 entries each; the last stays 0)
 __global__ void __launch_bounds__(kCT)
-    k_entry_sums(EntrySrc S, uint64_t *__restrict__ rows, uint32_t *__restrict__ ents) {
+    k_entry_sums(EntrySrc S, uint64_t *__restrict__ rows, uint64_t *__restrict__ ents) {
   __shared__ uint64_t scratch[33];
   const uint32_t r0 = blockIdx.x * kCChunk + threadIdx.x * kCRows;
   uint32_t v[kCRows];
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kCT)
   block_exclusive_scan<uint64_t>(packed_sum(v), scratch, &tot);
   if (threadIdx.x == 0) {
     rows[blockIdx.x] = tot >> 13;
-    ents[blockIdx.x] = (uint32_t)(tot & 8191);
+    ents[blockIdx.x] = tot & 8191;
   }
 }
 
@@ -602,8 +602,8 @@ __global__ void __launch_bounds__(kCT)
 // starts (pass 1's totals, or NULL for 0).  The chunk's entries are staged in
 // shared memory one array at a time and leave with coalesced stores.
 __global__ void __launch_bounds__(kCT)
-    k_entry_write(EntrySrc S, const uint64_t *__restrict__ rows, const uint32_t *__restrict__ ents,
-                  const uint64_t *__restrict__ rows0, const uint32_t *__restrict__ ents0, uint64_t *__restrict__ moff,
+    k_entry_write(EntrySrc S, const uint64_t *__restrict__ rows, const uint64_t *__restrict__ ents,
+                  const uint64_t *__restrict__ rows0, const uint64_t *__restrict__ ents0, uint64_t *__restrict__ moff,
                   uint32_t *__restrict__ mr, uint32_t *__restrict__ mg) {
   __shared__ uint64_t scratch[33];
   __shared__ uint64_t stage[kCChunk];
@@ -621,7 +621,9 @@ __global__ void __launch_bounds__(kCT)
   uint64_t tot;
   const uint64_t ex = block_exclusive_scan<uint64_t>(packed_sum(v), scratch, &tot);
   const uint64_t rbase = rows[blockIdx.x] + (rows0 ? *rows0 : 0ull);
-  const uint32_t ebase = ents[blockIdx.x] + (ents0 ? *ents0 : 0u), n = (uint32_t)(tot & 8191);
+  const uint64_t ebase = ents[blockIdx.x] + (ents0 ? *ents0 : 0ull);
+  moff += ebase, mr += ebase, mg += ebase;
+  const uint32_t n = (uint32_t)(tot & 8191);
   const uint32_t e0 = (uint32_t)(ex & 8191);
   {
     uint64_t at = rbase + (ex >> 13);
@@ -634,7 +636,7 @@ __global__ void __launch_bounds__(kCT)
       }
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < n; i += kCT) moff[ebase + i] = stage[i];
+  for (uint32_t i = threadIdx.x; i < n; i += kCT) moff[i] = stage[i];
   __syncthreads();
   {
     uint32_t e = e0;
@@ -643,7 +645,7 @@ __global__ void __launch_bounds__(kCT)
       if (v[k]) stage32[e++] = r[k];
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < n; i += kCT) mr[ebase + i] = stage32[i];
+  for (uint32_t i = threadIdx.x; i < n; i += kCT) mr[i] = stage32[i];
   __syncthreads();
   {
     uint32_t e = e0;
@@ -652,14 +654,14 @@ __global__ void __launch_bounds__(kCT)
       if (v[k]) stage32[e++] = g[k];
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < n; i += kCT) mg[ebase + i] = stage32[i];
+  for (uint32_t i = threadIdx.x; i < n; i += kCT) mg[i] = stage32[i];
 }
 
 // out = {total rows, entries, error}; moff[entries] = total rows.
-__global__ void k_stream_totals(const uint64_t *r1, const uint32_t *e1, const uint64_t *r2, const uint32_t *e2,
+__global__ void k_stream_totals(const uint64_t *r1, const uint64_t *e1, const uint64_t *r2, const uint64_t *e2,
                                 const int *err, uint64_t *__restrict__ moff, unsigned long long *__restrict__ out) {
   const uint64_t total = *r1 + (r2 ? *r2 : 0ull);
-  const uint32_t nm = *e1 + (e2 ? *e2 : 0u);
+  const uint64_t nm = *e1 + (e2 ? *e2 : 0ull);
   out[0] = total;
   out[1] = nm;
   out[2] = err[0] != 0;
@@ -730,7 +732,7 @@ __global__ void __launch_bounds__(kET, kEBlocks)
   // entry j of the tile: its first row in the tile (0 for the one that began
   // before it), probe row, group position of that row
   __shared__ uint32_t s_off[kETile + 1], s_r[kETile + 1], s_g[kETile + 1];
-  __shared__ uint32_t s_e;
+  __shared__ uint64_t s_e;
   const uint64_t ntiles = (rows + kETile - 1) / kETile;
   const uint64_t t_begin = (uint64_t)blockIdx.x * tiles_per_block;
   if (t_begin >= ntiles) return;
@@ -739,16 +741,14 @@ __global__ void __launch_bounds__(kET, kEBlocks)
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 32) {
     const uint64_t o = first + t_begin * kETile;
-    uint32_t lo = 0, hi = S.nm;  // moff[lo] <= o < moff[hi]
+    uint64_t lo = 0, hi = S.nm;  // moff[lo] <= o < moff[hi]
     while (hi - lo > 1) {
-      const uint32_t step = (hi - lo + 31) / 32;
-      const uint64_t p = (uint64_t)lo + (uint64_t)(lane + 1) * step;
+      const uint64_t step = (hi - lo + 31) / 32;
+      const uint64_t p = lo + (uint64_t)(lane + 1) * step;
       const bool le = p < hi && S.moff[p] <= o;
       const uint32_t c = __popc(__ballot_sync(0xffffffffu, le));
-      const uint32_t nlo = lo + c * step;
-      const uint64_t nhi = (uint64_t)lo + (uint64_t)(c + 1) * step;
-      lo = nlo;
-      hi = nhi < hi ? (uint32_t)nhi : hi;
+      hi = min(hi, lo + (uint64_t)(c + 1) * step);
+      lo += (uint64_t)c * step;
     }
     if (lane == 0) s_e = lo;
   }
@@ -756,8 +756,8 @@ __global__ void __launch_bounds__(kET, kEBlocks)
   for (uint64_t t = t_begin; t < t_end; t++) {
     const uint64_t o0 = first + t * kETile;
     const uint32_t n = (uint32_t)min((uint64_t)kETile, last - o0);  // rows of the tile
-    const uint32_t e = s_e;
-    const uint32_t ne = min((uint32_t)(kETile + 1), S.nm + 1 - e);
+    const uint64_t e = s_e;
+    const uint32_t ne = (uint32_t)min((uint64_t)(kETile + 1), S.nm + 1 - e);
     for (uint32_t j = threadIdx.x; j < ne; j += kET) {
       const uint64_t off = S.moff[e + j];
       const uint32_t into = j == 0 ? (uint32_t)(o0 - off) : 0u;  // rows of entry 0 before the tile (below its group's size)
@@ -938,22 +938,22 @@ unsigned grid_for(uint64_t units, int per_sm) {
 // One pass of the entries: sums per chunk, scan, rescan and write.  rows0 /
 // ents0: where the pass starts (NULL: 0).  Leaves the pass's totals at
 // crows[nchunks], cents[nchunks].
-int entries_pass(Workspace &tmp, const EntrySrc &src, const uint64_t *rows0, const uint32_t *ents0, uint64_t *moff,
-                 uint32_t *mr, uint32_t *mg, uint64_t **crows_out, uint32_t **cents_out, uint32_t *nchunks_out) {
+int entries_pass(Workspace &tmp, const EntrySrc &src, const uint64_t *rows0, const uint64_t *ents0, uint64_t *moff,
+                 uint32_t *mr, uint32_t *mg, uint64_t **crows_out, uint64_t **cents_out, uint32_t *nchunks_out) {
   cudaStream_t s = tmp.stream();
   const uint32_t nchunks = (uint32_t)(((size_t)src.n + kCChunk - 1) / kCChunk);
   uint64_t *crows = (uint64_t *)tmp.get((size_t)(nchunks + 1) * 8);
-  uint32_t *cents = (uint32_t *)tmp.get((size_t)(nchunks + 1) * 4);
+  uint64_t *cents = (uint64_t *)tmp.get((size_t)(nchunks + 1) * 8);
   if (!crows || !cents) return MDJ_ERR_OOM;
   MDJ_CUDA_TRY(cudaMemsetAsync(crows + nchunks, 0, 8, s));
-  MDJ_CUDA_TRY(cudaMemsetAsync(cents + nchunks, 0, 4, s));
+  MDJ_CUDA_TRY(cudaMemsetAsync(cents + nchunks, 0, 8, s));
   if (nchunks) {
     TraceScope tr("stream_entry_sums", s);
     k_entry_sums<<<nchunks, kCT, 0, s>>>(src, crows, cents);
   }
   MDJ_LAUNCH_CHECK();
   MDJ_TRY(exclusive_scan_u64(tmp, crows, crows, (size_t)nchunks + 1));
-  MDJ_TRY(exclusive_scan_u32(tmp, cents, cents, (size_t)nchunks + 1));
+  MDJ_TRY(exclusive_scan_u64(tmp, cents, cents, (size_t)nchunks + 1));
   if (nchunks) {
     TraceScope tr("stream_entries", s);
     k_entry_write<<<nchunks, kCT, 0, s>>>(src, crows, cents, rows0, ents0, moff, mr, mg);
@@ -1088,7 +1088,8 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
   if (!moff || !mr || !mg) return MDJ_ERR_OOM;
   const EntrySrc probe_src = {o.cnt, o.gbase, nR, keep_right ? SRC_PROBE_ALL : SRC_PROBE};
   uint64_t *crows1, *crows2 = nullptr;
-  uint32_t *cents1, *cents2 = nullptr, c1, c2 = 0;
+  uint64_t *cents1, *cents2 = nullptr;
+  uint32_t c1, c2 = 0;
   MDJ_TRY(entries_pass(tmp, probe_src, nullptr, nullptr, moff, mr, mg, &crows1, &cents1, &c1));
   if (keep_left) {
     const EntrySrc group_src = {o.gsize, o.hit, nL, SRC_UNMATCHED_GROUPS};
@@ -1107,12 +1108,11 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
   MDJ_CUDA_TRY(cudaStreamSynchronize(s));
   if (host[2]) return MDJ_ERR_INTERNAL;
   const uint64_t total = host[0];
-  const uint32_t nm = (uint32_t)host[1];
   h->total = total;
   S.moff = moff;
   S.mr = mr;
   S.mg = mg;
-  S.nm = nm;
+  S.nm = host[1];
   S.rkey = R.key;
   S.rrid = R.rid;
   S.nrc = R.ncols;

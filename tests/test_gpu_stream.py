@@ -374,3 +374,37 @@ def test_largest_probe_side_inner():
         assert np.array_equal(g[order[0]], w[order[1]])
     del rk, st, res
     torch.cuda.empty_cache()
+
+
+def test_entries_numbered_up_to_the_largest_right_side():
+    # a right join of 2^32 - 1 right rows has as many entries: entry numbers
+    # and their count + 1 pass 32 bits
+    mdj = _mdj()
+    n = 2**32 - 1
+    rk = _largest_right(n)
+    lk = np.array([5, 5, 5, 70, -1, 2**31 - 1, -7, -7, -2], np.int32)
+    total = n + 2 + 1
+    with mdj.MergeStream([torch.from_numpy(lk).to(DEV)], [rk], 1, how="right") as st:
+        assert st.total_rows == total
+        buf = st.buffers(6000)
+        for first, rows in [(0, 5000), (2**31 - 2999, 6000), (total - 5001, 5001)]:
+            # right rows in input order, each with every left row of its key
+            row = np.arange(max(0, first - 4), min(n, first + rows + 4), dtype=np.int64)
+            copies = np.where((row == 5), 3, np.where(row == 2**32 - 7, 2, 1))
+            at = row + 2 * (row > 5) + (row > 2**32 - 7)  # first output row of a right row
+            rrow = np.repeat(row, copies)
+            pos = np.repeat(at, copies) + np.concatenate([np.arange(c) for c in copies])
+            rrow = rrow[(pos >= first) & (pos < first + rows)]
+            res = st.emit(first, rows, buf)
+            bits = rrow.astype(np.uint32).view(np.int32)
+            assert np.array_equal(res.right_row.view(torch.int32).cpu().numpy(), bits)
+            assert np.array_equal(res.key.cpu().numpy(), bits)
+            lrow = res.left_row.view(torch.int32).cpu().numpy()
+            none = ~np.isin(bits, lk)
+            assert (lrow[none] == -1).all()
+            assert np.array_equal(lk[lrow[~none]], bits[~none])
+            for k in (5, -7):  # a key's left rows, each once
+                have = np.sort(lrow[bits == k])
+                assert have.size in (0, (lk == k).sum()) and np.array_equal(have, np.flatnonzero(lk == k)[:have.size])
+    del rk, st, buf, res
+    torch.cuda.empty_cache()
