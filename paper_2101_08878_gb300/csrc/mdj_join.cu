@@ -42,8 +42,7 @@ __global__ void k_items(const uint32_t *__restrict__ offL, const uint32_t *__res
                         uint32_t rch, uint64_t *__restrict__ items, unsigned long long *__restrict__ tail) {
   uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < nb) {
-    uint64_t nl = offL[b + 1] - offL[b], nr = offR[b + 1] - offR[b];
-    items[b] = (nl && nr) ? ((nl + cap - 1) / cap) * ((nr + rch - 1) / rch) : 0ull;
+    items[b] = (uint64_t)chunk_count(offL[b + 1] - offL[b], cap) * chunk_count(offR[b + 1] - offR[b], rch);
   } else if (b == nb) {
     items[nb] = 0;
     for (int w = 0; w < 5; w++) tail[w] = 0;
@@ -73,7 +72,7 @@ __global__ void k_expand(const uint32_t *__restrict__ offL, const uint32_t *__re
     }
     const uint32_t local = (uint32_t)(it - item_off[lo]);
     const uint32_t nl = offL[lo + 1] - offL[lo], nr = offR[lo + 1] - offR[lo];
-    const uint32_t nrc = (nr + rch - 1) / rch;
+    const uint32_t nrc = chunk_count(nr, rch);
     const uint32_t lc = local / nrc, rc = local % nrc;
     Item d;
     d.lbeg = offL[lo] + lc * cap;
@@ -105,7 +104,7 @@ __global__ void __launch_bounds__(kPlanThreads)
   uint32_t sum;
   const uint32_t l = block_exclusive_scan<uint32_t>(cl, scratch, &sum);
   const uint32_t r = block_exclusive_scan<uint32_t>(cr, scratch, &sum);
-  const uint64_t mine = cl && cr ? (uint64_t)((cl - 1) / cap + 1) * ((cr - 1) / rch + 1) : 0ull;
+  const uint64_t mine = (uint64_t)chunk_count(cl, cap) * chunk_count(cr, rch);
   uint64_t total;
   const uint64_t at = block_exclusive_scan<uint64_t>(mine, scratch64, &total);
   if (b < nb) {
@@ -135,7 +134,7 @@ __global__ void __launch_bounds__(kPlanThreads)
       else
         hi = mid - 1;
     }
-    const uint32_t nl = s_l[lo + 1] - s_l[lo], nr = s_r[lo + 1] - s_r[lo], nrc = (nr - 1) / rch + 1;
+    const uint32_t nl = s_l[lo + 1] - s_l[lo], nr = s_r[lo + 1] - s_r[lo], nrc = chunk_count(nr, rch);
     const uint32_t lc = (it - s_item[lo]) / nrc, rc = (it - s_item[lo]) % nrc;
     Item d;
     d.lbeg = s_l[lo] + lc * cap;

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "mdj_internal.cuh"
+#include "mdj_sizes.h"
 
 namespace mdj {
 namespace {

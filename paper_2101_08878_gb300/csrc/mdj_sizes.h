@@ -33,4 +33,7 @@ MDJ_HD constexpr TileRows tile_rows(uint32_t n, uint32_t tile, uint32_t t) {
 // fit the position type, so 32-bit positions serve only while m + 1 <= 2^32 - 1.
 inline constexpr bool compaction_needs_u64_positions(uint64_t m) { return m + 1 > 0xFFFFFFFFull; }
 
+// Chunks of `chunk` rows that n < 2^32 rows take, in 32 bits (device code).
+MDJ_HD constexpr uint32_t chunk_count(uint32_t n, uint32_t chunk) { return n ? (n - 1) / chunk + 1 : 0u; }
+
 }  // namespace mdj

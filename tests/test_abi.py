@@ -299,6 +299,15 @@ def test_probe_chunks_of_the_largest_table(tmp_path):
     assert out[1::2] == ["1"] * 10
 
 
+def test_join_items_of_the_largest_table(tmp_path):
+    # a bucket of nearly 2^32 probe rows: n + 4095 wrapped, the item's chunk
+    # number was divided by 0 chunks and its row ranges were arbitrary
+    out = _run_sizes_program(tmp_path, '''
+  for (unsigned n : {0u, 1u, 4096u, 4097u, 4294963200u, 4294963201u, 4294967295u}) printf("%u\\n", mdj::chunk_count(n, 4096));
+''')
+    assert [int(v) for v in out] == [0, 1, 1, 2, 1048575, 1048576, 1048576]
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and

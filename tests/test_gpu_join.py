@@ -252,3 +252,30 @@ def test_merge_host_end_to_end():
     a = torch.sort((out.key << 32) | out.right_row.view(torch.int32).to(torch.int64)).values
     b = torch.sort(((dev.key << 32) | dev.right_row.view(torch.int32).to(torch.int64)).cpu()).values
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("ordered", ["0", "1"])
+def test_largest_probe_side(ordered, monkeypatch):
+    # 2^32 - 1 probe rows (row i's key is i's bits), the most a table may
+    # have, in one bucket: 2^20 work items of one build chunk
+    from paper_2101_08878_gb300 import mdj
+    dev = torch.device("cuda", 0)
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info(dev)[0] < 120 << 30:
+        pytest.skip("needs 120 GB of device memory")
+    monkeypatch.setenv("MDJ_ORDERED_OUTPUT", ordered)
+    n, step = 2**32 - 1, 1 << 27
+    rk = torch.empty(n, dtype=torch.int32, device=dev)
+    for r0 in range(0, n, step):
+        rk[r0:r0 + step] = torch.arange(r0, min(n, r0 + step), device=dev)
+    rng = np.random.default_rng(9)
+    lk = np.concatenate([rng.integers(-2**31, 2**31, 2000), [-1, -2, 0, -1, 5, 5, 5]]).astype(np.int32)
+    res = mdj.mdj_merge([torch.from_numpy(lk).to(dev)], [rk], 1)
+    got = [t.cpu().numpy() for t in (res.key, res.left_row.view(torch.int32), res.right_row.view(torch.int32))]
+    lrow = np.flatnonzero(lk != -1).astype(np.int32)
+    want = [lk[lrow], lrow, lk[lrow]]
+    order = [np.lexsort((c[1], c[0])) for c in (got, want)]
+    for g, w in zip(got, want):
+        assert np.array_equal(g[order[0]], w[order[1]])
+    del rk, res
+    torch.cuda.empty_cache()
