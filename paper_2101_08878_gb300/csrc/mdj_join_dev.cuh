@@ -208,24 +208,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst_smem, const void *src_gmem, u
       : "memory");
 }
 
-// Elements [beg, beg + n) of a column of `es`-byte elements whose base is
-// 16-byte aligned: the 16-byte-aligned interior [a, b) goes by one bulk copy,
-// the head [beg, a) and tail [b, beg + n) by ordinary loads.  In shared
-// memory element beg + i sits at index sh + i of the staging buffer, sh =
-// beg mod (16 / es), so the interior starts on a 16-byte boundary.
-struct BulkPart {
-  uint32_t sh, a, b;
-};
-__device__ __forceinline__ BulkPart bulk_part(uint32_t beg, uint32_t n, uint32_t es) {
-  const uint32_t per = 16 / es;
-  BulkPart p;
-  p.sh = beg % per;
-  p.a = (beg + per - 1) / per * per;
-  p.b = (beg + n) / per * per;
-  if (p.b <= p.a) p.a = p.b = beg + n;  // no aligned interior: all by ordinary loads
-  return p;
-}
-
 // Non-key columns after the first of each side (gathered from global memory).
 __device__ __forceinline__ void copy_extra_cols(const JSide &L, const JSide &R, const JOut &out, uint64_t pos,
                                                 uint32_t lrow, uint32_t r) {

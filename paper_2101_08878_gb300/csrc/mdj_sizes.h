@@ -36,4 +36,19 @@ inline constexpr bool compaction_needs_u64_positions(uint64_t m) { return m + 1 
 // Chunks of `chunk` rows that n < 2^32 rows take, in 32 bits (device code).
 MDJ_HD constexpr uint32_t chunk_count(uint32_t n, uint32_t chunk) { return n ? (n - 1) / chunk + 1 : 0u; }
 
+// Elements [beg, beg + n) of a column of `es`-byte elements whose base is
+// 16-byte aligned: the 16-byte-aligned interior [a, b) goes by one bulk copy,
+// the head [beg, a) and tail [b, beg + n) by ordinary loads.  In shared
+// memory element beg + i sits at index sh + i of the staging buffer, sh =
+// beg mod (16 / es), so the interior starts on a 16-byte boundary.  beg rounded
+// up may be 2^32, which wraps to 0: there is no interior then.
+struct BulkPart {
+  uint32_t sh, a, b;
+};
+MDJ_HD constexpr BulkPart bulk_part(uint32_t beg, uint32_t n, uint32_t es) {
+  const uint32_t per = 16 / es, a = (beg + per - 1) / per * per, b = (beg + n) / per * per;
+  if (a < beg || b <= a) return {beg % per, beg + n, beg + n};  // no aligned interior: all by ordinary loads
+  return {beg % per, a, b};
+}
+
 }  // namespace mdj

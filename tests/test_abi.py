@@ -308,6 +308,25 @@ def test_join_items_of_the_largest_table(tmp_path):
     assert [int(v) for v in out] == [0, 1, 1, 2, 1048575, 1048576, 1048576]
 
 
+def test_bulk_part_covers_every_chunk(tmp_path):
+    # the bulk copy's aligned interior against its definition, to the last row
+    # a table may have, where the rounded-up start is 2^32
+    out = _run_sizes_program(tmp_path, '''
+  unsigned long long bad = 0;
+  for (unsigned es : {4u, 8u})
+    for (unsigned n = 1; n <= 24; n++)
+      for (unsigned k = 0; k < 64; k++) {
+        const unsigned long long per = 16 / es, beg = k < 32 ? k : 4294967295ull - n - (k - 32);
+        const mdj::BulkPart p = mdj::bulk_part((unsigned)beg, n, es);
+        unsigned long long a = (beg + per - 1) / per * per, b = (beg + n) / per * per;
+        if (b <= a) a = b = beg + n;
+        bad += p.sh != beg % per || p.a != a || p.b != b;
+      }
+  printf("%llu\\n", bad);
+''')
+    assert out == ["0"]
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and
