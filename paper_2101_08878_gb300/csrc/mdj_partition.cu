@@ -1309,16 +1309,10 @@ Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition,
     return pl;
   }
   const uint32_t fan = stable_passes ? kStableFanout : kMergeFanout;
-  uint32_t S1 = fan / P;
-  if (S1 < 1) S1 = 1;
-  uint64_t F2 = (S + S1 - 1) / S1;
-  uint64_t max_f2 = kMaxSubBuckets / ((uint64_t)P * S1);
-  if (F2 > max_f2) F2 = max_f2;  // larger inputs: sub-buckets split into several tables
-  if (F2 > kPass2SpanMax / 2) F2 = kPass2SpanMax / 2;
-  if (F2 < 1) F2 = 1;
-  pl.F2 = (uint32_t)F2;
-  pl.S = S1 * pl.F2;
-  pl.F1 = P * S1;
+  const TwoPassSplit sp = two_pass_split(P, S, fan, kMaxSubBuckets, kPass2SpanMax / 2);
+  pl.F2 = sp.F2;
+  pl.S = sp.S1 * sp.F2;
+  pl.F1 = P * sp.S1;
   pl.nbuckets = P * pl.S;
   return pl;
 }

@@ -327,6 +327,29 @@ def test_bulk_part_covers_every_chunk(tmp_path):
     assert out == ["0"]
 
 
+def test_two_pass_plans_keep_their_buckets(tmp_path):
+    # 1e8 to 1.7e8 build rows in P partitions, tables of 4096 rows filled to
+    # 85%: with 128 pass-1 buckets a plan has all the sub-buckets it needs, or
+    # as many as one with 256 pass-1 buckets.  Above (2.5e8), where 49152 are
+    # not enough, it has all of them but the rest of a division by P * S1.
+    out = _run_sizes_program(tmp_path, '''
+  unsigned long long bad = 0, raised = 0;
+  for (unsigned P = 1; P <= 1024; P++)
+    for (unsigned long long n = 100000000; n <= 250000000; n += 5000000) {
+      const unsigned long long need = (n + 3480) / 3481, S = (need + P - 1) / P;
+      if (P * S <= 1024) continue;
+      const mdj::TwoPassSplit a = mdj::two_pass_split(P, S, 128, 49152, 512);
+      const mdj::TwoPassSplit b = mdj::two_pass_split(P, S, 256, 49152, 512);
+      const unsigned long long na = 1ull * P * a.S1 * a.F2, nb = 1ull * P * b.S1 * b.F2;
+      if (n <= 170000000 ? na < std::min(need, nb) : na < std::min(need, 49153ull - P * a.S1)) bad++;
+      if (na > 49152 || a.F2 > 512 || P * a.S1 > 1024) bad++;
+      if (P <= 128 && a.S1 > 128 / P) raised++;
+    }
+  printf("%llu %d\\n", bad, raised > 0);
+''')
+    assert out == ["0", "1"]
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and

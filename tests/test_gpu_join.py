@@ -279,3 +279,28 @@ def test_largest_probe_side(ordered, monkeypatch):
         assert np.array_equal(g[order[0]], w[order[1]])
     del rk, res
     torch.cuda.empty_cache()
+
+
+def test_build_side_of_more_than_512_sub_buckets_per_partition():
+    # 65 partitions of 531 sub-buckets: two pass-1 buckets each.  Unique left
+    # keys, so every matching right row has one left row.
+    mdj = _mdj()
+    torch.cuda.empty_cache()
+    n_l, n_r = 120_000_000, 3_000_001
+    g = torch.Generator(device=DEV)
+    g.manual_seed(6)
+    lk = torch.randperm(n_l, generator=g, device=DEV, dtype=torch.int32)
+    rk = torch.randint(-n_l, 2 * n_l, (n_r,), generator=g, device=DEV, dtype=torch.int32)
+    rows = torch.nonzero((rk >= 0) & (rk < n_l)).view(-1)
+    place = torch.empty(n_l, dtype=torch.int32, device=DEV)
+    place[lk.long()] = torch.arange(n_l, dtype=torch.int32, device=DEV)
+    res = mdj.mdj_merge([lk], [rk], 65)
+    at = res.right_row.view(torch.int32).long()
+    order = torch.argsort(at)
+    assert torch.equal(at[order], rows)
+    assert torch.equal(res.key[order], rk[rows])
+    assert torch.equal(res.left_row.view(torch.int32)[order], place[rk[rows].long()])
+    counts = [mdj.mdj_count_checksum([lk], [rk], P) for P in (64, 65)]
+    assert counts[0] == counts[1] and counts[0][0] == rows.numel()
+    with mdj.MergeStream([lk], [rk], 65) as st:
+        assert st.total_rows == rows.numel()
