@@ -1012,8 +1012,8 @@ int count_rows(Workspace &ws, TotSide A, TotSide B, const BucketSpec &bs, uint32
   if (ca + cb == 0) return MDJ_OK;
   A.blocks = (uint32_t)ca;
   B.blocks = (uint32_t)cb;
-  if (ca + cb > full) {  // resident blocks, split by rows
-    A.blocks = cb ? (uint32_t)std::min(full - 1, std::max<uint64_t>(ca ? 1 : 0, full * ca / (ca + cb))) : (uint32_t)full;
+  if (ca + cb > full) {  // resident blocks
+    A.blocks = side_blocks(full, ca, cb);
     B.blocks = (uint32_t)full - A.blocks;
   }
   TraceScope tr("hist", ws.stream());

@@ -75,4 +75,19 @@ inline constexpr TwoPassSplit two_pass_split(uint32_t P, uint64_t S, uint32_t fa
   return {(uint32_t)S1, (uint32_t)F2};
 }
 
+// Side A's share of `full` blocks that two sides of ca and cb equal chunks
+// split: the whole number that lets the longer side end first.  Rounding down
+// alone left a small side's one block half as many chunks again as the others (1e6 +
+// 1e8 keys counted by 152 blocks: 0.186 ms, with it 0.131).
+inline constexpr uint32_t side_blocks(uint64_t full, uint64_t ca, uint64_t cb) {
+  if (ca == 0 || cb == 0) return (uint32_t)(cb == 0 ? full : 0);
+  uint64_t a = full * ca / (ca + cb), best = 0, time = 0;
+  for (uint64_t x = a; x <= a + 1; x++) {
+    const uint64_t n = x < 1 ? 1 : x > full - 1 ? full - 1 : x;
+    const uint64_t ta = (ca + n - 1) / n, tb = (cb + full - n - 1) / (full - n), t = ta > tb ? ta : tb;
+    if (best == 0 || t < time) best = n, time = t;
+  }
+  return (uint32_t)best;
+}
+
 }  // namespace mdj

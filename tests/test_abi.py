@@ -350,6 +350,28 @@ def test_two_pass_plans_keep_their_buckets(tmp_path):
     assert out == ["0", "1"]
 
 
+def test_count_blocks_split_between_two_sides(tmp_path):
+    # the longer side takes no more chunks per block than with any other
+    # split, also where one side is much the smaller
+    out = _run_sizes_program(tmp_path, '''
+  unsigned long long bad = 0;
+  for (unsigned long long full : {2ull, 152ull, 304ull})
+    for (unsigned long long ca : {0ull, 1ull, 2ull, 50ull, 123ull, 184ull, 2442ull, 12208ull, 524288ull})
+      for (unsigned long long cb : {0ull, 1ull, 3ull, 123ull, 12208ull, 30518ull}) {
+        if (ca + cb <= full) continue;
+        const unsigned long long a = mdj::side_blocks(full, ca, cb);
+        if (ca == 0 || cb == 0) { bad += a != (cb ? 0 : full); continue; }
+        if (a < 1 || a >= full) { bad++; continue; }
+        auto time = [&](unsigned long long x) { return std::max((ca + x - 1) / x, (cb + full - x - 1) / (full - x)); };
+        unsigned long long best = ~0ull;
+        for (unsigned long long x = 1; x < full; x++) best = std::min(best, time(x));
+        bad += time(a) > best;
+      }
+  printf("%llu\\n", bad);
+''')
+    assert out == ["0"]
+
+
 def test_workspace_give_back_keeps_arena_chunks(tmp_path):
     # Workspace (the library's per-call device memory) carves small buffers out
     # of arena chunks; the first buffer of a chunk has the chunk's address, and
