@@ -90,13 +90,18 @@ __global__ void k_expand(const uint32_t *__restrict__ offL, const uint32_t *__re
 // launches of the general path (two scans, two cursor kernels, items, their
 // scan, descriptors, and one count and one shuffle per side instead of both
 // in one) become one of about 6 us.
+// item_off: NULL, or receives the items before every sub-bucket and behind the
+// last, and k_expand writes the descriptors: one block takes 1.1 us per 1024
+// of them, k_expand 6 to 8 us in all.  1000 x 4e7 rows (9767 items) take 0.41 ms
+// either way, 1000 x 2e8 (48,829) 1.542 ms in one block and 1.511 with k_expand.
 constexpr int kPlanThreads = 1024;
+constexpr uint32_t kPlanItems = 8192;  // items that k_merge_plan describes itself
 static_assert(kMaxFanout <= kPlanThreads, "one sub-bucket per thread");
 __global__ void __launch_bounds__(kPlanThreads)
     k_merge_plan(const uint32_t *__restrict__ tot, uint32_t nL, uint32_t nR, uint32_t nb, uint32_t cap, uint32_t rch,
                  uint32_t ulim, uint32_t *__restrict__ offL, uint32_t *__restrict__ offR, uint32_t *__restrict__ curL,
                  uint32_t *__restrict__ curR, Item *__restrict__ desc, uint64_t *__restrict__ nitems,
-                 unsigned long long *__restrict__ tail) {
+                 uint64_t *__restrict__ item_off, unsigned long long *__restrict__ tail) {
   __shared__ uint32_t scratch[33], s_l[kPlanThreads + 1], s_r[kPlanThreads + 1], s_item[kPlanThreads + 1];
   __shared__ uint64_t scratch64[33];
   const uint32_t b = threadIdx.x;
@@ -113,7 +118,9 @@ __global__ void __launch_bounds__(kPlanThreads)
     s_l[b] = l;
     s_r[b] = r;
     s_item[b] = (uint32_t)at;
+    if (item_off) item_off[b] = at;
     if (b == nb - 1) {
+      if (item_off) item_off[nb] = total;
       offL[nb] = s_l[nb] = l + cl;
       offR[nb] = s_r[nb] = r + cr;
     }
@@ -124,7 +131,7 @@ __global__ void __launch_bounds__(kPlanThreads)
     *nitems = total;
   }
   __syncthreads();
-  if (total > ulim) return;
+  if (total > ulim || item_off) return;
   for (uint32_t it = b; it < (uint32_t)total; it += kPlanThreads) {
     uint32_t lo = 0, hi = nb - 1;  // last bucket with s_item <= it
     while (lo < hi) {
@@ -225,6 +232,17 @@ int resident_grid(KernelT kernel, size_t smem, uint64_t nitems, int *grid, int t
   return MDJ_OK;
 }
 
+// The descriptors of the items counted in item_off.
+int expand_items(Workspace &ws, const uint32_t *offL, const uint32_t *offR, uint32_t nb, uint32_t cap, uint32_t rch,
+                 const uint64_t *item_off, uint32_t ulim, Item *desc, int *flags) {
+  TraceScope tr("join_expand", ws.stream());
+  const uint64_t want = ((uint64_t)ulim + 255) / 256, most = (uint64_t)num_sms() * 8;
+  const unsigned g = (unsigned)std::max<uint64_t>(1, want < most ? want : most);
+  k_expand<<<g, 256, 0, ws.stream()>>>(offL, offR, nb, cap, rch, item_off, ulim, desc, flags);
+  MDJ_LAUNCH_CHECK();
+  return MDJ_OK;
+}
+
 // Work items of the whole join, with `rch` probe rows per item at most, into
 // a descriptor array of `ulim` items.  No host wait: the count stays on the
 // device at (*item_off)[nb] (per-bucket item prefix in *item_off), and a count
@@ -242,13 +260,7 @@ int make_items(Workspace &ws, const Side &Ls, const Side &Rs, uint32_t nb, uint3
   }
   MDJ_LAUNCH_CHECK();
   MDJ_TRY(exclusive_scan_u64(ws, item_off, item_off, nb + 1));
-  {
-    TraceScope tr("join_expand", s);
-    const uint64_t want = ((uint64_t)ulim + 255) / 256, most = (uint64_t)num_sms() * 8;
-    const unsigned g = (unsigned)std::max<uint64_t>(1, want < most ? want : most);
-    k_expand<<<g, 256, 0, s>>>(Ls.off, Rs.off, nb, cap, rch, item_off, ulim, *desc, flags);
-  }
-  MDJ_LAUNCH_CHECK();
+  MDJ_TRY(expand_items(ws, Ls.off, Rs.off, nb, cap, rch, item_off, ulim, *desc, flags));
   *item_off_out = item_off;
   return MDJ_OK;
 }
@@ -581,7 +593,10 @@ int merge_one_pass(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_t
   MDJ_TRY(alloc_join_arrays(ws, item_bound(nb, left->nrows, right->nrows, plan.cap, rch), &ja));
   ja.desc = (Item *)ws.get((size_t)ja.ulim * sizeof(Item));
   ja.nitems = nitems;
-  if (!w || !nitems || !ja.desc) return MDJ_ERR_OOM;
+  const bool many = (uint64_t)nb + chunk_count((uint32_t)left->nrows, plan.cap) +
+                        chunk_count((uint32_t)right->nrows, rch) > kPlanItems;
+  uint64_t *item_off = many ? (uint64_t *)ws.get((size_t)(nb + 1) * 8) : nullptr;
+  if (!w || !nitems || !ja.desc || (many && !item_off)) return MDJ_ERR_OOM;
   uint32_t *offL = w + 2 * (size_t)nb, *offR = offL + nb + 1, *curL = offR + nb + 1, *curR = curL + nb;
   if (plan.partition) {
     MDJ_CUDA_TRY(cudaMemsetAsync(w, 0, 2 * (size_t)nb * 4, s));
@@ -591,9 +606,10 @@ int merge_one_pass(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_t
     TraceScope tr("merge_plan", s);
     k_merge_plan<<<1, kPlanThreads, 0, s>>>(plan.partition ? w : nullptr, (uint32_t)left->nrows,
                                             (uint32_t)right->nrows, nb, plan.cap, rch, ja.ulim, offL, offR, curL, curR,
-                                            ja.desc, nitems, ja.total);
+                                            ja.desc, nitems, item_off, ja.total);
   }
   MDJ_LAUNCH_CHECK();
+  if (many) MDJ_TRY(expand_items(ws, offL, offR, nb, plan.cap, rch, item_off, ja.ulim, ja.desc, (int *)(ja.total + 2)));
   Side L, R;
   MDJ_TRY(shuffle_both(ws, left, lk, right, rk, plan, offL, offR, curL, curR, &L, &R));
   return left->cols[lk].dtype == MDJ_I64 ? run_join_t<int64_t, kWT>(ws, L, R, plan, out, false, nullptr, 0, &ja)

@@ -304,3 +304,21 @@ def test_build_side_of_more_than_512_sub_buckets_per_partition():
     assert counts[0] == counts[1] and counts[0][0] == rows.numel()
     with mdj.MergeStream([lk], [rk], 65) as st:
         assert st.total_rows == rows.numel()
+
+
+@pytest.mark.parametrize("n_l,P,chunks", [(100, 1, 8190), (100, 1, 8191), (6000, 8, 8182), (6000, 8, 8300)])
+def test_item_descriptors_around_one_plan_block(n_l, P, chunks):
+    # work items just within, and beyond, those one block describes (8192);
+    # row i of the right side has key i, the left keys are a sample of them
+    mdj = _mdj()
+    n_r = chunks * 4096 - 5
+    rng = np.random.default_rng(chunks)
+    lk = rng.integers(-n_r // 3, n_r, n_l).astype(np.int32)
+    lk[:2] = [0, n_r - 1]
+    res = mdj.mdj_merge([torch.from_numpy(lk).to(DEV)], [torch.arange(n_r, dtype=torch.int32, device=DEV)], P)
+    got = [t.cpu().numpy() for t in (res.key, res.left_row.view(torch.int32), res.right_row.view(torch.int32))]
+    lrow = np.flatnonzero(lk >= 0).astype(np.int32)
+    want = [lk[lrow], lrow, lk[lrow]]
+    order = [np.lexsort((c[1], c[0])) for c in (got, want)]
+    for g, w in zip(got, want):
+        assert np.array_equal(g[order[0]], w[order[1]])
