@@ -102,6 +102,7 @@ static_assert(kGTab * 4 >= kGCap * 8, "the slot table stages a sub-bucket's 8-by
 constexpr uint32_t kProbeChunk = 65536;    // probe rows per grouping unit
 constexpr int kHT = 256;                   // threads of a global-table block
 constexpr uint32_t kHChunk = 8192;         // rows per global-table unit
+constexpr uint32_t kLightRows = 4 * kGCap; // count: build rows of a sub-bucket that shared-memory tables serve
 constexpr int kET = 256;                   // threads of the emit block
 constexpr uint32_t kETile = 2048;          // output rows per emit tile
 constexpr int kERows = kETile / kET;
@@ -113,7 +114,7 @@ constexpr int kEBlocks = 3;
 
 struct LightUnit {
   uint32_t b, r0, nr;
-  int32_t dump;  // >= 0: the table is saved in (or, for later chunks, loaded from) dump slot `dump`
+  int32_t dump;  // >= 0: the table is saved in (or, for later chunks, loaded from) dump slot `dump`; count: the build chunk
 };
 // A sub-bucket grouped in global memory: build rows [lb, lb + nl), slots
 // [ts0, ts0 + tsz) (tsz = 2 nl) of the slot arrays, rows [hr0, hr0 + nl) of
@@ -1136,12 +1137,21 @@ int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R,
 // side, g(r) on the probe side.  Per sub-bucket a table of the distinct build
 // keys holds each one's rows and sum of f; a probe row adds rows to the count
 // and g(r) * sum to the checksum.  Nothing per row is written.
-//   light (build side <= kGCap rows): the table in shared memory, probed by
-//     units of kProbeChunk probe rows (each unit builds it anew);
+//   light (build side <= kLightRows): tables of kGCap build rows in shared
+//     memory, each probed by units of kProbeChunk probe rows (every unit
+//     builds its table anew); a probe row's terms add up over the tables;
 //   heavy: blocks build the same table from kGCap rows at a time and add its
-//     distinct keys to a global table (linear probing, 5/4 slots per row), so
+//     distinct keys to a global table (linear probing, 7/4 slots per row), so
 //     that a key of millions of rows costs a few thousand global additions;
 //     a second kernel probes that table.
+// kLightRows: a sub-bucket of mostly distinct keys (plans of more than 1024
+// partitions or 1.9e8 build rows have no others) is served best by shared
+// memory, one of a single hot key by the global table.  2.5e8 x 2.5e8 rows of 8
+// + 8 bytes: 113.2 ms with one table, 15.9 with 4 or 8; 2e7 x 2e7 in 2000
+// partitions 9.65 -> 2.57; 2e7 x 2e7 in groups of 20,000 rows 1.04 with 1 or 4,
+// 1.15 with 8.  Slots per row of the global table, 1e8 x 1e8 distinct 4-byte keys
+// in 2000 partitions against those groups: 5/4 57.8 and 1.03 ms, 3/2 33.6 and
+// 1.03, 7/4 27.8 and 1.04, 2 25.6 and 1.05 (more to clear).
 // Before, the count grouped the build side, wrote every probe row's group and
 // read it back: 5e7 x 2e8 Zipf rows, everything after the shuffle 4.2 -> 1.3 ms.
 
@@ -1253,7 +1263,9 @@ __device__ __forceinline__ void add_totals(uint64_t acc, uint64_t csum, unsigned
   }
 }
 
-template <typename KeyT>
+// MULTI: some units belong to sub-buckets of several tables (built with HOT:
+// a hot key may be why).  One kernel for both takes 1% longer where none do.
+template <typename KeyT, bool MULTI>
 __global__ void __launch_bounds__(kGT, 2)
     k_count_light(const __grid_constant__ GSide L, const __grid_constant__ GSide R,
                   const LightUnit *__restrict__ units, uint32_t nunits, uint32_t *ticket, unsigned long long *totals) {
@@ -1269,8 +1281,15 @@ __global__ void __launch_bounds__(kGT, 2)
     const uint32_t u = s_u;
     if (u >= nunits) break;
     const LightUnit U = units[u];
-    const uint32_t lb = L.off[U.b], nl = L.off[U.b + 1] - lb;
-    const uint32_t logt = tab.template build<false>((const KeyT *)L.key + lb, (const uint64_t *)L.cols[0] + lb, nl);
+    uint32_t lb = L.off[U.b], nl = L.off[U.b + 1] - lb;
+    const bool several = MULTI && nl > kGCap;  // this unit's table is number U.dump of several
+    if (several) {
+      lb += U.dump * kGCap;
+      nl = min(kGCap, nl - U.dump * kGCap);
+    }
+    const KeyT *bk = (const KeyT *)L.key + lb;
+    const uint64_t *bf = (const uint64_t *)L.cols[0] + lb;
+    const uint32_t logt = several ? tab.template build<true>(bk, bf, nl) : tab.template build<false>(bk, bf, nl);
     const uint32_t mask = (1u << logt) - 1;
     for (uint32_t i0 = threadIdx.x; i0 < U.nr; i0 += 4 * kGT) {
       KeyT kv[4];
@@ -1303,10 +1322,15 @@ __global__ void __launch_bounds__(kGT, 2)
   add_totals(acc, csum, totals);
 }
 
-// Per sub-bucket, packed for two scans: light units << 32 | heavy build units,
-// and heavy probe units << 40 | global-table slots (entry nb: 0).
+// Per sub-bucket, packed for two scans (entry nb: 0):
+//   a: light units (22 bits) | sub-buckets of several light tables (21) | heavy
+//      build units (21).  At most 2^16 sub-buckets and 2^32 rows a side: at
+//      most 4 (2^16 + 2^16) light units and 2^20 + 2^16 heavy ones.
+//   b: heavy probe units << 40 | global-table slots.
+constexpr uint32_t kLightShift = 42, kMultiShift = 21, kUnitMask = (1u << 21) - 1;
+static_assert(MDJ_MAX_PARTITIONS <= (1u << 16) && kMaxSubBuckets <= (1u << 16), "unit counts fit their bits");
 __host__ __device__ constexpr uint32_t count_slots(uint32_t nl) {
-  return nl / 4 < 0xFFFFFFFFu - nl ? nl + nl / 4 : 0xFFFFFFFFu;
+  return (uint64_t)nl * 7 / 4 < 0xFFFFFFFFu ? (uint32_t)((uint64_t)nl * 7 / 4) : 0xFFFFFFFFu;
 }
 constexpr uint64_t kSlotMask = (1ull << 40) - 1;
 __global__ void k_count_sizes(const uint32_t *__restrict__ offL, const uint32_t *__restrict__ offR, uint32_t nb,
@@ -1316,10 +1340,12 @@ __global__ void k_count_sizes(const uint32_t *__restrict__ offL, const uint32_t 
   uint64_t va = 0, vb = 0;
   if (i < nb) {
     const uint32_t nl = offL[i + 1] - offL[i], nr = offR[i + 1] - offR[i];
-    if (nl && nr && nl <= kGCap) va = (uint64_t)((nr - 1) / kProbeChunk + 1) << 32;
-    if (nr && nl > kGCap) {
-      va = (nl - 1) / kGCap + 1;
-      vb = (uint64_t)((nr - 1) / kHChunk + 1) << 40 | count_slots(nl);
+    if (nl <= kLightRows) {
+      va = (uint64_t)chunk_count(nl, kGCap) * chunk_count(nr, kProbeChunk) << kLightShift |
+           (uint64_t)(nr && nl > kGCap) << kMultiShift;
+    } else if (nr) {
+      va = chunk_count(nl, kGCap);
+      vb = (uint64_t)chunk_count(nr, kHChunk) << 40 | count_slots(nl);
     }
   }
   a[i] = va;
@@ -1335,15 +1361,17 @@ __global__ void k_count_expand(const uint32_t *__restrict__ offL, const uint32_t
   if (i >= nb) return;
   const uint32_t nl = offL[i + 1] - offL[i], r0 = offR[i], nr = offR[i + 1] - r0;
   if (!nl || !nr) return;
-  if (nl <= kGCap) {
-    const uint32_t u0 = (uint32_t)(a[i] >> 32), nu = (nr - 1) / kProbeChunk + 1;
-    for (uint32_t u = lane; u < nu; u += 32)
-      light[u0 + u] = {i, r0 + u * kProbeChunk, min(kProbeChunk, nr - u * kProbeChunk), -1};
+  if (nl <= kLightRows) {
+    const uint32_t u0 = (uint32_t)(a[i] >> kLightShift), nu = chunk_count(nr, kProbeChunk), all = nu * chunk_count(nl, kGCap);
+    for (uint32_t u = lane; u < all; u += 32) {
+      const TileRows t = tile_rows(nr, kProbeChunk, u % nu);
+      light[u0 + u] = {i, r0 + t.row0, t.rows, (int32_t)(u / nu)};
+    }
     return;
   }
-  const uint32_t b0 = (uint32_t)a[i], nbu = (nl - 1) / kGCap + 1;
+  const uint32_t b0 = (uint32_t)a[i] & kUnitMask, nbu = chunk_count(nl, kGCap);
   for (uint32_t u = lane; u < nbu; u += 32) hbuild[b0 + u] = {i, u * kGCap, min(kGCap, nl - u * kGCap)};
-  const uint32_t p0 = (uint32_t)(b[i] >> 40), npu = (nr - 1) / kHChunk + 1;
+  const uint32_t p0 = (uint32_t)(b[i] >> 40), npu = chunk_count(nr, kHChunk);
   for (uint32_t u = lane; u < npu; u += 32) hprobe[p0 + u] = {i, r0 + u * kHChunk, min(kHChunk, nr - u * kHChunk)};
 }
 
@@ -1456,7 +1484,8 @@ int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, ui
   MDJ_CUDA_TRY(cudaMemcpyAsync(&na, pa + nb, 8, cudaMemcpyDeviceToHost, s));
   MDJ_CUDA_TRY(cudaMemcpyAsync(&nbp, pb + nb, 8, cudaMemcpyDeviceToHost, s));
   MDJ_CUDA_TRY(cudaStreamSynchronize(s));
-  const uint32_t nlight = (uint32_t)(na >> 32), nhb = (uint32_t)na, nhp = (uint32_t)(nbp >> 40);
+  const uint32_t nlight = (uint32_t)(na >> kLightShift), nhb = (uint32_t)na & kUnitMask, nhp = (uint32_t)(nbp >> 40);
+  const bool multi = ((na >> kMultiShift) & kUnitMask) != 0;
   const uint64_t hslots = nbp & kSlotMask;
   LightUnit *d_light = (LightUnit *)ws.get((size_t)nlight * sizeof(LightUnit));
   HeavyUnit *d_hbuild = (HeavyUnit *)ws.get((size_t)nhb * sizeof(HeavyUnit));
@@ -1478,17 +1507,17 @@ int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, ui
   const size_t sm = CountTable<KeyT>::bytes();
   static PerDeviceOnce once;
   MDJ_TRY(once_per_device(once, [sm] {
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_light<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_light<KeyT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_light<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_count_heavy_build<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     return (int)MDJ_OK;
   }));
   if (nhb) {
-    uint32_t *hslot = (uint32_t *)ws.get((size_t)hslots * 4), *hrows = (uint32_t *)ws.get((size_t)hslots * 4);
-    unsigned long long *hsum = (unsigned long long *)ws.get((size_t)hslots * 8);
-    if (!hslot || !hrows || !hsum) return MDJ_ERR_OOM;
-    MDJ_CUDA_TRY(cudaMemsetAsync(hslot, 0, (size_t)hslots * 4, s));
-    MDJ_CUDA_TRY(cudaMemsetAsync(hrows, 0, (size_t)hslots * 4, s));
-    MDJ_CUDA_TRY(cudaMemsetAsync(hsum, 0, (size_t)hslots * 8, s));
+    // sums | slot words | rows
+    unsigned long long *hsum = (unsigned long long *)ws.get((size_t)hslots * 16);
+    if (!hsum) return MDJ_ERR_OOM;
+    uint32_t *hslot = (uint32_t *)(hsum + hslots), *hrows = hslot + hslots;
+    MDJ_CUDA_TRY(cudaMemsetAsync(hsum, 0, (size_t)hslots * 16, s));
     {
       TraceScope tr("count_heavy_build", s);
       k_count_heavy_build<KeyT><<<grid_for(nhb, 2), kGT, sm, s>>>(gL, pb, d_hbuild, nhb, hslot, hrows, hsum, err);
@@ -1503,7 +1532,8 @@ int grouped_count_t(Workspace &ws, const Side &L, const Side &R, uint32_t nb, ui
   }
   if (nlight) {
     TraceScope tr("count_light", s);
-    k_count_light<KeyT><<<grid_for(nlight, 2), kGT, sm, s>>>(gL, gR, d_light, nlight, ticket, tot);
+    auto kernel = multi ? k_count_light<KeyT, true> : k_count_light<KeyT, false>;
+    kernel<<<grid_for(nlight, 2), kGT, sm, s>>>(gL, gR, d_light, nlight, ticket, tot);
   }
   MDJ_LAUNCH_CHECK();
   unsigned long long host[4] = {0, 0, 0, 0};

@@ -81,3 +81,23 @@ def test_largest_probe_side_of_an_unpartitioned_plan():
     assert mdj.mdj_count_checksum([torch.from_numpy(lk).to(DEV)], [rk], 1) == (int(hit.sum()), want)
     del rk
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n_l,hot", [(6_000_000, 0), (18_000_000, 0), (200_000, 16_384), (200_000, 16_385), (200_000, 17_000)])
+def test_sub_buckets_around_four_tables(n_l, hot):
+    # 1025 partitions have no sub-buckets: 5.9K and 17.6K build rows each,
+    # mostly distinct keys (two tables, and the global one), or one partition
+    # with a key of about four tables' rows
+    rng = np.random.default_rng(n_l + hot)
+    key_range = 2 * n_l
+    lk = rng.integers(0, key_range, n_l).astype(np.int32)
+    rk = rng.integers(0, key_range, 1_000_003).astype(np.int32)
+    lk[:hot] = 77
+    rk[:hot // 2] = 77
+    lk, rk = rng.permutation(lk), rng.permutation(rk)
+    lp, rp = datagen.uniform_payload(rng, lk.size, np.float32), datagen.uniform_payload(rng, rk.size, np.float32)
+    from paper_2101_08878_gb300 import mdj
+    left, right = [[torch.from_numpy(c).to(DEV) for c in t] for t in ((lk, lp), (rk, rp))]
+    want = oracle.count_checksum_dense(lk, lp, rk, rp, key_range)
+    assert mdj.mdj_count_checksum(left, right, 1025) == want
+    assert mdj.mdj_count_checksum(left, right, 8) == want
