@@ -281,11 +281,14 @@ __global__ void __launch_bounds__(kNW * 32, 2)
 constexpr int kPtGroups = (int)(kShMaxTile / kShNT);  // 32-row groups of a warp's rows at most
 constexpr int kPtWarps = kShNT / 32;
 
+// shift: columns are staged at their offset within a 16-byte line.
 struct PtLayout {
   uint32_t pay, rid, perm, lst, whist, total;
-  __host__ __device__ PtLayout(uint32_t tile, uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F) {
-    pay = tile * key_width;
-    rid = pay + tile * pay_width;
+  __host__ __device__ PtLayout(uint32_t tile, uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F,
+                               bool shift) {
+    const uint32_t slack = shift ? 16 : 0;
+    pay = tile * key_width + slack;
+    rid = pay + tile * pay_width + slack;
     perm = rid + (with_rid ? tile * 4 : 0u);
     lst = perm + tile * 4;
     whist = lst + (2 * F + 32) * 4;
@@ -297,19 +300,18 @@ struct PtLayout {
 // SM.
 uint32_t partition_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t F) {
   uint32_t tile = kShMaxTile;
-  while (PtLayout(tile, key_width, pay_width, with_rid, F).total > kShSmem) tile -= kShNT;
+  while (PtLayout(tile, key_width, pay_width, with_rid, F, true).total > kShSmem) tile -= kShNT;
   return tile;
 }
 
-template <typename KeyT, bool EXTRA>
+template <typename KeyT, bool EXTRA, bool SHIFT>
 __global__ void __launch_bounds__(kShNT, kShBlocks)
     k_partition(const KeyT *__restrict__ keys, uint32_t n, uint32_t tile, uint32_t ntiles, uint32_t pay_width,
                 const __grid_constant__ BucketSpec bs, uint32_t F, const uint32_t *__restrict__ tile_base,
                 const __grid_constant__ ColMove cm, int reg_col, const uint32_t *__restrict__ rid_in,
                 uint32_t *__restrict__ rid_out) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const PtLayout lay(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F);
-  KeyT *skey = (KeyT *)smem;
+  const PtLayout lay(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F, SHIFT);
   unsigned char *spay = smem + lay.pay;
   uint32_t *srid = (uint32_t *)(smem + lay.rid);
   uint32_t *perm = (uint32_t *)(smem + lay.perm);
@@ -326,9 +328,9 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t row0 = t * tile, rows = min(tile, n - row0);
-    load_column<(int)sizeof(KeyT)>((unsigned char *)skey, (const unsigned char *)(keys + row0), rows);
+    const KeyT *skey = (const KeyT *)load_column<(int)sizeof(KeyT), SHIFT>(smem, (const unsigned char *)(keys + row0), rows);
     cp_async_commit();
-    if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
+    const unsigned char *pay = pw ? load_payload<SHIFT>(spay, cm.src[reg_col], pw, row0, rows) : spay;
     if (rid_in) load_column<4>((unsigned char *)srid, (const unsigned char *)(rid_in + row0), rows);
     cp_async_commit();
     for (uint32_t i = lane; i < F; i += 32) wh[i] = 0;
@@ -399,8 +401,8 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
       const uint32_t m = perm[p], i = m & 0xFFFFu;
       const uint32_t d = p + gdelta[m >> 16];
       kdst[d] = skey[i];
-      if (pw == 8) ((uint64_t *)pdst)[d] = ((const uint64_t *)spay)[i];
-      if (pw == 4) ((uint32_t *)pdst)[d] = ((const uint32_t *)spay)[i];
+      if (pw == 8) ((uint64_t *)pdst)[d] = ((const uint64_t *)pay)[i];
+      if (pw == 4) ((uint32_t *)pdst)[d] = ((const uint32_t *)pay)[i];
       if (rid_out) rid_out[d] = rid_in ? srid[i] : row0 + i;
     }
     __syncthreads();
@@ -408,14 +410,14 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 #pragma unroll 1
       for (int j = 0; j < cm.n; j++) {
         if (j == cm.key_index || j == reg_col) continue;
-        load_payload(spay, cm.src[j], cm.width[j], row0, rows);
+        pay = load_payload<SHIFT>(spay, cm.src[j], cm.width[j], row0, rows);
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
         if (cm.width[j] == 8)
-          write_column<uint64_t>((uint64_t *)cm.dst[j], (const uint64_t *)spay, perm, gdelta, rows);
+          write_column<uint64_t>((uint64_t *)cm.dst[j], (const uint64_t *)pay, perm, gdelta, rows);
         else
-          write_column<uint32_t>((uint32_t *)cm.dst[j], (const uint32_t *)spay, perm, gdelta, rows);
+          write_column<uint32_t>((uint32_t *)cm.dst[j], (const uint32_t *)pay, perm, gdelta, rows);
         __syncthreads();
       }
     }
@@ -755,6 +757,12 @@ int hist_grid(size_t smem) {
 }
 
 template <typename KeyT>
+auto partition_kernel(bool extra, bool shift) {
+  if (shift) return extra ? k_partition<KeyT, true, true> : k_partition<KeyT, false, true>;
+  return extra ? k_partition<KeyT, true, false> : k_partition<KeyT, false, false>;
+}
+
+template <typename KeyT>
 int set_smem_attrs() {
   static PerDeviceOnce once;
   return once_per_device(once, [] {
@@ -762,8 +770,10 @@ int set_smem_attrs() {
                                       (int)scatter_smem_bytes(kMaxFanout)));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_scatter<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)scatter_smem_bytes(kPass2SpanMax)));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_partition<KeyT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_partition<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
+    for (int extra = 0; extra < 2; extra++)
+      for (int shift = 0; shift < 2; shift++)
+        MDJ_CUDA_TRY(cudaFuncSetAttribute(partition_kernel<KeyT>(extra != 0, shift != 0),
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_hist<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)((kMaxFanout + kMaxSubBuckets) * 4)));
     return (int)MDJ_OK;
@@ -805,10 +815,16 @@ void launch_partition(const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32
                                                                            rid_in, rid_out);
     return;
   }
-  const uint32_t sm = PtLayout(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F).total;
+  // Columns off 16-byte boundaries take a kernel that stages them at their own
+  // offset.  5e7 rows of 8 + 8 bytes, 8 buckets, one element off: 0.430 ms copied
+  // element by element, 0.323 so (aligned columns 0.308; 0.316 with this kernel).
+  uintptr_t bases = 0;
+  for (int j = 0; j < cm.n; j++) bases |= (uintptr_t)cm.src[j];
+  const bool shift = (bases & 15) != 0;
+  const uint32_t sm = PtLayout(tile, sizeof(KeyT), pay_width, rid_in != nullptr, F, shift).total;
   const uint32_t most = (uint32_t)num_sms() * kShBlocks;
   const int reg_col = cm.n < 2 ? -1 : (cm.key_index == 0 ? 1 : 0);
-  auto kernel = cm.n > 2 ? k_partition<KeyT, true> : k_partition<KeyT, false>;
+  auto kernel = partition_kernel<KeyT>(cm.n > 2, shift);
   kernel<<<std::min(ntiles, most), kShNT, sm, s>>>(keys, n, tile, ntiles, pay_width, bs, F, hist, cm, reg_col, rid_in,
                                                    rid_out);
 }

@@ -128,23 +128,36 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// `rows` elements of W bytes from src to the 16-byte-aligned dst: 16-byte
-// copies where src is 16-byte aligned, else one copy per element.
-template <int W>
-__device__ __forceinline__ void load_column(unsigned char *dst, const unsigned char *src, uint32_t rows) {
+// `rows` elements of W bytes from src to the 16-byte-aligned dst; returns the
+// first element's place.  16-byte copies where src is 16-byte aligned, else
+// one copy per element.  SHIFT: 16-byte copies from any element-aligned src;
+// dst (with 16 bytes of slack) takes them at src's offset within a 16-byte line.
+template <int W, bool SHIFT = false>
+__device__ __forceinline__ unsigned char *load_column(unsigned char *dst, const unsigned char *src, uint32_t rows) {
   uint32_t done = 0;
-  if (((uintptr_t)src & 15) == 0) {
+  if (SHIFT) {
+    const uint32_t sh = (uint32_t)((uintptr_t)src & 15), head = min(rows, ((16 - sh) & 15) / W);
+    dst += sh;
+    const uint32_t n16 = (rows - head) * W / 16;
+    for (uint32_t c = threadIdx.x; c < n16; c += kShNT)
+      cp_async<16>(dst + head * W + c * 16, src + head * W + (size_t)c * 16);
+    if (threadIdx.x < head) cp_async<W>(dst + threadIdx.x * W, src + threadIdx.x * W);
+    done = head + n16 * (16 / W);
+  } else if (((uintptr_t)src & 15) == 0) {
     const uint32_t n16 = rows * W / 16;
     for (uint32_t c = threadIdx.x; c < n16; c += kShNT) cp_async<16>(dst + c * 16, src + (size_t)c * 16);
     done = n16 * (16 / W);
   }
   for (uint32_t i = done + threadIdx.x; i < rows; i += kShNT) cp_async<W>(dst + i * W, src + (size_t)i * W);
+  return dst;
 }
 
-__device__ __forceinline__ void load_payload(unsigned char *dst, const void *col, int width, uint32_t row0,
-                                             uint32_t rows) {
-  if (width == 8) load_column<8>(dst, (const unsigned char *)col + (size_t)row0 * 8, rows);
-  if (width == 4) load_column<4>(dst, (const unsigned char *)col + (size_t)row0 * 4, rows);
+template <bool SHIFT = false>
+__device__ __forceinline__ unsigned char *load_payload(unsigned char *dst, const void *col, int width, uint32_t row0,
+                                                       uint32_t rows) {
+  if (width == 8) return load_column<8, SHIFT>(dst, (const unsigned char *)col + (size_t)row0 * 8, rows);
+  if (width == 4) return load_column<4, SHIFT>(dst, (const unsigned char *)col + (size_t)row0 * 4, rows);
+  return dst;
 }
 
 // Keys of the row pairs this thread ranks: rows 2q, 2q + 1 of the tile, q =

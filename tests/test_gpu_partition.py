@@ -150,3 +150,23 @@ def test_partition_of_the_largest_table(P):
         assert bool(torch.isin(down, starts).all())
     del out
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("shifts", [(1, 0, 0, 0), (0, 1, 1, 1), (1, 0, 2, 3), (0, 1, 3, 2)])
+@pytest.mark.parametrize("n,P", [(1, 3), (5, 1), (6143, 8), (50_001, 64), (50_001, 65), (20_000, 5000)])
+def test_partition_of_columns_off_16_bytes(n, P, shifts):
+    # columns that start at any element of a 16-byte line (slices), 8 and 4 bytes wide
+    mdj = _mdj()
+    for key_col in (0, 3):
+        cols_np = _table(n, np.int64, seed=n + P)
+        cols = []
+        for c, shift in zip(cols_np, shifts):
+            t = torch.empty(n + shift, dtype=torch.from_numpy(c).dtype, device="cuda:0")
+            t[shift:] = torch.from_numpy(c).to("cuda:0")
+            cols.append(t[shift:])
+        off, rid, outs = mdj.mdj_partition(cols, key_col, P)
+        w_off, w_rid, w_cols = oracle.partition_table(cols_np, key_col, P)
+        assert np.array_equal(off.cpu().numpy(), w_off)
+        assert np.array_equal(rid.cpu().numpy().view(np.uint32), w_rid)
+        for g, w in zip(outs, w_cols):
+            assert np.array_equal(g.cpu().numpy().view(np.uint8), w.view(np.uint8))
