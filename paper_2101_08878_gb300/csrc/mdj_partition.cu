@@ -47,7 +47,7 @@ constexpr int kHistU = 8;  // keys per thread in flight
 // `copies` (a power of two) neighbouring copies, one per group of lanes.
 // TWO: also the rows of every sub-bucket (total2), one copy of each counter.
 template <typename KeyT, bool TWO>
-__global__ void __launch_bounds__(kHistThreads, TWO ? 3 : 4) k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
+__global__ void __launch_bounds__(kHistThreads, 4) k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
                                                        uint32_t F, uint32_t copies, uint32_t tile, uint32_t ntiles,
                                                        uint32_t *__restrict__ hist, uint32_t *__restrict__ total2,
                                                        uint32_t nsub) {
@@ -62,15 +62,15 @@ __global__ void __launch_bounds__(kHistThreads, TWO ? 3 : 4) k_hist(const KeyT *
     for (uint32_t b = threadIdx.x; b < F * copies; b += kHistThreads) cnt[b] = 0;
     __syncthreads();
     const TileRows tr = tile_rows(n, tile, t);
-    const KeyT *__restrict__ k = keys + tr.row0 + threadIdx.x;
-    for (uint32_t left = tr.rows; left > 0; left -= min(left, (uint32_t)(kHistThreads * kHistU))) {
+    for (uint32_t i0 = 0; i0 < tr.rows; i0 += kHistThreads * kHistU) {
+      const int left = (int)(tr.rows - i0) - (int)threadIdx.x;  // (a tile has few rows)
+      const KeyT *__restrict__ k = keys + (tr.row0 + i0 + threadIdx.x);
       KeyT kv[kHistU];
 #pragma unroll
-      for (int u = 0; u < kHistU; u++) kv[u] = u * kHistThreads + threadIdx.x < left ? k[u * kHistThreads] : KeyT(0);
-      k += kHistThreads * kHistU;
+      for (int u = 0; u < kHistU; u++) kv[u] = u * kHistThreads < left ? k[u * kHistThreads] : KeyT(0);
 #pragma unroll
       for (int u = 0; u < kHistU; u++) {
-        if (u * kHistThreads + threadIdx.x < left) {
+        if (u * kHistThreads < left) {
           const uint64_t h = fmix64(key_bits(kv[u]));
           if (TWO) {
             const uint32_t p = mod_p(h, bs), x = (uint32_t)(h >> 32);
