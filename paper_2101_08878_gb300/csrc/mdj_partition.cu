@@ -537,11 +537,12 @@ struct ShSides {
 //   4. perm: each row's number goes to its bucket-ordered position;
 //   5. write-out: the columns are gathered through perm and leave as runs.
 // `pay_width`: bytes of a row's place in the payload area.  EXTRA: further
-// columns, one at a time through that area.
-template <typename KeyT, int MODE, bool EXTRA>
-__global__ void __launch_bounds__(kShNT, kShBlocks)
+// columns, one at a time through that area.  NT: threads, kShNT or kShWideNT.
+template <typename KeyT, int MODE, bool EXTRA, int NT>
+__global__ void __launch_bounds__(NT, kShNT * kShBlocks / NT)
     k_shuffle(const __grid_constant__ ShSides sides, uint32_t tile, uint32_t ntiles, uint32_t pay_width,
               const __grid_constant__ BucketSpec bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs sg) {
+  constexpr int kScan = (1024 + NT - 1) / NT;  // local buckets a thread scans at most
   extern __shared__ __align__(16) unsigned char smem[];
   const bool with_rid = MODE == SH_PASS2 && sides.s[0].rid_in != nullptr;
   const ShLayout lay(tile, sizeof(KeyT), pay_width, with_rid, span);
@@ -554,7 +555,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
   uint32_t *gdelta = lst + span;
   uint32_t *wsum = gdelta + span;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (uint32_t i = threadIdx.x; i < span; i += kShNT) cnt[i] = 0;
+  for (uint32_t i = threadIdx.x; i < span; i += NT) cnt[i] = 0;
   __syncthreads();
 
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -570,10 +571,10 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     const uint32_t row0 = MODE == SH_SEG ? td.row0 : (second ? t - sides.s[0].ntiles : t) * tile;
     const uint32_t rows = MODE == SH_SEG ? td.rows : min(tile, sd.n - row0);
     // 1. load
-    load_key_pairs<KeyT>(skey, keys + row0, rows);
+    load_key_pairs<KeyT, NT>(skey, keys + row0, rows);
     cp_async_commit();
-    if (pw) load_payload(spay, cm.src[reg_col], pw, row0, rows);
-    if (with_rid) load_column<4>((unsigned char *)srid, (const unsigned char *)(sd.rid_in + row0), rows);
+    if (pw) load_payload<false, NT>(spay, cm.src[reg_col], pw, row0, rows);
+    if (with_rid) load_column<4, false, NT>((unsigned char *)srid, (const unsigned char *)(sd.rid_in + row0), rows);
     cp_async_commit();
     uint32_t lb0 = 0, Floc = F;
     BucketSpec sp;
@@ -591,7 +592,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
       if (Floc > span) {  // uniform over the block
         cp_async_wait<0>();
         __syncthreads();
-        shuffle_direct<KeyT>(skey, srid, row0, rows, bs, cursors, cm, sd.rid_out);
+        shuffle_direct<KeyT, NT>(skey, srid, row0, rows, bs, cursors, cm, sd.rid_out);
         __syncthreads();
         continue;
       }
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     uint32_t pk[2 * kShPairs];
 #pragma unroll
     for (int k = 0; k < kShPairs; k++) {
-      const uint32_t r = 2 * (threadIdx.x + k * kShNT);
+      const uint32_t r = 2 * (threadIdx.x + k * NT);
       KeyT kv[2] = {KeyT(0), KeyT(0)};
       if (r >= rows) {  // past the tile: nothing there to read
       } else if (sizeof(KeyT) == 8) {
@@ -625,11 +626,11 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     }
     __syncthreads();
     // 3. counts: this thread's buckets [s0, s1); its counters are cleared for the next tile
-    const uint32_t per = (Floc + kShNT - 1) / kShNT;
+    const uint32_t per = (Floc + NT - 1) / NT;
     const uint32_t s0 = min(Floc, threadIdx.x * per), s1 = min(Floc, s0 + per);
-    uint32_t cb[kShScan], gb[kShScan], own = 0;
+    uint32_t cb[kScan], gb[kScan], own = 0;
 #pragma unroll
-    for (int i = 0; i < kShScan; i++) {
+    for (int i = 0; i < kScan; i++) {
       cb[i] = gb[i] = 0;
       if (s0 + i < s1) {
         cb[i] = cnt[s0 + i];
@@ -643,10 +644,10 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     __syncthreads();
     uint32_t ex = inc - own;
 #pragma unroll
-    for (int w = 0; w < kShNT / 32; w++)
+    for (int w = 0; w < NT / 32; w++)
       if (w < warp) ex += wsum[w];
 #pragma unroll
-    for (int i = 0; i < kShScan; i++)
+    for (int i = 0; i < kScan; i++)
       if (s0 + i < s1) {
         lst[s0 + i] = ex;
         gb[i] -= ex;
@@ -660,11 +661,11 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
       for (int e = 0; e < 2; e++) {
         const uint32_t q = pk[2 * k + e];
         if (q != 0xFFFFFFFFu)
-          perm[lst[q >> 16] + (q & 0xFFFFu)] = (q & 0xFFFF0000u) | (2 * (threadIdx.x + k * kShNT) + e);
+          perm[lst[q >> 16] + (q & 0xFFFFu)] = (q & 0xFFFF0000u) | (2 * (threadIdx.x + k * NT) + e);
       }
     }
 #pragma unroll
-    for (int i = 0; i < kShScan; i++)
+    for (int i = 0; i < kScan; i++)
       if (s0 + i < s1) gdelta[s0 + i] = gb[i];
     cp_async_wait<0>();
     __syncthreads();
@@ -673,7 +674,7 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
     void *pdst = pw ? cm.dst[reg_col] : nullptr;
     uint32_t *__restrict__ rid_out = sd.rid_out;
 #pragma unroll 4
-    for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
+    for (uint32_t p = threadIdx.x; p < rows; p += NT) {
       const uint32_t m = perm[p], i = m & 0xFFFFu;
       const uint32_t d = p + gdelta[m >> 16];
       kdst[d] = skey[i];
@@ -694,14 +695,14 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 #pragma unroll 1
       for (int j = 0; j < cm.n; j++) {
         if (j == cm.key_index || j == reg_col) continue;
-        load_payload(spay, cm.src[j], cm.width[j], row0, rows);
+        load_payload<false, NT>(spay, cm.src[j], cm.width[j], row0, rows);
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
         if (cm.width[j] == 8)
-          write_column<uint64_t>((uint64_t *)cm.dst[j], (const uint64_t *)spay, perm, gdelta, rows);
+          write_column<uint64_t, NT>((uint64_t *)cm.dst[j], (const uint64_t *)spay, perm, gdelta, rows);
         else
-          write_column<uint32_t>((uint32_t *)cm.dst[j], (const uint32_t *)spay, perm, gdelta, rows);
+          write_column<uint32_t, NT>((uint32_t *)cm.dst[j], (const uint32_t *)spay, perm, gdelta, rows);
         __syncthreads();
       }
     }
@@ -937,11 +938,13 @@ bool fast_shuffle_enabled() {
 }
 
 template <typename KeyT>
-auto shuffle_kernel(int mode, bool extra) {
-  if (mode == SH_PASS2) return extra ? k_shuffle<KeyT, SH_PASS2, true> : k_shuffle<KeyT, SH_PASS2, false>;
-  if (mode == SH_SEG) return extra ? k_shuffle<KeyT, SH_SEG, true> : k_shuffle<KeyT, SH_SEG, false>;
-  if (mode == SH_TERM) return k_shuffle<KeyT, SH_TERM, false>;
-  return extra ? k_shuffle<KeyT, SH_PASS1, true> : k_shuffle<KeyT, SH_PASS1, false>;
+auto shuffle_kernel(int mode, bool extra, bool wide) {
+  constexpr int N = kShNT, W = kShWideNT;
+  if (mode == SH_PASS2) return extra ? k_shuffle<KeyT, SH_PASS2, true, N> : k_shuffle<KeyT, SH_PASS2, false, N>;
+  if (mode == SH_SEG) return extra ? k_shuffle<KeyT, SH_SEG, true, N> : k_shuffle<KeyT, SH_SEG, false, N>;
+  if (mode == SH_TERM) return k_shuffle<KeyT, SH_TERM, false, N>;
+  if (wide) return extra ? k_shuffle<KeyT, SH_PASS1, true, W> : k_shuffle<KeyT, SH_PASS1, false, W>;
+  return extra ? k_shuffle<KeyT, SH_PASS1, true, N> : k_shuffle<KeyT, SH_PASS1, false, N>;
 }
 
 template <typename KeyT>
@@ -949,10 +952,13 @@ int set_shuffle_attrs() {
   static PerDeviceOnce once;
   return once_per_device(once, [] {
     const int sm = (int)kShSmem;
-    for (int extra = 0; extra < 2; extra++)
+    for (int extra = 0; extra < 2; extra++) {
       for (int mode = 0; mode < 4; mode++)
-        MDJ_CUDA_TRY(cudaFuncSetAttribute(shuffle_kernel<KeyT>(mode, extra != 0),
+        MDJ_CUDA_TRY(cudaFuncSetAttribute(shuffle_kernel<KeyT>(mode, extra != 0, false),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+      MDJ_CUDA_TRY(cudaFuncSetAttribute(shuffle_kernel<KeyT>(SH_PASS1, extra != 0, true),
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShWideSmem));
+    }
     MDJ_CUDA_TRY(cudaFuncSetAttribute(k_tot<KeyT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kMaxSubBuckets * 4)));
     return (int)MDJ_OK;
@@ -986,7 +992,7 @@ ShSide shuffle_side(const mdj_table *t, int32_t key_col, const void *const *src,
 // have rows in pass 1 only).
 template <typename KeyT>
 int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_t pay_width, uint32_t ntiles,
-                 const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs &sg) {
+                 const BucketSpec &bs, uint32_t F, uint32_t F2, uint32_t span, const SegArgs &sg, bool wide = false) {
   bool extra = false;
   for (ShSide &sd : sides.s) {
     sd.ntiles = tile_count(sd.n, tile);
@@ -996,22 +1002,34 @@ int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_
   if (ntiles == 0) return MDJ_OK;
   const bool with_rid = mode == SH_PASS2 && sides.s[0].rid_in;
   const uint32_t sm = ShLayout(tile, sizeof(KeyT), pay_width, with_rid, span).total;
-  const uint32_t most = (uint32_t)num_sms() * kShBlocks;
+  const uint32_t most = (uint32_t)num_sms() * (wide ? 1 : kShBlocks);
   TraceScope tr(mode == SH_SEG ? "seg_scatter" : (mode == SH_PASS2 ? "shuffle_pass2" : "shuffle_pass1"), ws.stream());
-  shuffle_kernel<KeyT>(mode, extra)<<<std::min(ntiles, most), kShNT, sm, ws.stream()>>>(sides, tile, ntiles, pay_width,
-                                                                                        bs, F, F2, span, sg);
+  shuffle_kernel<KeyT>(mode, extra, wide)<<<std::min(ntiles, most), wide ? kShWideNT : kShNT, sm, ws.stream()>>>(
+      sides, tile, ntiles, pay_width, bs, F, F2, span, sg);
   MDJ_LAUNCH_CHECK();
   return MDJ_OK;
 }
 
-// Tile rows of a pass over n rows: the largest tile, or, where that leaves the
+// Tile rows of a pass over n rows (wide: in wide blocks): the largest tile, or, where that leaves the
 // last wave of blocks part empty, the same number of waves of equal tiles
 // (1024 rows at least: a tile has fixed costs of its own).
-uint32_t balanced_tile(uint64_t n, uint32_t largest) {
-  const uint64_t slots = (uint64_t)num_sms() * kShBlocks;
+uint32_t balanced_tile(uint64_t n, uint32_t largest, bool wide = false) {
+  const uint64_t slots = (uint64_t)num_sms() * (wide ? 1 : kShBlocks);
   const uint64_t waves = std::max<uint64_t>(1, (n + slots * largest - 1) / (slots * largest));
   const uint64_t even = ((n + slots * waves - 1) / (slots * waves) + 15) / 16 * 16;
   return (uint32_t)std::min<uint64_t>(largest, std::max<uint64_t>(even, 1024));
+}
+
+// Whether a pass 1 of n rows into F buckets runs in wide blocks: where two
+// blocks per SM leave runs of 11 rows and fewer, and from 300 buckets on where
+// there are many rows with a payload.  1e8 rows of 8 + 8 bytes, two blocks
+// against one wide: 304 buckets 0.802 / 0.709 ms, 489 0.939 / 0.766, 604 1.094 /
+// 0.781, 862 1.317 / 0.849, 1006 1.426 / 0.889 (before the two blocks: 0.793,
+// 0.918, 0.961, 1.138, 1.233).  7e6 rows of 4 + 4 bytes: 304 0.041 / 0.044, 489
+// 0.056 / 0.056, 604 0.072 / 0.060, 862 0.094 / 0.069; 1e6 at 604 0.027 / 0.024;
+// 4e7 lone 8-byte keys: 374 0.217 / 0.232, 604 0.281 / 0.254.
+bool wide_pass(uint32_t F, uint64_t n, uint32_t pay_width) {
+  return F > 512 || (F >= 300 && pay_width > 0 && n >= (1u << 25));
 }
 
 // Rows per sub-bucket of one or both sides (n = 0: none) added to their tot.
@@ -1075,7 +1093,8 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   const BucketSpec spec1 = plan.F2 == 1 ? sub : make_spec(plan.P, plan.S, plan.F2);
   const int32_t pay_col = t->ncols < 2 ? -1 : (key_col == 0 ? 1 : 0);
   const uint32_t pw = !term ? shuffle_pay_width(t, key_col) : pay_col < 0 ? 0u : dtype_width(t->cols[pay_col].dtype);
-  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, false, F1));
+  const bool wide = !term && wide_pass(F1, n, pw);
+  const uint32_t tile = balanced_tile(n, shuffle_tile_rows(sizeof(KeyT), pw, false, F1, wide), wide);
   ShSides sides;
   memset(&sides, 0, sizeof sides);
   if (term) {
@@ -1087,7 +1106,7 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   } else {
     sides.s[0] = shuffle_side(t, key_col, src, out->cols, nullptr, out->rid, cur);
   }
-  MDJ_TRY(shuffle_pass<KeyT>(ws, term ? SH_TERM : SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}));
+  MDJ_TRY(shuffle_pass<KeyT>(ws, term ? SH_TERM : SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}, wide));
   ws.give_back(cur);
   return MDJ_OK;
 }
@@ -1138,11 +1157,13 @@ int shuffle_both_t(Workspace &ws, const mdj_table *left, int32_t lk, const mdj_t
   for (int j = 0; j < left->ncols; j++) src[0][j] = left->cols[j].data;
   for (int j = 0; j < right->ncols; j++) src[1][j] = right->cols[j].data;
   const uint32_t F = plan.nbuckets, pw = std::max(shuffle_pay_width(left, lk), shuffle_pay_width(right, rk));
-  const uint32_t tile = balanced_tile(left->nrows + right->nrows, shuffle_tile_rows(sizeof(KeyT), pw, false, F));
+  const bool wide = wide_pass(F, left->nrows + right->nrows, pw);
+  const uint32_t tile =
+      balanced_tile(left->nrows + right->nrows, shuffle_tile_rows(sizeof(KeyT), pw, false, F, wide), wide);
   ShSides sides;
   sides.s[0] = shuffle_side(left, lk, src[0], fl->cols, nullptr, fl->rid, curL);
   sides.s[1] = shuffle_side(right, rk, src[1], fr->cols, nullptr, fr->rid, curR);
-  return shuffle_pass<KeyT>(ws, SH_PASS1, sides, tile, pw, 0, make_spec(plan.P, plan.S, 1), F, 1, F, SegArgs{});
+  return shuffle_pass<KeyT>(ws, SH_PASS1, sides, tile, pw, 0, make_spec(plan.P, plan.S, 1), F, 1, F, SegArgs{}, wide);
 }
 
 // Stable partition by p with P > kMaxFanout: two stable LSD digit passes

@@ -5,6 +5,8 @@
 
 #include <string.h>
 
+#include <algorithm>
+
 #include "mdj_internal.cuh"
 
 namespace mdj {
@@ -85,7 +87,13 @@ constexpr int kShBlocks = 2;                              // blocks per SM
 constexpr uint32_t kShMaxTile = (uint32_t)kShNT * kShPairs * 2;
 constexpr uint32_t kShSmem = 228u * 1024 / kShBlocks - 1024;  // shared memory of a block
 constexpr int kShScan = (1024 + kShNT - 1) / kShNT;       // local buckets a thread scans at most
-static_assert(kShMaxTile <= 65536, "perm keeps the row in tile in 16 bits");
+// The wide block: one per SM, with all of its shared memory (a tile of 11,000
+// rows of an 8-byte key and payload).  Nothing overlaps its phases, but into
+// many buckets its runs are twice as long.
+constexpr int kShWideNT = 1024;
+constexpr uint32_t kShWideMaxTile = (uint32_t)kShWideNT * kShPairs * 2;
+constexpr uint32_t kShWideSmem = 228u * 1024 - 1024;
+static_assert(kShWideMaxTile <= 65536, "perm keeps the row in tile in 16 bits");
 
 // SH_TERM: pass 1 whose rows leave as (key, checksum term) without row ids.
 enum { SH_PASS1 = 0, SH_PASS2 = 1, SH_SEG = 2, SH_TERM = 3 };
@@ -105,10 +113,11 @@ struct ShLayout {
 };
 
 // Rows of the largest tile that fits a block's shared memory.
-inline uint32_t shuffle_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t span) {
+inline uint32_t shuffle_tile_rows(uint32_t key_width, uint32_t pay_width, bool with_rid, uint32_t span,
+                                  bool wide = false) {
   const uint32_t row = key_width + pay_width + (with_rid ? 4u : 0u) + 4u;
-  const uint32_t rows = (kShSmem - (3 * span + 32) * 4) / row / 16 * 16;
-  return rows < kShMaxTile ? rows : kShMaxTile;
+  const uint32_t rows = ((wide ? kShWideSmem : kShSmem) - (3 * span + 32) * 4) / row / 16 * 16;
+  return std::min(rows, wide ? kShWideMaxTile : kShMaxTile);
 }
 
 template <int W>
@@ -132,44 +141,44 @@ __device__ __forceinline__ void cp_async_wait() {
 // first element's place.  16-byte copies where src is 16-byte aligned, else
 // one copy per element.  SHIFT: 16-byte copies from any element-aligned src;
 // dst (with 16 bytes of slack) takes them at src's offset within a 16-byte line.
-template <int W, bool SHIFT = false>
+template <int W, bool SHIFT = false, int NT = kShNT>
 __device__ __forceinline__ unsigned char *load_column(unsigned char *dst, const unsigned char *src, uint32_t rows) {
   uint32_t done = 0;
   if (SHIFT) {
     const uint32_t sh = (uint32_t)((uintptr_t)src & 15), head = min(rows, ((16 - sh) & 15) / W);
     dst += sh;
     const uint32_t n16 = (rows - head) * W / 16;
-    for (uint32_t c = threadIdx.x; c < n16; c += kShNT)
+    for (uint32_t c = threadIdx.x; c < n16; c += NT)
       cp_async<16>(dst + head * W + c * 16, src + head * W + (size_t)c * 16);
     if (threadIdx.x < head) cp_async<W>(dst + threadIdx.x * W, src + threadIdx.x * W);
     done = head + n16 * (16 / W);
   } else if (((uintptr_t)src & 15) == 0) {
     const uint32_t n16 = rows * W / 16;
-    for (uint32_t c = threadIdx.x; c < n16; c += kShNT) cp_async<16>(dst + c * 16, src + (size_t)c * 16);
+    for (uint32_t c = threadIdx.x; c < n16; c += NT) cp_async<16>(dst + c * 16, src + (size_t)c * 16);
     done = n16 * (16 / W);
   }
-  for (uint32_t i = done + threadIdx.x; i < rows; i += kShNT) cp_async<W>(dst + i * W, src + (size_t)i * W);
+  for (uint32_t i = done + threadIdx.x; i < rows; i += NT) cp_async<W>(dst + i * W, src + (size_t)i * W);
   return dst;
 }
 
-template <bool SHIFT = false>
+template <bool SHIFT = false, int NT = kShNT>
 __device__ __forceinline__ unsigned char *load_payload(unsigned char *dst, const void *col, int width, uint32_t row0,
                                                        uint32_t rows) {
-  if (width == 8) return load_column<8, SHIFT>(dst, (const unsigned char *)col + (size_t)row0 * 8, rows);
-  if (width == 4) return load_column<4, SHIFT>(dst, (const unsigned char *)col + (size_t)row0 * 4, rows);
+  if (width == 8) return load_column<8, SHIFT, NT>(dst, (const unsigned char *)col + (size_t)row0 * 8, rows);
+  if (width == 4) return load_column<4, SHIFT, NT>(dst, (const unsigned char *)col + (size_t)row0 * 4, rows);
   return dst;
 }
 
 // Keys of the row pairs this thread ranks: rows 2q, 2q + 1 of the tile, q =
-// threadIdx.x + k * kShNT, so that a thread reads only keys it copied itself
+// threadIdx.x + k * NT, so that a thread reads only keys it copied itself
 // (visible after its own wait, no barrier).
-template <typename KeyT>
+template <typename KeyT, int NT>
 __device__ __forceinline__ void load_key_pairs(KeyT *skey, const KeyT *keys, uint32_t rows) {
   constexpr int W2 = 2 * (int)sizeof(KeyT);
   const bool al = ((uintptr_t)keys & (W2 - 1)) == 0;
 #pragma unroll
   for (int k = 0; k < kShPairs; k++) {
-    const uint32_t r = 2 * (threadIdx.x + k * kShNT);
+    const uint32_t r = 2 * (threadIdx.x + k * NT);
     if (al && r + 1 < rows) {
       cp_async<W2>(skey + r, keys + r);
     } else {
@@ -182,12 +191,12 @@ __device__ __forceinline__ void load_key_pairs(KeyT *skey, const KeyT *keys, uin
 // A pass-2 tile whose rows span too many buckets for shared memory (tiny or
 // very skewed pass-1 buckets): warp-aggregated reservation, each row written
 // straight to its slot.  key/rid come from the staged tile.
-template <typename KeyT>
+template <typename KeyT, int NT>
 __device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *srid, uint32_t row0, uint32_t rows,
                                             const BucketSpec &bs, uint32_t *__restrict__ cursors, const ColMove &cm,
                                             uint32_t *__restrict__ rid_out) {
   const int lane = threadIdx.x & 31;
-  for (uint32_t i0 = threadIdx.x & ~31u; i0 < rows; i0 += kShNT) {
+  for (uint32_t i0 = threadIdx.x & ~31u; i0 < rows; i0 += NT) {
     const uint32_t i = i0 + lane;
     const bool valid = i < rows;
     const KeyT k = valid ? skey[i] : KeyT(0);
@@ -212,11 +221,11 @@ __device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *sr
 
 // One column of the staged tile to its destinations: consecutive threads
 // store consecutive rows of one run.
-template <typename V>
+template <typename V, int NT = kShNT>
 __device__ __forceinline__ void write_column(V *__restrict__ dst, const V *stage, const uint32_t *perm,
                                              const uint32_t *gdelta, uint32_t rows) {
 #pragma unroll 4
-  for (uint32_t p = threadIdx.x; p < rows; p += kShNT) {
+  for (uint32_t p = threadIdx.x; p < rows; p += NT) {
     const uint32_t m = perm[p];
     dst[p + gdelta[m >> 16]] = stage[m & 0xFFFFu];
   }

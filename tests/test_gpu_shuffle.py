@@ -116,3 +116,44 @@ def test_one_pass_plan_with_many_items_per_bucket():
     lk = np.repeat(rng.permutation(10_000)[:400], 20).astype(np.int64)
     rk = rng.choice(np.concatenate([lk[:40], rng.integers(0, 10_000, 300)]), 60_001)
     _check([lk, datagen.uniform_payload(rng, lk.size)], [rk, datagen.uniform_payload(rng, rk.size)], 16)
+
+
+@pytest.mark.parametrize("P", [512, 513, 1024])
+@pytest.mark.parametrize("nl,nr,shift", [(1, 2, 0), (70_001, 171_111, 1), (900_001, 1_800_003, 0), (10, 3_600_001, 1)])
+@pytest.mark.parametrize("kd,pd", [(np.int64, np.float64), (np.int32, np.float32)])
+def test_pass_in_wide_blocks(P, nl, nr, shift, kd, pd):
+    # more than 512 buckets: one 1024-thread block per SM and tiles of up to 12288 rows
+    left, right = _tables(nl, nr, kd, pd, nl + P)
+    _check(left, right, P, shift)
+
+
+@pytest.mark.parametrize("ncols", [0, 3])
+def test_wide_blocks_column_counts(ncols):
+    rng = np.random.default_rng(ncols)
+    left, right = _tables(300_011, 2_000_013, np.int64, np.float64, 9)
+    kinds = [np.float32, np.float64, np.float32]
+    left = left[:1] + [datagen.uniform_payload(rng, 300_011, k) for k in kinds[:ncols]]
+    right = right[:1] + [datagen.uniform_payload(rng, 2_000_013, k) for k in kinds[:ncols]]
+    _check(left, right, 600, 1)
+
+
+@pytest.mark.parametrize("P,short", [(299, 0), (300, 1), (300, 0), (512, 0)])
+def test_wide_blocks_from_many_rows(P, short):
+    # from 300 buckets on when both sides have 2^25 rows or more; row i of the
+    # right side has key i, the left keys are a sample of them
+    from paper_2101_08878_gb300 import mdj
+    n_l = 5000
+    n_r = 2**25 - n_l - short
+    rng = np.random.default_rng(P)
+    lk = rng.integers(-n_r // 3, n_r, n_l).astype(np.int32)
+    lk[:2] = [0, n_r - 1]
+    rp = torch.arange(n_r, dtype=torch.int32, device=DEV) * 3
+    left = [torch.from_numpy(lk).to(DEV), torch.arange(n_l, dtype=torch.int32, device=DEV) * 7]
+    res = mdj.mdj_merge(left, [torch.arange(n_r, dtype=torch.int32, device=DEV), rp], P)
+    cols = (res.key, res.left_row.view(torch.int32), res.right_row.view(torch.int32), res.left_cols[0], res.right_cols[0])
+    got = [t.cpu().numpy() for t in cols]
+    lrow = np.flatnonzero(lk >= 0).astype(np.int32)
+    want = [lk[lrow], lrow, lk[lrow], lrow * 7, lk[lrow] * 3]
+    order = [np.lexsort((c[1], c[0])) for c in (got, want)]
+    for g, w in zip(got, want):
+        assert np.array_equal(g[order[0]], w[order[1]])
