@@ -322,3 +322,14 @@ def test_item_descriptors_around_one_plan_block(n_l, P, chunks):
     order = [np.lexsort((c[1], c[0])) for c in (got, want)]
     for g, w in zip(got, want):
         assert np.array_equal(g[order[0]], w[order[1]])
+
+
+@pytest.mark.parametrize("n,P,bound", [(4_000_003, 8, 1), (4_000_003, 8, 700), (60_001, 2000, 5)])
+def test_item_count_above_bound_reruns_partitioned_plans(monkeypatch, n, P, bound):
+    # the rerun of the general path without ordered output: two-pass plans,
+    # and more than 1024 partitions (fewer descriptors than items)
+    monkeypatch.setenv("MDJ_TEST_ITEM_BOUND", str(bound))
+    rng = np.random.default_rng(n + bound)
+    left = [rng.permutation(2 * n)[:n].astype(np.int32), datagen.uniform_payload(rng, n, np.float32)]
+    right = [rng.integers(0, 2 * n, 50_001).astype(np.int32), datagen.uniform_payload(rng, 50_001, np.float32)]
+    _check(left, right, P=P)
