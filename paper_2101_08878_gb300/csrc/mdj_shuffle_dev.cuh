@@ -26,7 +26,31 @@ struct ColMove {
 
 // Direct path of a pass-2 tile whose rows span too many buckets for shared
 // memory (tiny or very skewed pass-1 buckets): warp-aggregated reservation,
-// each row written straight to its slot.
+// each row written straight to its slot.  One row per lane: key k and row id
+// rid of input row r (all lanes call it).
+template <typename KeyT>
+__device__ __forceinline__ void place_direct(KeyT k, bool valid, size_t r, uint32_t rid, const BucketSpec &bs,
+                                             uint32_t *__restrict__ cursors, const ColMove &cm,
+                                             uint32_t *__restrict__ rid_out) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t fb = valid ? sub_bucket_of(fmix64(key_bits(k)), bs) : 0xFFFFFFFFu;
+  const uint32_t peers = __match_any_sync(0xffffffffu, fb);
+  const int leader = __ffs(peers) - 1;
+  uint32_t base = 0;
+  if (valid && lane == leader) base = atomicAdd(&cursors[fb], (uint32_t)__popc(peers));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  if (!valid) return;
+  const uint32_t pos = base + __popc(peers & lanemask_lt());
+  for (int j = 0; j < cm.n; j++) {
+    if (cm.width[j] == 8)
+      ((uint64_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint64_t)k : ((const uint64_t *)cm.src[j])[r];
+    else
+      ((uint32_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint32_t)k : ((const uint32_t *)cm.src[j])[r];
+  }
+  if (rid_out) rid_out[pos] = rid;
+}
+
+// The stable passes' tiles: keys in registers, row ids in global memory.
 template <typename KeyT>
 __device__ void scatter_direct(const KeyT (&kv)[kRPL], uint32_t wrow0, uint32_t rend, const BucketSpec &bs,
                                uint32_t *__restrict__ cursors, const ColMove &cm,
@@ -34,26 +58,9 @@ __device__ void scatter_direct(const KeyT (&kv)[kRPL], uint32_t wrow0, uint32_t 
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int c = 0; c < kRPL; c++) {
-    uint32_t r = wrow0 + c * 32 + lane;
-    bool valid = r < rend;
-    uint32_t fb = valid ? sub_bucket_of(fmix64(key_bits(kv[c])), bs) : 0xFFFFFFFFu;
-    uint32_t peers = __match_any_sync(0xffffffffu, fb);
-    int leader = __ffs(peers) - 1;
-    uint32_t base = 0;
-    if (valid && lane == leader) base = atomicAdd(&cursors[fb], (uint32_t)__popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (!valid) continue;
-    uint32_t pos = base + __popc(peers & lanemask_lt());
-    for (int j = 0; j < cm.n; j++) {
-      if (cm.width[j] == 8) {
-        uint64_t v = j == cm.key_index ? (uint64_t)kv[c] : ((const uint64_t *)cm.src[j])[r];
-        ((uint64_t *)cm.dst[j])[pos] = v;
-      } else {
-        uint32_t v = j == cm.key_index ? (uint32_t)kv[c] : ((const uint32_t *)cm.src[j])[r];
-        ((uint32_t *)cm.dst[j])[pos] = v;
-      }
-    }
-    if (rid_out) rid_out[pos] = rid_in ? rid_in[r] : r;
+    const uint32_t r = wrow0 + c * 32 + lane;
+    const bool valid = r < rend;
+    place_direct<KeyT>(kv[c], valid, r, valid && rid_in ? rid_in[r] : r, bs, cursors, cm, rid_out);
   }
 }
 
@@ -188,9 +195,7 @@ __device__ __forceinline__ void load_key_pairs(KeyT *skey, const KeyT *keys, uin
   }
 }
 
-// A pass-2 tile whose rows span too many buckets for shared memory (tiny or
-// very skewed pass-1 buckets): warp-aggregated reservation, each row written
-// straight to its slot.  key/rid come from the staged tile.
+// The shuffle's tiles: key and row id come from the staged tile.
 template <typename KeyT, int NT>
 __device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *srid, uint32_t row0, uint32_t rows,
                                             const BucketSpec &bs, uint32_t *__restrict__ cursors, const ColMove &cm,
@@ -199,23 +204,8 @@ __device__ __noinline__ void shuffle_direct(const KeyT *skey, const uint32_t *sr
   for (uint32_t i0 = threadIdx.x & ~31u; i0 < rows; i0 += NT) {
     const uint32_t i = i0 + lane;
     const bool valid = i < rows;
-    const KeyT k = valid ? skey[i] : KeyT(0);
-    const uint32_t fb = valid ? sub_bucket_of(fmix64(key_bits(k)), bs) : 0xFFFFFFFFu;
-    const uint32_t peers = __match_any_sync(0xffffffffu, fb);
-    const int leader = __ffs(peers) - 1;
-    uint32_t base = 0;
-    if (valid && lane == leader) base = atomicAdd(&cursors[fb], (uint32_t)__popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (!valid) continue;
-    const uint32_t pos = base + __popc(peers & lanemask_lt());
-    const size_t r = (size_t)row0 + i;
-    for (int j = 0; j < cm.n; j++) {
-      if (cm.width[j] == 8)
-        ((uint64_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint64_t)k : ((const uint64_t *)cm.src[j])[r];
-      else
-        ((uint32_t *)cm.dst[j])[pos] = j == cm.key_index ? (uint32_t)k : ((const uint32_t *)cm.src[j])[r];
-    }
-    if (rid_out) rid_out[pos] = srid[i];
+    place_direct<KeyT>(valid ? skey[i] : KeyT(0), valid, (size_t)row0 + i, valid && rid_out ? srid[i] : 0u, bs, cursors,
+                       cm, rid_out);
   }
 }
 

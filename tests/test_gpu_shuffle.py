@@ -157,3 +157,12 @@ def test_wide_blocks_from_many_rows(P, short):
     order = [np.lexsort((c[1], c[0])) for c in (got, want)]
     for g, w in zip(got, want):
         assert np.array_equal(g[order[0]], w[order[1]])
+
+
+@pytest.mark.parametrize("env", ["MDJ_ORDERED_OUTPUT", "MDJ_STABLE_SHUFFLE"])
+@pytest.mark.parametrize("nr", [3, 1000, 60_001])
+def test_two_level_stable_plan_small_probe_side(monkeypatch, env, nr):
+    # the stable passes' direct path: a tile of the small side touches most pass-1 buckets
+    monkeypatch.setenv(env, "1")
+    left, right = _tables(4_000_003, nr, np.int64, np.float32, nr)
+    _check(left, right, 8, 1)
