@@ -21,7 +21,8 @@ namespace mdj {
 // ------------------------------------------------------------------ limits
 
 constexpr uint32_t kMaxFanout = 1024;     // buckets of one stable scatter pass
-// Pass-1 buckets of a two-pass join plan.  Both passes of a 1e8-row side in
+// Pass-1 buckets of a two-pass join plan (more where a partition needs two,
+// see two_pass_split).  Both passes of a 1e8-row side in
 // 28.7K sub-buckets: 1.39 ms with 128, 1.41 with 160, 1.40 with 192; with
 // 14.4K sub-buckets (250M rows): 3.28 ms with 128, 3.42 with 192.
 // The stable passes' smaller tiles do better with 256: ordered output of 1e8 x

@@ -16,9 +16,9 @@
 // counts are already known, so one exact write pass at the recorded item
 // offsets follows.  The grand total is the one value read back to the host.
 //
-// The pair count and checksum of a join (mdj_count_checksum) come from the
-// streamed output's grouping instead (mdj_stream.cu), which handles key groups
-// of any size without re-reading probe rows.
+// The pair count and checksum of a join (mdj_count_checksum) come from tables
+// of rows and terms per distinct build key instead (mdj_stream.cu), which no
+// key group's size makes larger.
 #include <stdlib.h>
 #include <string.h>
 

@@ -16,7 +16,9 @@
 //                by pass-1 bucket are split further; each tile reserves its
 //                runs with one atomicAdd per (tile, bucket)
 //
-// Every kernel is bandwidth-bound: no tensor cores, integer hashing only.
+// Memory kernels: no tensor cores, integer hashing only.  What bounds a scatter
+// is the length of the runs it writes (see k_shuffle's comments): DRAM for few
+// buckets, partial sectors and the shared-memory pipe for many.
 #include <stdlib.h>
 #include <string.h>
 
@@ -490,7 +492,6 @@ __global__ void __launch_bounds__(kTotThreads) k_tot(const TotSide A, const TotS
     if (cnt[i]) atomicAdd(&tot[i], cnt[i]);
 }
 
-// cur[b] = off[b * F2]: the first row of pass-1 bucket b
 // Pass-1 cursors (the first row of every pass-1 bucket) and, for two-level
 // plans, pass 2's: the first row of every sub-bucket (cur2 may be NULL).
 __global__ void k_pass1_cursors(const uint32_t *__restrict__ off, uint32_t F1, uint32_t F2,
@@ -1312,10 +1313,14 @@ Plan make_plan(uint64_t n_build, uint32_t P, uint32_t cap, bool force_partition,
   // target mean build rows per sub-bucket: ~85% of a table, so that hash
   // variance rarely overflows one table
   uint64_t target = (uint64_t)cap * 85 / 100;
-  // small build sides: enough sub-buckets for every resident join block (two
-  // per SM), of at least kMinBucketRows rows; a side that fits one table
-  // still stays whole.  Not for the stable passes, whose cost grows with the
-  // buckets (ordered output of 500K x 500K rows 0.21 ms, 0.23 with more).
+  // small build sides: enough sub-buckets for every resident block of the join,
+  // the count and the grouping (two per SM), of at least kMinBucketRows rows; a
+  // side that fits one table still stays whole.  With whole tables instead:
+  // merge of 1e6 x 2e8 rows 4.00 ms (3.86), count of 2e5 x 1e8 1.60 (1.54),
+  // stream of 2e5 x 5e7 1.66 (1.62), but merge of 2e5 x 2e8 3.56 (3.65: the join
+  // 0.15 less, the shuffle 0.25 more).  Not for the stable passes, whose cost
+  // grows with the buckets (ordered output of 500K x 500K rows 0.21 ms, 0.23
+  // with more).
   if (!stable_passes && n_build > target)
     target = std::min(target, std::max<uint64_t>(kMinBucketRows, n_build / (2 * (uint64_t)num_sms()) + 1));
   uint64_t need = (n_build + target - 1) / target;

@@ -1,6 +1,6 @@
-// Device code of the merge's shuffle passes: the column set of a pass, the
-// direct (unstaged) path of a tile, the register load of a tile and one
-// staged tile (shuffle_tile).
+// Device code of the scatter and shuffle passes: the column set of a pass, the
+// direct (unstaged) path of a tile, a shuffle tile's shared-memory layout, its
+// asynchronous loads and the write-out of one column.
 #pragma once
 
 #include <string.h>
@@ -67,7 +67,8 @@ __device__ void scatter_direct(const KeyT (&kv)[kRPL], uint32_t wrow0, uint32_t 
 // ---------------------------------------------------------------- k_shuffle
 //
 // Two blocks of kShNT threads per SM, each with a tile of as many rows as its
-// half of the shared memory holds (5,700 rows of an 8-byte key and payload):
+// half of the shared memory holds (of an 8-byte key and payload about 5,700 in
+// pass 1, and 4,580 in pass 2 with row ids and 452 local buckets):
 //   key  [tile]   the key column
 //   pay  [tile]   the first non-key column (every further one in turn)
 //   rid  [tile]   pass 2: row ids (none where rows carry a term)

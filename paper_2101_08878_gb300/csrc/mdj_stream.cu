@@ -114,7 +114,9 @@ constexpr int kEBlocks = 3;
 
 struct LightUnit {
   uint32_t b, r0, nr;
-  int32_t dump;  // >= 0: the table is saved in (or, for later chunks, loaded from) dump slot `dump`; count: the build chunk
+  // >= 0: the table is saved in (or, for later chunks, loaded from) dump slot
+  // `dump`; count: which of the sub-bucket's tables
+  int32_t dump;
 };
 // A sub-bucket grouped in global memory: build rows [lb, lb + nl), slots
 // [ts0, ts0 + tsz) (tsz = 2 nl) of the slot arrays, rows [hr0, hr0 + nl) of
@@ -966,12 +968,11 @@ int entries_pass(Workspace &tmp, const EntrySrc &src, const uint64_t *rows0, con
   return MDJ_OK;
 }
 
-// Groups the build side, probes, and builds the entries into the handle.
 // Groups the build side and finds every probe row's group (steps 2-4 of the
 // open): fills `o` (grouped build rows in `keep`, per-probe-row arrays in
 // `tmp`).  keep_left: also the grouped keys, and the group sizes and hit flags
-// that the unmatched-group entries need.  *err_out: a device
-// word set when a global-table probe sequence ran out (read it after a sync).
+// that the unmatched-group entries need.  *err_out: a device word set when a
+// global-table probe sequence ran out (read it after a sync).
 template <typename KeyT>
 int group_sides(Workspace &tmp, Workspace &keep, const Side &L, const Side &R, uint32_t nb, bool keep_left, GOut &o,
                 int **err_out) {
@@ -1070,6 +1071,7 @@ int group_sides(Workspace &tmp, Workspace &keep, const Side &L, const Side &R, u
   return MDJ_OK;
 }
 
+// Groups the build side, probes, and builds the entries into the handle.
 template <typename KeyT>
 int group_and_index(Workspace &tmp, mdj_stream *h, const Side &L, const Side &R, uint32_t nb, int32_t how) {
   const bool keep_left = how == MDJ_LEFT || how == MDJ_OUTER;
