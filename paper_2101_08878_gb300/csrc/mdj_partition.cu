@@ -330,7 +330,8 @@ __global__ void __launch_bounds__(kShNT, kShBlocks)
 
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t row0 = t * tile, rows = min(tile, n - row0);
-    const KeyT *skey = (const KeyT *)load_column<(int)sizeof(KeyT), SHIFT>(smem, (const unsigned char *)(keys + row0), rows);
+    const KeyT *skey =
+        (const KeyT *)load_column<(int)sizeof(KeyT), SHIFT>(smem, (const unsigned char *)(keys + row0), rows);
     cp_async_commit();
     const unsigned char *pay = pw ? load_payload<SHIFT>(spay, cm.src[reg_col], pw, row0, rows) : spay;
     if (rid_in) load_column<4>((unsigned char *)srid, (const unsigned char *)(rid_in + row0), rows);
@@ -1011,9 +1012,9 @@ int shuffle_pass(Workspace &ws, int mode, ShSides &sides, uint32_t tile, uint32_
   return MDJ_OK;
 }
 
-// Tile rows of a pass over n rows (wide: in wide blocks): the largest tile, or, where that leaves the
-// last wave of blocks part empty, the same number of waves of equal tiles
-// (1024 rows at least: a tile has fixed costs of its own).
+// Tile rows of a pass over n rows (wide: in wide blocks): the largest tile, or,
+// where that leaves the last wave of blocks part empty, the same number of
+// waves of equal tiles (1024 rows at least: a tile has fixed costs of its own).
 uint32_t balanced_tile(uint64_t n, uint32_t largest, bool wide = false) {
   const uint64_t slots = (uint64_t)num_sms() * (wide ? 1 : kShBlocks);
   const uint64_t waves = std::max<uint64_t>(1, (n + slots * largest - 1) / (slots * largest));
@@ -1107,7 +1108,8 @@ int shuffle_count_pass1_t(Workspace &ws, const mdj_table *t, int32_t key_col, co
   } else {
     sides.s[0] = shuffle_side(t, key_col, src, out->cols, nullptr, out->rid, cur);
   }
-  MDJ_TRY(shuffle_pass<KeyT>(ws, term ? SH_TERM : SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{}, wide));
+  MDJ_TRY(shuffle_pass<KeyT>(ws, term ? SH_TERM : SH_PASS1, sides, tile, pw, 0, spec1, F1, plan.F2, F1, SegArgs{},
+                             wide));
   ws.give_back(cur);
   return MDJ_OK;
 }

@@ -1364,7 +1364,8 @@ __global__ void k_count_expand(const uint32_t *__restrict__ offL, const uint32_t
   const uint32_t nl = offL[i + 1] - offL[i], r0 = offR[i], nr = offR[i + 1] - r0;
   if (!nl || !nr) return;
   if (nl <= kLightRows) {
-    const uint32_t u0 = (uint32_t)(a[i] >> kLightShift), nu = chunk_count(nr, kProbeChunk), all = nu * chunk_count(nl, kGCap);
+    const uint32_t u0 = (uint32_t)(a[i] >> kLightShift), nu = chunk_count(nr, kProbeChunk);
+    const uint32_t all = nu * chunk_count(nl, kGCap);
     for (uint32_t u = lane; u < all; u += 32) {
       const TileRows t = tile_rows(nr, kProbeChunk, u % nu);
       light[u0 + u] = {i, r0 + t.row0, t.rows, (int32_t)(u / nu)};
