@@ -48,11 +48,14 @@ constexpr int kHistU = 8;  // keys per thread in flight
 // lanes of a warp would add to the same few counters, so each counter has
 // `copies` (a power of two) neighbouring copies, one per group of lanes.
 // TWO: also the rows of every sub-bucket (total2), one copy of each counter.
-template <typename KeyT, bool TWO>
-__global__ void __launch_bounds__(kHistThreads, 4) k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs,
-                                                       uint32_t F, uint32_t copies, uint32_t tile, uint32_t ntiles,
-                                                       uint32_t *__restrict__ hist, uint32_t *__restrict__ total2,
-                                                       uint32_t nsub) {
+// BLOCKS: blocks per SM, as many as the counters leave room for.  Where they
+// leave room for one, the keys in flight have to come from more registers: 1e8
+// + 1e8 8-byte keys in 28.9K sub-buckets 0.642 ms with 32, 0.588 with 80; 5e7 in
+// 14.4K 0.228 with 32, 0.209 with 64; but 3e7 in 8.6K 0.122 with 32, 0.138 with 64.
+template <typename KeyT, bool TWO, int BLOCKS>
+__global__ void __launch_bounds__(kHistThreads, BLOCKS)
+    k_hist(const KeyT *__restrict__ keys, uint32_t n, BucketSpec bs, uint32_t F, uint32_t copies, uint32_t tile,
+           uint32_t ntiles, uint32_t *__restrict__ hist, uint32_t *__restrict__ total2, uint32_t nsub) {
   extern __shared__ uint32_t sh[];
   if (TWO) copies = 1;
   uint32_t *cnt = sh;
@@ -752,11 +755,13 @@ __global__ void k_u32_to_i64(const uint32_t *__restrict__ a, int64_t *__restrict
 
 // ------------------------------------------------------------- host passes
 
-int hist_grid(size_t smem) {
-  int per_sm = 1;
-  if (smem <= 48 * 1024) per_sm = 4;
-  else if (smem <= 100 * 1024) per_sm = 2;
-  return num_sms() * per_sm;
+// Histogram blocks per SM beside `smem` bytes of counters each.
+int hist_blocks(size_t smem) { return smem <= 48 * 1024 ? 4 : smem <= 100 * 1024 ? 2 : 1; }
+
+template <typename KeyT>
+auto hist_kernel(bool two, int blocks) {
+  if (!two) return k_hist<KeyT, false, 4>;
+  return blocks == 4 ? k_hist<KeyT, true, 4> : blocks == 2 ? k_hist<KeyT, true, 2> : k_hist<KeyT, true, 1>;
 }
 
 template <typename KeyT>
@@ -777,8 +782,9 @@ int set_smem_attrs() {
       for (int shift = 0; shift < 2; shift++)
         MDJ_CUDA_TRY(cudaFuncSetAttribute(partition_kernel<KeyT>(extra != 0, shift != 0),
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShSmem));
-    MDJ_CUDA_TRY(cudaFuncSetAttribute(k_hist<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((kMaxFanout + kMaxSubBuckets) * 4)));
+    for (int blocks : {1, 2, 4})
+      MDJ_CUDA_TRY(cudaFuncSetAttribute(hist_kernel<KeyT>(true, blocks), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)((kMaxFanout + kMaxSubBuckets) * 4)));
     return (int)MDJ_OK;
   });
 }
@@ -803,8 +809,9 @@ void launch_hist(const KeyT *keys, uint32_t n, const BucketSpec &bs, uint32_t F,
   const uint32_t copies = total2 ? 1u : hist_copies(F);
   const size_t hsmem = (size_t)(F * copies + (total2 ? nsub : 0)) * 4;
   TraceScope tr("hist", s);
-  const unsigned hgrid = (unsigned)(ntiles < (uint32_t)hist_grid(hsmem) ? ntiles : (uint32_t)hist_grid(hsmem));
-  auto kernel = total2 ? k_hist<KeyT, true> : k_hist<KeyT, false>;
+  const int blocks = hist_blocks(hsmem);
+  const unsigned hgrid = std::min(ntiles, (uint32_t)(num_sms() * blocks));
+  auto kernel = hist_kernel<KeyT>(total2 != nullptr, blocks);
   kernel<<<hgrid, kHistThreads, hsmem, s>>>(keys, n, bs, F, copies, tile, ntiles, hist, total2, nsub);
 }
 
